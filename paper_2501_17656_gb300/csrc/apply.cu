@@ -20,6 +20,7 @@
 // product are in the same format; the multigrid vectors outside are float64.
 #include <algorithm>
 
+#include "fixed.cuh"
 #include "internal.h"
 
 namespace h2mg {
@@ -307,6 +308,316 @@ __global__ void __launch_bounds__(256, bsgemv_min_ctas<FMT, NR>()) k_bsgemv(cons
     for (int ww = 1; ww < 8; ++ww) A::add(s, red[ww][i]);
     A::atomic_add(yrow + (int64_t)row * K * NR + i, A::out(s));
   }
+}
+
+// ----------------------------------------------------------------------------- float64 block GEMV
+// Exponent of every stored float64 block (one warp per block): the biased exponent of its
+// largest magnitude, FX_EMIN for an all-zero block, FX_NONE where fixed point does not
+// serve: exponents outside FX_EMIN..FX_VMAX (Inf and NaN among them), or, with `skip`
+// given, a row or column cluster it marks.
+__global__ void k_block_exponents(const void* const* __restrict__ blk, const int* __restrict__ row,
+                                  const int* __restrict__ col, const unsigned char* __restrict__ skip, int nnz,
+                                  int elems, short* __restrict__ bexp) {
+  const int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (e >= nnz) return;
+  const double2* B = (const double2*)blk[e];
+  int m = 0;
+  bool any = false;
+  for (int i = lane; i < elems / 2; i += 32) {
+    const double2 v = B[i];
+    any = any || v.x != 0.0 || v.y != 0.0;
+    m = max(m, max(fx_exponent(v.x), fx_exponent(v.y)));
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  any = __any_sync(0xffffffffu, any);
+  if (lane == 0) {
+    int E = any ? ((m < FX_EMIN || m > FX_VMAX) ? FX_NONE : m) : FX_EMIN;
+    if (skip && (skip[row[e]] || skip[col[e]])) E = FX_NONE;
+    bexp[e] = (short)E;
+  }
+}
+
+// Leaves whose diagonal entries |A_ii| differ by more than 2^12: their rows have natural
+// scales sqrt(A_ii) of their own (widely varying weights), which one exponent per block
+// would not carry, so their close blocks stay with the float64 path.
+__global__ void k_leaf_spread(const int* __restrict__ leafoff, const double* __restrict__ dg, int nleaf,
+                              unsigned char* __restrict__ skip) {
+  const int l = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (l >= nleaf) return;
+  int lo = 4095, hi = 0;
+  for (int p = leafoff[l] + lane; p < leafoff[l + 1]; p += 32) {
+    const int x = fx_exponent(dg[p]);
+    lo = min(lo, x);
+    hi = max(hi, x);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) skip[l] = hi - lo > 12;
+}
+
+// The product of k_bsgemv for float64 blocks in fixed point (fixed.cuh). Every warp owns
+// `per` consecutive units of work, a unit being CH of the T column passes of one entry, and
+// flushes its row sums when the row changes: no CTA-wide step, and operators with few
+// entries spread over the whole GPU. A block's values are encoded as they arrive (16 integer
+// operations each) and used for both products (6 multiply-adds); the sums of a unit are
+// exact and are scaled into float64 once. The blocks stream through a ring of FX_RING
+// passes (2 KB each) per warp in shared memory, filled by cp.async: a lane reads back what
+// it asked for itself, so the ring needs no synchronisation. What bounds it: see
+// launch_bsgemv_fx.
+constexpr int FX_RING = 4;
+template <int K, int NR>
+constexpr size_t fx_smem() {
+  return 8 * (FX_RING * 2048 + sizeof(double) * 8 * NR * 32 + sizeof(Fx) * K * NR);
+}
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+template <int K, int NR>
+__global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
+    k_bsgemv_fx(const int* __restrict__ erow, const int* __restrict__ col, const void* const* __restrict__ blk,
+                const short* __restrict__ bexp, const double* __restrict__ x, double* __restrict__ yrow,
+                int64_t units, int per) {
+  constexpr int LPC = K / 8, CPP = 32 / LPC, T = K * K / 256, CH = T < LPC ? T : LPC, NCH = T / CH;
+  constexpr int XL = K * NR / 32;                // elements of x_s per lane
+  extern __shared__ __align__(16) unsigned char dsm[];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int rb = 8 * (lane % LPC), cl = lane / LPC;
+  const int64_t u0 = ((int64_t)blockIdx.x * 8 + w) * per;
+  const int64_t u1 = u0 + per < units ? u0 + per : units;
+  if (u0 >= u1) return;
+  double2* ring = (double2*)dsm + w * FX_RING * 128 + lane;          // [FX_RING][4][32], this lane's column
+  double(*yad)[32] = (double(*)[32])(dsm + 8 * FX_RING * 2048) + w * 8 * NR;   // float64 row sums, between entries
+  Fx* xs = (Fx*)(dsm + 8 * (FX_RING * 2048 + sizeof(double) * 8 * NR * 32)) + w * K * NR;   // encoded x of the column
+  Fx xt[8][NR];
+  int Et[NR];
+  bool tfast = false;
+  int row = -1;
+  const double* xrow = x;
+
+  // first pass of a unit, as this lane reads it (nullptr past the end)
+  auto unit_ptr = [&](int64_t u) -> const double2* {
+    return u < u1 ? (const double2*)blk[u / NCH] + (u % NCH) * (CH * 128) + lane : nullptr;
+  };
+  const double2* cur = unit_ptr(u0);
+  const double2* nxt = unit_ptr(u0 + 1);
+  // starts the copy of pass tt of the unit at p; one group per call, an empty one past the end
+  auto issue = [&](const double2* p, int tt) {
+    if (p)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) cp_async16(ring + (tt % FX_RING) * 128 + k * 32, p + tt * 128 + k * 32);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  // reads pass tt of the current unit; the slot read before it is refilled
+  auto take = [&](int tt, double2* d) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(FX_RING - 2) : "memory");
+#pragma unroll
+    for (int k = 0; k < 4; ++k) d[k] = ring[(tt % FX_RING) * 128 + k * 32];
+    constexpr int A = FX_RING - 1;
+    if (tt + A < CH)
+      issue(cur, tt + A);
+    else
+      issue(nxt, tt + A - CH);
+  };
+  auto next_unit = [&](int64_t u) {              // u: the unit that has just been finished
+    cur = nxt;
+    nxt = unit_ptr(u + 2);
+  };
+  static_assert(CH % FX_RING == 0, "a unit starts at slot 0");
+#pragma unroll
+  for (int tt = 0; tt < FX_RING - 1; ++tt) issue(cur, tt);
+
+  // adds the row sums of the lanes that share rows (32 / LPC of them) and stores them
+  auto flush = [&]() {
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int j = 0; j < NR; ++j) {
+        double v = yad[r * NR + j][lane];
+#pragma unroll
+        for (int h = 16; h >= LPC; h >>= 1) v += __shfl_xor_sync(0xffffffffu, v, h);
+        // every lane of a group holds the sum; lane group cl stores rows cl, cl + CPP, ..
+        if (r % CPP == cl) atomicAdd(yrow + ((int64_t)row * K + rb + r) * NR + j, v);
+      }
+  };
+
+  for (int64_t u = u0; u < u1;) {
+    const int e = (int)(u / NCH);
+    const int c0 = (int)(u % NCH), c1 = (int)min((int64_t)NCH, c0 + (u1 - u));
+    int64_t uc = u;                              // the unit in hand
+    u += c1 - c0;
+    const int t = erow[e], s = col[e], Eb = bexp[e];
+    if (t != row) {
+      if (row >= 0) flush();
+      row = t;
+      xrow = x + (int64_t)t * K * NR;
+      double v[8][NR];
+      tfast = true;
+#pragma unroll
+      for (int j = 0; j < NR; ++j) {
+        int m = 0;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          v[r][j] = xrow[(rb + r) * NR + j];
+          m = max(m, fx_exponent(v[r][j]));
+          yad[r * NR + j][lane] = 0.0;
+        }
+        m = __reduce_max_sync(0xffffffffu, m);
+        Et[j] = m == 0 ? FX_EMIN : m;   // a zero column (subnormals count as zero only if all are 0, below)
+        tfast = tfast && Et[j] >= FX_EMIN && Et[j] <= FX_VMAX;
+        if (m == 0) {
+          bool nz = false;
+#pragma unroll
+          for (int r = 0; r < 8; ++r) nz = nz || v[r][j] != 0.0;
+          tfast = tfast && !__any_sync(0xffffffffu, nz);
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int j = 0; j < NR; ++j) xt[r][j] = fx_encode(v[r][j], Et[j]);
+    }
+    const bool off = (s != t);
+    // x of the entry's column: its exponents, then encoded into this warp's shared row
+    const double* xcol = x + (int64_t)s * K * NR;
+    int Es[NR];
+    bool fast = tfast && Eb != FX_NONE;
+    {
+      double v[XL];
+      int m[NR];
+      bool nz = false;
+#pragma unroll
+      for (int j = 0; j < NR; ++j) m[j] = 0;
+#pragma unroll
+      for (int q = 0; q < XL; ++q) {
+        v[q] = xcol[lane * XL + q];          // XL is a multiple of NR: element q is column q % NR
+        m[q % NR] = max(m[q % NR], fx_exponent(v[q]));
+        nz = nz || (fx_exponent(v[q]) == 0 && v[q] != 0.0);
+      }
+      nz = __any_sync(0xffffffffu, nz);
+#pragma unroll
+      for (int j = 0; j < NR; ++j) {
+        m[j] = __reduce_max_sync(0xffffffffu, m[j]);
+        Es[j] = m[j] == 0 ? FX_EMIN : m[j];
+        fast = fast && Es[j] >= FX_EMIN && Es[j] <= FX_VMAX && !(m[j] == 0 && nz);
+      }
+      __syncwarp();                          // the previous entry's reads are done
+      if (fast)
+#pragma unroll
+        for (int q = 0; q < XL; ++q) xs[lane * XL + q] = fx_encode(v[q], Es[q % NR]);
+      __syncwarp();
+    }
+    if (fast) {
+      int64_t yh[8][NR], ym[8][NR];
+      double sr[NR], sc[NR];
+#pragma unroll
+      for (int j = 0; j < NR; ++j) {
+        sr[j] = fx_scale_a(Eb) * fx_scale_b(Es[j]);
+        sc[j] = fx_scale_a(Eb) * fx_scale_b(Et[j]);
+      }
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int j = 0; j < NR; ++j) {
+          yh[r][j] = 0;
+          ym[r][j] = FX_HALF;
+        }
+#pragma unroll 1
+      for (int ch = c0; ch < c1; ++ch) {
+        int64_t z[CH][NR];
+#pragma unroll
+        for (int tt = 0; tt < CH; ++tt) {
+          const int p = ch * CH + tt;
+          double2 d[4];
+          take(tt, d);
+          Fx xv[NR];
+#pragma unroll
+          for (int j = 0; j < NR; ++j) xv[j] = xs[(cl + CPP * p) * NR + j];
+          int64_t zh[NR], zm[NR];
+#pragma unroll
+          for (int j = 0; j < NR; ++j) {
+            zh[j] = 0;
+            zm[j] = FX_HALF;
+          }
+#pragma unroll
+          for (int r = 0; r < 8; ++r) {
+            const Fx b = fx_encode((r & 1) ? d[r / 2].y : d[r / 2].x, Eb);
+#pragma unroll
+            for (int j = 0; j < NR; ++j) {
+              fx_mad(yh[r][j], b.h, xv[j].h);
+              fx_mad(ym[r][j], b.h, xv[j].l);
+              fx_mad(ym[r][j], b.l, xv[j].h);
+              fx_mad(zh[j], b.h, xt[r][j].h);
+              fx_mad(zm[j], b.h, xt[r][j].l);
+              fx_mad(zm[j], b.l, xt[r][j].h);
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < NR; ++j) z[tt][j] = fx_join(zh[j], zm[j]);
+        }
+        if (off) {
+          // sum over the LPC lanes that share a column; lane keeps column lane % CH
+#pragma unroll
+          for (int j = 0; j < NR; ++j) {
+#pragma unroll
+            for (int h = CH / 2; h >= 1; h >>= 1) {
+              const bool up = (lane & h) != 0;
+#pragma unroll
+              for (int q = 0; q < h; ++q) {
+                const int64_t send = up ? z[q][j] : z[q + h][j], keep = up ? z[q + h][j] : z[q][j];
+                z[q][j] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+              }
+            }
+#pragma unroll
+            for (int h = CH; h < LPC; h <<= 1) z[0][j] += __shfl_xor_sync(0xffffffffu, z[0][j], h);
+            if ((lane % LPC) < CH)
+              atomicAdd(yrow + ((int64_t)s * K + cl + CPP * (ch * CH + (lane & (CH - 1)))) * NR + j,
+                        (double)z[0][j] * sc[j]);
+          }
+        }
+        next_unit(uc++);
+      }
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int j = 0; j < NR; ++j) {
+          double& y = yad[r * NR + j][lane];
+          y = fma((double)fx_join(yh[r][j], ym[r][j]), sr[j], y);
+        }
+    } else {
+      // float64 arithmetic: blocks or vectors outside the range of fixed point
+#pragma unroll 1
+      for (int ch = c0; ch < c1; ++ch) {
+#pragma unroll
+        for (int tt = 0; tt < CH; ++tt) {
+          const int p = ch * CH + tt;
+          double2 d[4];
+          take(tt, d);
+          const double m[8] = {d[0].x, d[0].y, d[1].x, d[1].y, d[2].x, d[2].y, d[3].x, d[3].y};
+#pragma unroll
+          for (int j = 0; j < NR; ++j) {
+            const double xv = xcol[(cl + CPP * p) * NR + j];
+            double z = 0.0;
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+              double& y = yad[r * NR + j][lane];
+              y = fma(m[r], xv, y);
+              z = fma(m[r], xrow[(rb + r) * NR + j], z);
+            }
+            if (off) {
+#pragma unroll
+              for (int h = 1; h < LPC; h <<= 1) z += __shfl_xor_sync(0xffffffffu, z, h);
+              if ((lane % LPC) == 0) atomicAdd(yrow + ((int64_t)s * K + cl + CPP * p) * NR + j, z);
+            }
+          }
+        }
+        next_unit(uc++);
+      }
+    }
+  }
+  flush();
 }
 
 // ----------------------------------------------------------------------------- passes
@@ -731,8 +1042,12 @@ static std::vector<int64_t> ubase(const HostCSR& C, int nrows, bool strict) {
   return ub;
 }
 
+// Float64 blocks multiplied in fixed point: 16 x 16 blocks hold too few terms per scaled
+// sum (8 per lane) to pay for their scaling.
+static bool fx_product(int fmt, int K) { return fmt == FMT_F64 && K >= 32; }
+
 static SymOp upload_op(Matrix& M, const OpHost& H, int K, const void* pool0, const void* pool1,
-                       const void* pool0_32, const void* pool1_32) {
+                       const void* pool0_32, const void* pool1_32, const unsigned char* skip = nullptr) {
   SymOp op;
   op.K = K;
   op.nrows = (int)H.rowptr.size() - 1;
@@ -755,9 +1070,21 @@ static SymOp upload_op(Matrix& M, const OpHost& H, int K, const void* pool0, con
   op.blk = (const void**)up(p.data(), sizeof(void*) * p.size());
   op.blk32 = (const void**)up(p32.data(), sizeof(void*) * p32.size());
   int64_t noff = 0;
+  std::vector<int> rowof(op.nnz);
   for (int t = 0; t < op.nrows; ++t)
-    for (int e = H.rowptr[t]; e < H.rowptr[t + 1]; ++e) noff += (H.col[e] != t);
+    for (int e = H.rowptr[t]; e < H.rowptr[t + 1]; ++e) {
+      noff += (H.col[e] != t);
+      rowof[e] = t;
+    }
   op.noff = noff;
+  if (fx_product(M.fmt, K) && op.nnz > 0) {
+    op.erow = (int*)up(rowof.data(), sizeof(int) * rowof.size());
+    op.bexp = (short*)M.alloc(sizeof(short) * op.nnz);
+    { k_block_exponents<<<ceil_div(op.nnz, 8), 256, 0, s>>>(op.blk, op.erow, op.col, skip, op.nnz, K * K, op.bexp);
+      ::h2mg::count_launch(); }
+    H2_LAUNCH_CHECK();
+  }
+  H2_CUDA(cudaStreamSynchronize(s));   // the host lists go out of scope
   return op;
 }
 
@@ -792,8 +1119,11 @@ static OpHost coupling_rows(const Matrix& M, int top, int i) {
   return H;
 }
 
+static void allow_fx_smem();
+
 void setup_operators(Matrix& M) {
   cudaStream_t s = M.stream;
+  if (M.fmt == FMT_F64) allow_fx_smem();
   const int L = M.L;
   // close part of level 1
   {
@@ -810,7 +1140,14 @@ void setup_operators(Matrix& M) {
         }
       H.rowptr.push_back((int)H.col.size());
     }
-    M.opD = upload_op(M, H, M.KD, M.poolD.p, nullptr, M.poolD32.p, nullptr);
+    unsigned char* skip = nullptr;
+    if (fx_product(M.fmt, M.KD)) {
+      skip = (unsigned char*)M.alloc(1 << L);
+      { k_leaf_spread<<<ceil_div(1 << L, 8), 256, 0, s>>>(M.d_leafoff, M.d_dg, 1 << L, skip); ::h2mg::count_launch(); }
+      H2_LAUNCH_CHECK();
+    }
+    M.opD = upload_op(M, H, M.KD, M.poolD.p, nullptr, M.poolD32.p, nullptr, skip);
+    M.free_owned(skip);
   }
   M.opC.assign(M.lev + 1, SymOp{});
   if (M.tstar >= 0) {
@@ -865,6 +1202,46 @@ void setup_operators(Matrix& M) {
   H2_CUDA(cudaStreamSynchronize(s));
 }
 
+// Fixed-point product: work in units of one chunk of an entry, dealt to CTAs of 8 warps;
+// `waves` CTAs per SM in all (0: the default), fewer when there is less than one unit per
+// warp. Float64 FMAs (k_bsgemv) take 2 x 4096 / 2 clocks of an SM per 64 x 64 block, where
+// its 32 KB take 1500 at the copy bandwidth; in fixed point the encoding (22 operations a
+// value) and the multiply-adds (6) keep the integer pipes at 60% and the stream at 64% of the
+// DRAM bandwidth, with 16 resident warps (128 registers) as the limit. Measured, one column
+// on level 2 of 65536 Gaussian points in the cube (3.6 GB of blocks): 1790 -> 880 us; the
+// whole product of 100003 points 4.38 -> 2.06 ms, with two columns per block read
+// (255 registers, 8 warps) 3.74 -> 1.81 ms at 65536 points. Error against the double-double
+// product, before / after (20000 .. 65536 points): Gaussian 3.6e-16 / 3.9e-16, Matern
+// 4.3e-16 / 4.4e-16, square 2.8e-16 / 2.9e-16, sphere 3.8e-16 / 4.1e-16, cubic polynomial
+// 1.63e-15 / 1.60e-15 (both repeat to about 0.3e-16 with the order of the atomic sums).
+constexpr int FX_WAVES = 8, FX_SMS = 152;
+template <int NR>
+static void launch_bsgemv_fx(const SymOp& op, const double* x, double* yrow, int waves, cudaStream_t s) {
+  const int nch = op.K == 64 ? 2 : 1;
+  const int64_t units = (int64_t)op.nnz * nch;
+  if (units == 0) return;
+  const int64_t warps = (int64_t)(waves > 0 ? waves : FX_WAVES) * FX_SMS * 8;
+  const int per = (int)((units + warps - 1) / warps);
+  const int grid = (int)((units + 8 * (int64_t)per - 1) / (8 * (int64_t)per));
+  if (op.K == 64) {
+    k_bsgemv_fx<64, NR><<<grid, 256, fx_smem<64, NR>(), s>>>(op.erow, op.col, op.blk, op.bexp, x, yrow, units, per);
+  } else {
+    k_bsgemv_fx<32, NR><<<grid, 256, fx_smem<32, NR>(), s>>>(op.erow, op.col, op.blk, op.bexp, x, yrow, units, per);
+  }
+  ::h2mg::count_launch();
+}
+
+// Once per matrix (setup_operators): the kernels' dynamic shared memory.
+static void allow_fx_smem() {
+  auto allow = [](const void* f, size_t bytes) {
+    H2_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  };
+  allow((const void*)k_bsgemv_fx<64, 1>, fx_smem<64, 1>());
+  allow((const void*)k_bsgemv_fx<64, 2>, fx_smem<64, 2>());
+  allow((const void*)k_bsgemv_fx<32, 1>, fx_smem<32, 1>());
+  allow((const void*)k_bsgemv_fx<32, 2>, fx_smem<32, 2>());
+}
+
 template <int FMT, int NR>
 static void launch_bsgemv(Matrix& M, const SymOp& op, bool f32, const void* x, void* yrow, cudaStream_t s,
                           int force_split = 0) {
@@ -894,7 +1271,18 @@ static void launch_bsgemv(Matrix& M, const SymOp& op, bool f32, const void* x, v
     }
     H2_CUDA(cudaEventRecord(P.ev[2 * P.used], s));
   }
-  switch (op.K) {
+  // the float64 product has no instances of k_bsgemv for the block edges of the fixed-point one
+  if constexpr (FMT == FMT_F64) {
+    if (op.bexp) {
+      launch_bsgemv_fx<NR>(op, (const double*)x, (double*)yrow, force_split > 0 ? force_split : tuned, s);
+    } else {
+      H2_REQUIRE(op.K == 16 || op.nnz == 0, H2MG_ERR_UNSUPPORTED, "block size not supported");
+      if (op.nnz > 0) {
+        k_bsgemv<16, FMT, NR><<<grid, 256, 0, s>>>(op.rowptr, op.col, blk, (const vt*)x, (yt*)yrow, split);
+        ::h2mg::count_launch();
+      }
+    }
+  } else switch (op.K) {
     case 16:
       { k_bsgemv<16, FMT, NR><<<grid, 256, 0, s>>>(op.rowptr, op.col, blk, (const vt*)x, (yt*)yrow, split); ::h2mg::count_launch(); }
       break;
@@ -1113,14 +1501,15 @@ template <int FMT, int NR>
 static void tune_one(Matrix& M, SymOp& op, bool pts, int opi, cudaStream_t s, cudaEvent_t e0, cudaEvent_t e1,
                      std::vector<double>& rep) {
   if (op.nrows == 0 || op.nnz == 0) return;
-  const int heur = split_heuristic(op.nrows);
+  const bool fx = FMT == FMT_F64 && op.bexp;   // there a candidate is the CTAs per SM of the launch
+  const int heur = fx ? FX_WAVES : split_heuristic(op.nrows);
   const int cands[] = {1, 2, 4, 8, 16, 32, 64};
   const float base = time_product<FMT, NR>(M, op, pts, heur, 3, s, e0, e1);
   float best = base;
   int bs = heur;
   for (int c : cands) {
-    if (c == heur || (int64_t)op.nrows * c > (1 << 22)) continue;
-    if (c > 1 && op.nnz < op.nrows * c) continue;       // more CTAs than blocks: idle CTAs
+    if (c == heur || (!fx && (int64_t)op.nrows * c > (1 << 22))) continue;
+    if (!fx && c > 1 && op.nnz < op.nrows * c) continue;       // more CTAs than blocks: idle CTAs
     const float t = time_product<FMT, NR>(M, op, pts, c, 3, s, e0, e1);
     if (t < best) {
       best = t;
