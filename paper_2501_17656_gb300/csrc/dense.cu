@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "fx_tile.cuh"
 #include "internal.h"
 
 namespace h2mg {
@@ -88,143 +89,204 @@ __global__ void k_pad_diag(double* __restrict__ A, int64_t n, const unsigned cha
   if (i < n && !valid[i]) A[i + i * n] = 1.0;
 }
 
-// ----------------------------------------------------------------------------- Cholesky
-constexpr int NB = 32;
+// ----------------------------------------------------------------------------- factor and inverse
+// A_l = L L^T, X = L^-1 and A_l^-1 = X^T X by 64 x 64 blocks, all three with n^3 / 6 FMAs.
+// Step k of one sweep over the block columns finishes L's column k and X's row k, then
+// updates every block below: A_ij -= L_ik L_jk^T for k < j <= i and, on the rows of the
+// forward substitution L X = I (zero at the start), B_ij -= L_ik X_kj for j <= k. The
+// products run on the integer pipe (fx_tile.cuh); the 64 x 64 diagonal block is factored and
+// inverted in float64 by the CTA that updates it first, beside the rest of its step.
+// X and B are stored transposed, so that every tile is read along consecutive addresses.
+//
+// Bound by the integer multiply-adds: n^3 / 2 FMAs at 3 each, 12 ms for n = 4096 at 27 per
+// clock and SM (the float64 pipe, 2 FMAs per clock and SM, would need 55 ms). Measured for
+// n = 4096: 21.7 ms (updates 14.7, inverse 5.3, panels 1.5), before 180 ms (32-column panels
+// with unblocked substitution, and an inverse from two dense triangular solves).
+constexpr int DB = FXT;                                     // block edge
+constexpr size_t DENSE_SMEM = FX_PAIR_BYTES;
 
-__global__ void k_potrf_diag(double* __restrict__ A, int64_t n, int k0, int nb, int* __restrict__ flag) {
-  __shared__ double S[NB * NB];
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    int i = e % nb, j = e / nb;
-    S[e] = A[(k0 + i) + (int64_t)(k0 + j) * n];
-  }
-  __syncthreads();
-  for (int j = 0; j < nb; ++j) {
-    double d = S[j + j * nb];
-    if (!(d > 0.0)) {
-      if (threadIdx.x == 0) atomicOr(flag, 1);
-      d = 1.0;
+// Cholesky factor of the lower triangle of S (64 x 64, column-major, ld FXLD; rows from nb
+// on are a unit diagonal) and the inverse X of the factor. 256 threads.
+__device__ void factor_diag(double* S, double* X, double* dg, int nb, int* flag) {
+  const int tid = threadIdx.x;
+  for (int j = 0; j < DB; ++j) {
+    if (tid < DB) {
+      double d = S[j + j * FXLD];
+      if (!(d > 0.0)) {
+        if (tid == 0 && j < nb) atomicOr(flag, 1);
+        d = 1.0;
+      }
+      const double l = sqrt(d);
+      if (tid == j) dg[j] = l;
+      if (tid > j) S[tid + j * FXLD] /= l;
     }
-    double ljj = sqrt(d);
     __syncthreads();
-    if (threadIdx.x == 0) S[j + j * nb] = ljj;
-    for (int i = j + 1 + threadIdx.x; i < nb; i += blockDim.x) S[i + j * nb] /= ljj;
-    __syncthreads();
-    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-      int i = e % nb, c = e / nb;
-      if (c > j && i >= c) S[i + c * nb] -= S[i + j * nb] * S[c + j * nb];
-    }
+    const int i = tid & 63;
+    const double lij = S[i + j * FXLD];
+    for (int c = j + 1 + (tid >> 6); c <= i; c += 4) S[i + c * FXLD] = fma(-lij, S[c + j * FXLD], S[i + c * FXLD]);
     __syncthreads();
   }
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    int i = e % nb, j = e / nb;
-    if (i >= j) A[(k0 + i) + (int64_t)(k0 + j) * n] = S[e];
+  // rows of X = L^-1 in turn: four lanes per column
+  const int c = tid >> 2, part = tid & 3;
+  for (int i = 0; i < DB; ++i) {
+    double s = 0.0;
+    for (int m = part; m < i; m += 4) s = fma(S[i + m * FXLD], X[m + c * FXLD], s);
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    if (part == 0) X[i + c * FXLD] = c > i ? 0.0 : ((c == i ? 1.0 : 0.0) - s) / dg[i];
+    __syncthreads();
   }
 }
 
-// Rows below the diagonal block: L21 = A21 L11^{-T} (one thread per row).
-__global__ void k_trsm_panel(double* __restrict__ A, int64_t n, int k0, int nb) {
-  __shared__ double L11[NB * NB];
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    int i = e % nb, j = e / nb;
-    L11[e] = A[(k0 + i) + (int64_t)(k0 + j) * n];
-  }
+// The diagonal block at k0, read from shared memory S: its factor's inverse goes to Li
+// (column-major, 64 x 64).
+__device__ void finish_diag(double* S, double* X, double* dg, int nb, int* flag, double* __restrict__ Li) {
   __syncthreads();
-  int64_t i = (int64_t)k0 + nb + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  for (int j = 0; j < nb; ++j) {
-    double v = A[i + (int64_t)(k0 + j) * n];
-    for (int t = 0; t < j; ++t) v -= A[i + (int64_t)(k0 + t) * n] * L11[j + t * nb];
-    A[i + (int64_t)(k0 + j) * n] = v / L11[j + j * nb];
-  }
+  factor_diag(S, X, dg, nb, flag);
+  for (int e = threadIdx.x; e < DB * DB; e += blockDim.x) Li[e] = X[(e & 63) + (e >> 6) * FXLD];
 }
 
-// Trailing update of the lower triangle: A22 -= L21 L21^T, 64 x 64 tiles.
-__global__ void k_syrk_update(double* __restrict__ A, int64_t n, int k0, int nb, int tiles) {
-  int bi = blockIdx.x % tiles, bj = blockIdx.x / tiles;
-  if (bj > bi) return;
-  __shared__ double Li[64 * NB], Lj[64 * NB];
-  int64_t r0 = (int64_t)k0 + nb + (int64_t)bi * 64, c0 = (int64_t)k0 + nb + (int64_t)bj * 64;
-  for (int e = threadIdx.x; e < 64 * nb; e += blockDim.x) {
-    int i = e % 64, t = e / 64;
-    Li[e] = (r0 + i < n) ? A[(r0 + i) + (int64_t)(k0 + t) * n] : 0.0;
-    Lj[e] = (c0 + i < n) ? A[(c0 + i) + (int64_t)(k0 + t) * n] : 0.0;
+__global__ void __launch_bounds__(256) k_chol_first(const double* __restrict__ A, int64_t n, int* __restrict__ flag,
+                                                    double* __restrict__ Li) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  double* S = (double*)dsm;
+  double* X = S + DB * FXLD;
+  double* dg = X + DB * FXLD;
+  const int nb = (int)min((int64_t)DB, n);
+  for (int e = threadIdx.x; e < DB * DB; e += blockDim.x) {
+    const int i = e & 63, j = e >> 6;
+    S[i + j * FXLD] = i < n && j < n ? A[i + (int64_t)j * n] : (i == j ? 1.0 : 0.0);
   }
+  finish_diag(S, X, dg, nb, flag, Li);
+}
+
+// Step k, first half: block b > k: L_bk = A_bk L_kk^-T; b < k: X_kb = L_kk^-1 B_kb; b = k:
+// X_kk = L_kk^-1. XT holds X (and B) transposed.
+__global__ void __launch_bounds__(256, 2) k_chol_panel(double* __restrict__ A, double* __restrict__ XT, int64_t n,
+                                                       int k, const double* __restrict__ Li) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  const int b = blockIdx.x;
+  const int64_t k0 = (int64_t)k * DB, b0 = (int64_t)b * DB;
+  if (b == k) {
+    for (int e = threadIdx.x; e < DB * DB; e += blockDim.x) {
+      const int j = e & 63, m = e >> 6;
+      if (k0 + j < n && k0 + m < n) XT[k0 + j + (k0 + m) * n] = Li[m + j * DB];
+    }
+    return;
+  }
+  FxPair t(dsm);
+  double* M = b > k ? A : XT;
+  fx_tile_load(t.P, t.ep, [&](int a, int m) { return Li[a + m * DB]; });
+  fx_tile_load(t.Q, t.eq, [&](int i, int m) { return b0 + i < n && k0 + m < n ? M[b0 + i + (k0 + m) * n] : 0.0; });
   __syncthreads();
-  for (int e = threadIdx.x; e < 64 * 64; e += blockDim.x) {
-    int i = e % 64, j = e / 64;
-    int64_t r = r0 + i, c = c0 + j;
-    if (r < n && c < n && r >= c) {
-      double v = 0.0;
-      for (int t = 0; t < nb; ++t) v += Li[i + t * 64] * Lj[j + t * 64];
-      A[r + c * n] -= v;
+  FxAcc c;
+  c.clear();
+  fx_tile_mma(t, c);
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int64_t col = k0 + fx_a() + r, row = b0 + fx_b() + 16 * q;
+      if (row < n && col < n) M[row + col * n] = fx_value(t, c, r, q);
     }
-  }
 }
 
-// ----------------------------------------------------------------------------- inverse
-// A_l^{-1} from the Cholesky factor, by substitution on the identity, all columns at
-// once: L Y = I (forward, block row by block row), then L^T X = Y (backward). Each
-// step solves the NB x NB diagonal block for every column (one thread per column),
-// then updates the remaining rows with a 64 x 64-tiled product.
-__global__ void k_inv_diag(const double* __restrict__ L, int64_t n, int k0, int nb, int fwd,
-                           double* __restrict__ B) {
-  __shared__ double Lk[NB * NB];
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    int i = e % nb, j = e / nb;
-    Lk[e] = L[(k0 + i) + (int64_t)(k0 + j) * n];
+// Step k, second half: the updates of block row i > k, one tile (i, j <= i) per CTA; the
+// first CTA takes tile (k + 1, k + 1) and factors it.
+__global__ void __launch_bounds__(256, 2) k_chol_update(double* __restrict__ A, double* __restrict__ XT, int64_t n,
+                                                        int k, int* __restrict__ flag, double* __restrict__ Li) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  const int first = k + 1;                                   // the first row has tiles 0 .. k + 1
+  int idx = blockIdx.x == 0 ? first : (blockIdx.x == first ? 0 : blockIdx.x);
+  int i = first, j = idx;
+  while (j > i) {
+    j -= i + 1;
+    ++i;
   }
+  const int64_t k0 = (int64_t)k * DB, i0 = (int64_t)i * DB, j0 = (int64_t)j * DB;
+  const bool inv = j <= k;
+  // tile (a, b): A^T's (column c of block j, row r of block i), or B^T's (row r, column c)
+  const double* pm = A + (inv ? i0 : j0);
+  const double* qm = inv ? XT + j0 : A + i0;
+  const int64_t pn = n - (inv ? i0 : j0), qn = n - (inv ? j0 : i0);
+  FxPair t(dsm);
+  fx_tile_load(t.P, t.ep, [&](int a, int m) { return a < pn && k0 + m < n ? pm[a + (k0 + m) * n] : 0.0; });
+  fx_tile_load(t.Q, t.eq, [&](int b, int m) { return b < qn && k0 + m < n ? qm[b + (k0 + m) * n] : 0.0; });
   __syncthreads();
-  int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= n) return;
-  double v[NB];
-  for (int i = 0; i < nb; ++i) v[i] = B[(k0 + i) + c * n];
-  if (fwd) {
-    for (int i = 0; i < nb; ++i) {
-      double t = v[i];
-      for (int j = 0; j < i; ++j) t -= Lk[i + j * nb] * v[j];
-      v[i] = t / Lk[i + i * nb];
+  FxAcc c;
+  c.clear();
+  fx_tile_mma(t, c);
+  double* out = inv ? XT + j0 + i0 * n : A + i0 + j0 * n;
+  double v[4][4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int a = fx_a() + r, b = fx_b() + 16 * q;
+      v[r][q] = a == b ? 1.0 : 0.0;                          // rows past n: a unit diagonal
+      if (a < pn && b < qn) {
+        v[r][q] = out[b + a * n] - fx_value(t, c, r, q);
+        out[b + a * n] = v[r][q];
+      }
     }
-  } else {
-    for (int i = nb - 1; i >= 0; --i) {
-      double t = v[i];
-      for (int j = i + 1; j < nb; ++j) t -= Lk[j + i * nb] * v[j];
-      v[i] = t / Lk[i + i * nb];
-    }
+  if (i == first && j == first) {
+    double* S = (double*)dsm;
+    double* X = S + DB * FXLD;
+    double* dg = X + DB * FXLD;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) S[fx_b() + 16 * q + (fx_a() + r) * FXLD] = v[r][q];
+    finish_diag(S, X, dg, (int)min((int64_t)DB, n - i0), flag, Li);
   }
-  for (int i = 0; i < nb; ++i) B[(k0 + i) + c * n] = v[i];
 }
 
-// fwd: B[i, c] -= sum_t L[i, k0+t] B[k0+t, c] for i >= k0+nb;
-// bwd: B[i, c] -= sum_t L[k0+t, i] B[k0+t, c] for i < k0.
-__global__ void k_inv_update(const double* __restrict__ L, int64_t n, int k0, int nb, int fwd, int row0,
-                             int rows, double* __restrict__ B) {
-  __shared__ double Lp[64 * NB], Bb[NB * 64];
-  int rt = blockIdx.x, ct = blockIdx.y;
-  int64_t r0 = row0 + (int64_t)rt * 64, c0 = (int64_t)ct * 64;
-  for (int e = threadIdx.x; e < 64 * nb; e += blockDim.x) {
-    int i = e % 64, t = e / 64;
-    int64_t r = r0 + i;
-    double v = 0.0;
-    if (r < row0 + rows) v = fwd ? L[r + (int64_t)(k0 + t) * n] : L[(k0 + t) + r * n];
-    Lp[e] = v;
-    int tt = e % nb, cc = e / nb;
-    Bb[e] = (c0 + cc < n) ? B[(k0 + tt) + (c0 + cc) * n] : 0.0;
+// A_l^-1 = X^T X, tile (i, j <= i) per CTA: the sum over block rows m >= i of X_mi^T X_mj.
+__global__ void __launch_bounds__(256, 2) k_chol_inverse(const double* __restrict__ XT, int64_t n, int blocks,
+                                                         double* __restrict__ Ainv) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  int i = 0, j = blockIdx.x;
+  while (j > i) {
+    j -= i + 1;
+    ++i;
   }
+  const int64_t i0 = (int64_t)i * DB, j0 = (int64_t)j * DB;
+  FxPair t(dsm);
+  double s[4][4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s[r][q] = 0.0;
+  for (int m = i; m < blocks; ++m) {
+    const int64_t m0 = (int64_t)m * DB;
+    fx_tile_load(t.P, t.ep, [&](int a, int k) { return j0 + a < n && m0 + k < n ? XT[j0 + a + (m0 + k) * n] : 0.0; });
+    fx_tile_load(t.Q, t.eq, [&](int b, int k) { return i0 + b < n && m0 + k < n ? XT[i0 + b + (m0 + k) * n] : 0.0; });
+    __syncthreads();
+    FxAcc c;
+    c.clear();
+    fx_tile_mma(t, c);
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) s[r][q] += fx_value(t, c, r, q);
+    __syncthreads();
+  }
+  double* S = (double*)dsm;
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int a = fx_a() + r, b = fx_b() + 16 * q;
+      if (j0 + a < n && i0 + b < n) Ainv[i0 + b + (j0 + a) * n] = s[r][q];
+      S[a + b * FXLD] = s[r][q];
+    }
+  if (i == j) return;
   __syncthreads();
-  for (int e = threadIdx.x; e < 64 * 64; e += blockDim.x) {
-    int i = e % 64, j = e / 64;
-    int64_t r = r0 + i, c = c0 + j;
-    if (r < row0 + rows && c < n) {
-      double s = 0.0;
-      for (int t = 0; t < nb; ++t) s += Lp[i + t * 64] * Bb[t + j * nb];
-      B[r + c * n] -= s;
-    }
+  for (int e = threadIdx.x; e < DB * DB; e += blockDim.x) {
+    const int a = e & 63, b = e >> 6;
+    if (j0 + a < n && i0 + b < n) Ainv[j0 + a + (i0 + b) * n] = S[a + b * FXLD];
   }
-}
-
-__global__ void k_identity(double* __restrict__ B, int64_t n) {
-  int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < n * n) B[e] = (e % n == e / n) ? 1.0 : 0.0;
 }
 
 // e[i] = sum_j Ainv[j, i] r[j]: one warp per output, reading column i (contiguous).
@@ -264,37 +326,40 @@ __global__ void k_symv_multi(const double* __restrict__ Ainv, int64_t n, const d
   }
 }
 
-static void build_inverse(Matrix& M) {
+// Factors A_l (d_Al) and, if it is positive definite, overwrites it with its inverse.
+static void factor_and_invert(Matrix& M) {
   cudaStream_t s = M.stream;
-  int64_t n = M.nl;
-  double* B = (double*)M.alloc(sizeof(double) * n * n);
-  { k_identity<<<ceil_div(n * n, 256), 256, 0, s>>>(B, n); ::h2mg::count_launch(); }
+  const int64_t n = M.nl;
+  const int blocks = ceil_div(n, DB);
+  H2_CUDA(cudaFuncSetAttribute(k_chol_first, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DENSE_SMEM));
+  H2_CUDA(cudaFuncSetAttribute(k_chol_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DENSE_SMEM));
+  H2_CUDA(cudaFuncSetAttribute(k_chol_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DENSE_SMEM));
+  H2_CUDA(cudaFuncSetAttribute(k_chol_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DENSE_SMEM));
+  double* XT = (double*)M.alloc(sizeof(double) * n * n);
+  double* Li = (double*)M.alloc(sizeof(double) * DB * DB);
+  H2_CUDA(cudaMemsetAsync(M.d_flag, 0, sizeof(int), s));
+  { k_chol_first<<<1, 256, DENSE_SMEM, s>>>(M.d_Al, n, M.d_flag, Li); ::h2mg::count_launch(); }
   H2_LAUNCH_CHECK();
-  int cgrid = ceil_div(n, 128);
-  for (int k0 = 0; k0 < n; k0 += NB) {
-    int nb = (int)std::min<int64_t>(NB, n - k0);
-    { k_inv_diag<<<cgrid, 128, 0, s>>>(M.d_Al, n, k0, nb, 1, B); ::h2mg::count_launch(); }
+  for (int k = 0; k < blocks; ++k) {
+    { k_chol_panel<<<blocks, 256, DENSE_SMEM, s>>>(M.d_Al, XT, n, k, Li); ::h2mg::count_launch(); }
     H2_LAUNCH_CHECK();
-    int64_t rem = n - k0 - nb;
-    if (rem > 0) {
-      dim3 grid(ceil_div(rem, 64), ceil_div(n, 64));
-      { k_inv_update<<<grid, 256, 0, s>>>(M.d_Al, n, k0, nb, 1, k0 + nb, (int)rem, B); ::h2mg::count_launch(); }
+    const int64_t tiles = (int64_t)blocks * (blocks + 1) / 2 - (int64_t)(k + 1) * (k + 2) / 2;
+    if (tiles > 0) {
+      { k_chol_update<<<(int)tiles, 256, DENSE_SMEM, s>>>(M.d_Al, XT, n, k, M.d_flag, Li); ::h2mg::count_launch(); }
       H2_LAUNCH_CHECK();
     }
   }
-  int last = (int)((n - 1) / NB) * NB;
-  for (int k0 = last; k0 >= 0; k0 -= NB) {
-    int nb = (int)std::min<int64_t>(NB, n - k0);
-    { k_inv_diag<<<cgrid, 128, 0, s>>>(M.d_Al, n, k0, nb, 0, B); ::h2mg::count_launch(); }
-    H2_LAUNCH_CHECK();
-    if (k0 > 0) {
-      dim3 grid(ceil_div(k0, 64), ceil_div(n, 64));
-      { k_inv_update<<<grid, 256, 0, s>>>(M.d_Al, n, k0, nb, 0, 0, k0, B); ::h2mg::count_launch(); }
-      H2_LAUNCH_CHECK();
-    }
-  }
+  int flag = 0;
+  H2_CUDA(cudaMemcpyAsync(&flag, M.d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
   H2_CUDA(cudaStreamSynchronize(s));
-  M.d_Ainv = B;
+  M.coarse_ok = (flag == 0);
+  if (M.coarse_ok) {
+    { k_chol_inverse<<<blocks * (blocks + 1) / 2, 256, DENSE_SMEM, s>>>(XT, n, blocks, M.d_Al); ::h2mg::count_launch(); }
+    H2_LAUNCH_CHECK();
+    M.d_Ainv = M.d_Al;
+  }
+  M.free_owned(XT);
+  M.free_owned(Li);
 }
 
 static void upload_i32(Matrix& M, const std::vector<int>& v, int** d) {
@@ -384,27 +449,7 @@ void build_dense_coarse(Matrix& M) {
   H2_CUDA(cudaMemcpyAsync(dv, valid.data(), valid.size(), cudaMemcpyHostToDevice, s));
   { k_pad_diag<<<ceil_div(M.nl, 256), 256, 0, s>>>(M.d_Al, M.nl, dv); ::h2mg::count_launch(); }
   H2_LAUNCH_CHECK();
-  // Cholesky (lower), pivot check into d_flag
-  H2_CUDA(cudaMemsetAsync(M.d_flag, 0, sizeof(int), s));
-  int64_t n = M.nl;
-  for (int k0 = 0; k0 < n; k0 += NB) {
-    int nb = (int)std::min<int64_t>(NB, n - k0);
-    { k_potrf_diag<<<1, 256, 0, s>>>(M.d_Al, n, k0, nb, M.d_flag); ::h2mg::count_launch(); }
-    H2_LAUNCH_CHECK();
-    int64_t rem = n - k0 - nb;
-    if (rem > 0) {
-      { k_trsm_panel<<<ceil_div(rem, 128), 128, 0, s>>>(M.d_Al, n, k0, nb); ::h2mg::count_launch(); }
-      H2_LAUNCH_CHECK();
-      int tiles = ceil_div(rem, 64);
-      { k_syrk_update<<<tiles * tiles, 256, 0, s>>>(M.d_Al, n, k0, nb, tiles); ::h2mg::count_launch(); }
-      H2_LAUNCH_CHECK();
-    }
-  }
-  int flag = 0;
-  H2_CUDA(cudaMemcpyAsync(&flag, M.d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
-  H2_CUDA(cudaStreamSynchronize(s));
-  M.coarse_ok = (flag == 0);
-  if (M.coarse_ok) build_inverse(M);
+  factor_and_invert(M);
   M.wcoarse.bytes = sizeof(double) * 3 * (size_t)M.nl;
   M.wcoarse.p = M.alloc(M.wcoarse.bytes);
 }

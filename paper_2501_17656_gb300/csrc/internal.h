@@ -139,8 +139,8 @@ struct Matrix {
 
   // ---- dense coarsest operator and Cholesky factor
   int nl = 0;                   // size of A_l
-  double* d_Al = nullptr;       // [nl * nl] column-major; lower triangle holds the factor
-  double* d_Ainv = nullptr;     // [nl * nl] A_l^{-1} formed from the factor
+  double* d_Al = nullptr;       // [nl * nl] column-major: A_l until it is factored
+  double* d_Ainv = nullptr;     // [nl * nl] A_l^{-1} formed from the factor (A_l's memory)
   bool coarse_ok = false;
 
   // ---- workspaces
