@@ -16,6 +16,7 @@
 #include <cmath>
 #include <unordered_map>
 
+#include "fx_tile.cuh"
 #include "internal.h"
 
 namespace h2mg {
@@ -529,6 +530,117 @@ __global__ void k_fill_Pi(const int* __restrict__ pt, const int* __restrict__ ps
   store_block(pool, fmt, b, KC, acc);
 }
 
+// ----------------------------------------------------------------------------- 64 x 64 blocks
+// P_i (i >= 3) of 64 x 64 blocks takes six products of 64 x 64 matrices per block (eight in
+// k_fill_Pi): on the float64 pipe 131 k clocks of an SM each, which bounded it; here they run
+// on the integer pipe (fx_tile.cuh), 29 k clocks each. One CTA per block, two CTAs per SM so
+// that one's loads and encodings run beside the other's products. Measured on 20000 Gaussian
+// points in the cube (Chebyshev, P_3 .. P_5): 77.8 -> 12.5 ms. The couplings S = R_t k R_s^T
+// (k_fill_S) and P_2 = U^T D U (k_fill_P2) stay in float64: the factors R are graded, and one
+// exponent per row of the intermediate product would carry small rows with fewer digits;
+// P_2 was built and measured too (21.7 -> 4.4 ms), but solves whose last cycles sit at the
+// float64 floor then took other cycle counts than the oracle's (10 instead of 12 to 14).
+constexpr size_t FILL64_SMEM = FX_PAIR_BYTES + sizeof(double) * FXT * FXLD;
+
+// Writes this thread's elements of a 64 x 64 block into the pool, swizzled.
+__device__ __forceinline__ void store_block64(void* pool, int fmt, int64_t blk, const double (&v)[4][4]) {
+  const int V = fmt == FMT_F32 ? 4 : 2;
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      store_elem(pool, fmt, blk * FXT * FXT + swz(fx_a() + r, fx_b() + 16 * q, FXT, V), v[r][q]);
+}
+
+__device__ __forceinline__ void fx_values(const FxPair& t, const FxAcc& c, double (&v)[4][4]) {
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[r][q] = fx_value(t, c, r, q);
+}
+
+// Encodes a stored block (transposed where its reference says so) as operand P (row, k),
+// with exponents that cover the block of `O` too and one bit of headroom. Threads read the
+// pool in storage order.
+__device__ void fx_tile_load_block(Fx* T, int* ex, const ChildRef& R, const ChildRef& O,
+                                   const void* __restrict__ poolPf, const void* __restrict__ poolS, int fmt) {
+  const int V = fmt == FMT_F32 ? 4 : 2;
+  if (threadIdx.x < FXT) ex[threadIdx.x] = FX_EMIN;
+  __syncthreads();
+  double v[16];
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const int e = threadIdx.x + 256 * q;
+    int i, j;
+    unswz(e, FXT, V, i, j);
+    v[q] = load_elem(R.pool ? poolS : poolPf, fmt, R.blk * FXT * FXT + e);
+    atomicMax(ex + (R.trans ? j : i), fx_exponent(v[q]) + 1);
+    const double o = load_elem(O.pool ? poolS : poolPf, fmt, O.blk * FXT * FXT + e);
+    atomicMax(ex + (O.trans ? j : i), fx_exponent(o) + 1);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    int i, j;
+    unswz(threadIdx.x + 256 * q, FXT, V, i, j);
+    if (R.trans) {
+      const int x = i;
+      i = j;
+      j = x;
+    }
+    T[j * FXLD + i] = fx_encode(v[q], ex[i]);
+  }
+}
+
+// k_fill_Pi for 64 x 64 blocks: for each child a of c, T = sum over the children a' of c' of
+// M(a, a') E'_a' (one sum of 128 terms: the exponents cover both children), then E'_a^T T.
+__global__ void __launch_bounds__(256, 2)
+    k_fill_Pi64(const int* __restrict__ pt, const int* __restrict__ ps, const ChildRef* __restrict__ ref,
+                const void* __restrict__ poolPf, const void* __restrict__ poolS, int fmt,
+                const double* __restrict__ E, void* __restrict__ pool) {
+  extern __shared__ __align__(16) double sm[];
+  FxPair t(sm);
+  double* S = sm + FX_PAIR_BYTES / sizeof(double);     // the first child's product
+  const int64_t b = blockIdx.x;
+  const int cr = pt[b], cc = ps[b];
+  double v[4][4];
+  FxAcc c;
+  for (int a = 0; a < 2; ++a) {
+    c.clear();
+    for (int x = 0; x < 2; ++x) {
+      const ChildRef R = ref[b * 4 + 2 * a + x], O = ref[b * 4 + 2 * a + 1 - x];
+      const double* Ex = E + (int64_t)(2 * cc + x) * FXT * FXT;
+      const double* Eo = E + (int64_t)(2 * cc + 1 - x) * FXT * FXT;
+      __syncthreads();
+      fx_tile_load_k(t.Q, t.eq, [&](int j, int l) { return Ex[l + j * FXT]; }, 1,
+                     [&](int j, int l) { return Eo[l + j * FXT]; });
+      fx_tile_load_block(t.P, t.ep, R, O, poolPf, poolS, fmt);
+      __syncthreads();
+      fx_tile_mma(t, c);
+    }
+    fx_values(t, c, v);
+    __syncthreads();
+    fx_tile_store_q(t.Q, t.eq, v);
+    const double* Ea = E + (int64_t)(2 * cr + a) * FXT * FXT;
+    fx_tile_load_k(t.P, t.ep, [&](int r, int l) { return Ea[l + r * FXT]; });
+    __syncthreads();
+    c.clear();
+    fx_tile_mma(t, c);
+    fx_values(t, c, v);
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        double& s = S[fx_b() + 16 * q + (fx_a() + r) * FXLD];
+        if (a == 0)
+          s = v[r][q];
+        else
+          v[r][q] += s;
+      }
+  }
+  store_block64(pool, fmt, b, v);
+}
+
 // Re-store a pool in another format (the swizzle depends on the element width).
 __global__ void k_convert_pool(const void* __restrict__ src, int fsrc, void* __restrict__ dst,
                                int fdst, int K) {
@@ -679,6 +791,7 @@ void build_coarse_near(Matrix& M) {
   // ---- P_i, i >= 3, level by level
   size_t sm = sizeof(double) * 3 * KC * KC;
   H2_CUDA(cudaFuncSetAttribute(k_fill_Pi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  H2_CUDA(cudaFuncSetAttribute(k_fill_Pi64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FILL64_SMEM));
   for (int i = 3; i <= M.lev; ++i) {
     int mc = L - i + 2, mf = mc + 1;
     const HostCSR& Ic = M.inadm[mc];
@@ -721,7 +834,11 @@ void build_coarse_near(Matrix& M) {
     M.poolP[i].p = M.alloc(M.poolP[i].bytes);
     const double* Ef = M.d_E + (size_t)M.slot0(mf) * KC * KC;
     chunked(M.nP[i], [&](int64_t b0, int nb) {
-      { k_fill_Pi<<<nb, 256, sm, s>>>(d_t + b0, d_s + b0, d_ref + b0 * 4, M.poolP[i - 1].p, M.poolS.p,
+      if (KC == FXT) {
+        k_fill_Pi64<<<nb, 256, FILL64_SMEM, s>>>(d_t + b0, d_s + b0, d_ref + b0 * 4, M.poolP[i - 1].p, M.poolS.p,
+                                                 M.fmt, Ef, (char*)M.poolP[i].p + pool_bytes(b0, KC, M.fmt));
+        ::h2mg::count_launch();
+      } else { k_fill_Pi<<<nb, 256, sm, s>>>(d_t + b0, d_s + b0, d_ref + b0 * 4, M.poolP[i - 1].p, M.poolS.p,
                                     M.fmt, Ef, KC, (char*)M.poolP[i].p + pool_bytes(b0, KC, M.fmt)); ::h2mg::count_launch(); }
       H2_LAUNCH_CHECK();
     });
