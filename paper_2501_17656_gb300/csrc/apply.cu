@@ -161,6 +161,23 @@ __device__ __forceinline__ void load_row(const T* p, T* out) {
   }
 }
 
+// yrow[0..NR-1] += v: one vector reduction for two or four FP32 columns (interleaved, so
+// aligned to their size), else one atomic per column. Four columns on the second level of a
+// sphere of 18000 panels: 89 -> 80 us.
+template <int FMT, int NR>
+__device__ __forceinline__ void add_columns(typename Ar<FMT>::yo_t* p, const typename Ar<FMT>::acc_t (&v)[NR]) {
+  using A = Ar<FMT>;
+  if constexpr (FMT == FMT_F32 && NR == 4) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3])
+                 : "memory");
+  } else if constexpr (FMT == FMT_F32 && NR == 2) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(v[0]), "f"(v[1]) : "memory");
+  } else {
+#pragma unroll
+    for (int j = 0; j < NR; ++j) A::atomic_add(p + j, A::out(v[j]));
+  }
+}
+
 // ----------------------------------------------------------------------------- block GEMV
 // One CTA (8 warps) per block row t of a symmetric upper-stored block operator:
 // yrow[t] += sum_e B_e x_col(e) and, for every off-diagonal entry e = (t, s),
@@ -259,6 +276,7 @@ __global__ void __launch_bounds__(256, bsgemv_min_ctas<FMT, NR>()) k_bsgemv(cons
       }
       if (off) {
         // reduce the CH partial columns over the LPC lanes that share them
+        acc_t zs[NR];
 #pragma unroll
         for (int j = 0; j < NR; ++j) {
           if (CH == LPC) {
@@ -273,15 +291,14 @@ __global__ void __launch_bounds__(256, bsgemv_min_ctas<FMT, NR>()) k_bsgemv(cons
                 zc[q][j] = keep;
               }
             }
-            const int tt = lane & (CH - 1);
-            A::atomic_add(yrow + ((int64_t)s * K + cl + CPP * (ch * CH + tt)) * NR + j, A::out(zc[0][j]));
           } else {
 #pragma unroll
             for (int h = LPC / 2; h >= 1; h >>= 1) A::add(zc[0][j], A::shfl(zc[0][j], h));
-            if ((lane % LPC) == 0)
-              A::atomic_add(yrow + ((int64_t)s * K + cl + CPP * (ch * CH)) * NR + j, A::out(zc[0][j]));
           }
+          zs[j] = zc[0][j];
         }
+        if (CH == LPC || (lane % LPC) == 0)
+          add_columns<FMT, NR>(yrow + ((int64_t)s * K + cl + CPP * (ch * CH + (lane & (CH - 1)))) * NR, zs);
       }
     }
 #pragma unroll
@@ -308,6 +325,94 @@ __global__ void __launch_bounds__(256, bsgemv_min_ctas<FMT, NR>()) k_bsgemv(cons
     for (int ww = 1; ww < 8; ++ww) A::add(s, red[ww][i]);
     A::atomic_add(yrow + (int64_t)row * K * NR + i, A::out(s));
   }
+}
+
+// ----------------------------------------------------------------------------- small blocks
+// The product of k_bsgemv for blocks of 16 and 32: every warp owns `per` consecutive entries
+// and adds its row sums when the row changes. A block is one pass (16) or four (32) of a
+// warp, so a CTA per row with eight warps and a CTA-wide sum leaves most warps without an
+// entry. Bound by latency at the sizes where it matters: the 112 block rows of 16 of the
+// second level of 4096 points (F64, 1.3 MB of blocks) took 35 us and now take 6.
+template <int K, int FMT, int NR>
+__global__ void __launch_bounds__(256) k_bsgemv_small(const int* __restrict__ erow, const int* __restrict__ col,
+                                                      const void* const* __restrict__ blk,
+                                                      const typename Ar<FMT>::vec_t* __restrict__ x,
+                                                      typename Ar<FMT>::yo_t* __restrict__ yrow, int nnz, int per) {
+  using A = Ar<FMT>;
+  using vec_t = typename A::vec_t;
+  using mel_t = typename A::mel_t;
+  using acc_t = typename A::acc_t;
+  using ld_t = typename A::ld_t;
+  constexpr int LPC = K / 8, CPP = 32 / LPC, T = K * K / 256;
+  constexpr int V = A::V, P = 8 / V;
+  const int lane = threadIdx.x & 31;
+  const int rb = 8 * (lane % LPC), cl = lane / LPC;
+  const int64_t e0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * per;
+  const int e1 = (int)min(e0 + per, (int64_t)nnz);
+  acc_t ya[8][NR];
+  vec_t xt[8][NR];
+  int row = -1;
+  auto flush = [&]() {
+    // sum over the lanes that share rows; lane group cl keeps rows cl, cl + CPP, ..
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      acc_t v[NR];
+#pragma unroll
+      for (int j = 0; j < NR; ++j) {
+        A::norm(ya[r][j]);
+#pragma unroll
+        for (int h = LPC; h < 32; h <<= 1) A::add(ya[r][j], A::shfl(ya[r][j], h));
+        v[j] = ya[r][j];
+      }
+      if (r == cl) add_columns<FMT, NR>(yrow + ((int64_t)row * K + rb + r) * NR, v);
+    }
+  };
+  for (int e = (int)e0; e < e1; ++e) {
+    const int t = erow[e], s = col[e];
+    const ld_t* B = (const ld_t*)blk[e];
+    ld_t q[T][P];
+#pragma unroll
+    for (int p = 0; p < T; ++p)
+#pragma unroll
+      for (int k = 0; k < P; ++k) q[p][k] = __ldcs(B + (p * P + k) * 32 + lane);
+    const vec_t* xs = x + (int64_t)s * K * NR;
+    if (t != row) {
+      if (row >= 0) flush();
+      row = t;
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int j = 0; j < NR; ++j) {
+          xt[r][j] = x[((int64_t)t * K + rb + r) * NR + j];
+          ya[r][j] = A::zero();
+        }
+    }
+#pragma unroll
+    for (int p = 0; p < T; ++p) {
+      mel_t m[8];
+#pragma unroll
+      for (int k = 0; k < P; ++k) A::decode(q[p][k], m + k * V);
+      acc_t z[NR];
+#pragma unroll
+      for (int j = 0; j < NR; ++j) {
+        const vec_t xv = xs[(cl + CPP * p) * NR + j];
+        z[j] = A::zero();
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          A::fma(ya[r][j], m[r], xv);
+          A::fma(z[j], m[r], xt[r][j]);
+        }
+#pragma unroll
+        for (int h = 1; h < LPC; h <<= 1) A::add(z[j], A::shfl(z[j], h));
+      }
+      if (s != t && (lane % LPC) == 0) add_columns<FMT, NR>(yrow + ((int64_t)s * K + cl + CPP * p) * NR, z);
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int j = 0; j < NR; ++j) A::norm(ya[r][j]);
+  }
+  if (row >= 0) flush();
 }
 
 // ----------------------------------------------------------------------------- float64 block GEMV
@@ -1077,8 +1182,8 @@ static SymOp upload_op(Matrix& M, const OpHost& H, int K, const void* pool0, con
       rowof[e] = t;
     }
   op.noff = noff;
+  op.erow = (int*)up(rowof.data(), sizeof(int) * rowof.size());
   if (fx_product(M.fmt, K) && op.nnz > 0) {
-    op.erow = (int*)up(rowof.data(), sizeof(int) * rowof.size());
     op.bexp = (short*)M.alloc(sizeof(short) * op.nnz);
     { k_block_exponents<<<ceil_div(op.nnz, 8), 256, 0, s>>>(op.blk, op.erow, op.col, skip, op.nnz, K * K, op.bexp);
       ::h2mg::count_launch(); }
@@ -1252,7 +1357,8 @@ static void launch_bsgemv(Matrix& M, const SymOp& op, bool f32, const void* x, v
   // CTAs per block row: the autotuner's choice, else enough CTAs to fill the GPU when
   // the operator has few block rows
   const int tuned = op.split[FMT == FMT_DD ? FMT_F64 : FMT][nr_index(NR)];
-  const int split = force_split > 0 ? force_split : (tuned > 0 ? tuned : split_heuristic(op.nrows));
+  const int waves = force_split > 0 ? force_split : tuned;   // CTAs per SM of the kernels that take warps by entry
+  const int split = waves > 0 ? waves : split_heuristic(op.nrows);
   const int grid = op.nrows * split;
   const void* const* blk = f32 ? op.blk32 : op.blk;
   Profile& P = M.prof;
@@ -1271,29 +1377,25 @@ static void launch_bsgemv(Matrix& M, const SymOp& op, bool f32, const void* x, v
     }
     H2_CUDA(cudaEventRecord(P.ev[2 * P.used], s));
   }
-  // the float64 product has no instances of k_bsgemv for the block edges of the fixed-point one
   if constexpr (FMT == FMT_F64) {
-    if (op.bexp) {
-      launch_bsgemv_fx<NR>(op, (const double*)x, (double*)yrow, force_split > 0 ? force_split : tuned, s);
-    } else {
-      H2_REQUIRE(op.K == 16 || op.nnz == 0, H2MG_ERR_UNSUPPORTED, "block size not supported");
-      if (op.nnz > 0) {
-        k_bsgemv<16, FMT, NR><<<grid, 256, 0, s>>>(op.rowptr, op.col, blk, (const vt*)x, (yt*)yrow, split);
-        ::h2mg::count_launch();
-      }
+    if (op.bexp) launch_bsgemv_fx<NR>(op, (const double*)x, (double*)yrow, waves, s);
+  }
+  if (op.bexp && FMT == FMT_F64) {
+  } else if (op.K == 64) {
+    if constexpr (FMT != FMT_F64) {
+      k_bsgemv<64, FMT, NR><<<grid, 256, 0, s>>>(op.rowptr, op.col, blk, (const vt*)x, (yt*)yrow, split);
+      ::h2mg::count_launch();
     }
-  } else switch (op.K) {
-    case 16:
-      { k_bsgemv<16, FMT, NR><<<grid, 256, 0, s>>>(op.rowptr, op.col, blk, (const vt*)x, (yt*)yrow, split); ::h2mg::count_launch(); }
-      break;
-    case 32:
-      { k_bsgemv<32, FMT, NR><<<grid, 256, 0, s>>>(op.rowptr, op.col, blk, (const vt*)x, (yt*)yrow, split); ::h2mg::count_launch(); }
-      break;
-    case 64:
-      { k_bsgemv<64, FMT, NR><<<grid, 256, 0, s>>>(op.rowptr, op.col, blk, (const vt*)x, (yt*)yrow, split); ::h2mg::count_launch(); }
-      break;
-    default:
-      throw Error{H2MG_ERR_UNSUPPORTED, "block size not supported"};
+  } else if (op.nnz > 0) {
+    const int64_t warps = (int64_t)(waves > 0 ? waves : FX_WAVES) * FX_SMS * 8;
+    const int per = (int)((op.nnz + warps - 1) / warps);
+    const int g = ceil_div(op.nnz, 8 * (int64_t)per);
+    if (op.K == 16) {
+      k_bsgemv_small<16, FMT, NR><<<g, 256, 0, s>>>(op.erow, op.col, blk, (const vt*)x, (yt*)yrow, op.nnz, per);
+    } else if constexpr (FMT != FMT_F64) {
+      k_bsgemv_small<32, FMT, NR><<<g, 256, 0, s>>>(op.erow, op.col, blk, (const vt*)x, (yt*)yrow, op.nnz, per);
+    }
+    ::h2mg::count_launch();
   }
   H2_LAUNCH_CHECK();
   if (rec && P.cap_ev) {
@@ -1501,7 +1603,7 @@ template <int FMT, int NR>
 static void tune_one(Matrix& M, SymOp& op, bool pts, int opi, cudaStream_t s, cudaEvent_t e0, cudaEvent_t e1,
                      std::vector<double>& rep) {
   if (op.nrows == 0 || op.nnz == 0) return;
-  const bool fx = FMT == FMT_F64 && op.bexp;   // there a candidate is the CTAs per SM of the launch
+  const bool fx = op.K < 64 || (FMT == FMT_F64 && op.bexp);   // a candidate is the CTAs per SM of the launch
   const int heur = fx ? FX_WAVES : split_heuristic(op.nrows);
   const int cands[] = {1, 2, 4, 8, 16, 32, 64};
   const float base = time_product<FMT, NR>(M, op, pts, heur, 3, s, e0, e1);

@@ -28,10 +28,10 @@ struct SymOp {
   int* col = nullptr;     // [nnz]
   const void** blk = nullptr;      // [nnz] block pointers into the primary pool
   const void** blk32 = nullptr;    // [nnz] block pointers into the FP32 pool (or null)
-  int* erow = nullptr;    // [nnz] row of each entry, and
-  short* bexp = nullptr;  // [nnz] its block's exponent (fixed.cuh): float64 blocks of 32 and 64 only
+  int* erow = nullptr;    // [nnz] row of each entry
+  short* bexp = nullptr;  // [nnz] exponent of each block (fixed.cuh): float64 blocks of 32 and 64 only
   int64_t noff = 0;       // off-diagonal entries (each adds K transposed partials)
-  // CTAs per block row (with bexp: CTAs per SM) chosen by the autotuner, per element format
+  // CTAs per block row (per SM, for the kernels that deal warps by entry) chosen by the autotuner, per element format
   // (F64, DF, F32) and column group size (NR = 1, 2, 4); 0 = the fixed heuristic
   int split[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
   int64_t bytes(int eb, int vb) const {   // algorithmic bytes of one product
