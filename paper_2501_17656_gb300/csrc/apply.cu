@@ -11,8 +11,8 @@
 // K x K blocks (swizzled so that every warp load is one contiguous 512 B segment),
 // and each block is used twice -- y_t += B x_s for its row and, for s != t, the
 // transposed product B^T x_t for its column, both added atomically into a zeroed row
-// buffer. The upward pass (k_up_leaf, k_up_multi) forms the cluster coefficients of
-// every level; the downward pass (k_down_multi) adds the transfer from the parent to
+// buffer. The upward pass (k_leaf_in, k_up_tree) forms the cluster coefficients of
+// every level; the downward pass (k_down_tree) adds the transfer from the parent to
 // each level's row results and writes the finest level out (k_leaf_final at i = 1).
 //
 // Arithmetic per block format: F64 (DFMA), DF (double-float on the FP32 pipes: the
@@ -726,69 +726,192 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
 }
 
 // ----------------------------------------------------------------------------- passes
-// point vectors (float64, user order, column j at x + j*ldx) -> padded tree slots
-template <int FMT, int NR>
-__global__ void k_pts_in(const double* __restrict__ x, int64_t ldx, const int* __restrict__ slot_of, int64_t n,
-                         typename Ar<FMT>::vec_t* __restrict__ xp) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int64_t sl = slot_of[i];
+// A value another CTA of this launch has written: read from L2.
+__device__ __forceinline__ float load_cg(const float* p) { return __ldcg(p); }
+__device__ __forceinline__ double load_cg(const double* p) { return __ldcg(p); }
+__device__ __forceinline__ float2 load_cg(const float2* p) { return __ldcg(p); }
+__device__ __forceinline__ double2 load_cg(const double2* p) { return __ldcg(p); }
+
+// What a product's first kernel does besides its own work. Its input vector is x (float64,
+// column j at x + j * ldx) or, inside a CG step (r given), the new direction: per column,
+// rho' = r^T r from its partials; stop if rho' <= thresh, else p = r + (rho' / rho) p, which
+// is written back to p = x. Every CTA takes the same decision from the same partials, and
+// the state it writes is not what the others read. It also clears the row sums that the
+// block products add into.
+struct VecIn {
+  const double* x;
+  int64_t ldx;
+  const double* r;          // CG: residual (leading dimension ldx), or null
+  const double* prr;        // CG: partials of r^T r, CG_PARTS per column
+  int np, par;
+  CGState* st;
+  uint4* zero[3];           // regions cleared by the grid
+  int64_t nzero[3];         // their sizes in 16-byte units
+};
+
+// Per column: whether the direction changes, and by which factor. Warp j sums column j's
+// partials (every CTA in the same order), so that the columns take one barrier together.
+template <int NR>
+__device__ __forceinline__ void cg_beta(const VecIn& in, bool* go, double* be) {
+  __shared__ double sbe[NR];
+  __shared__ int sgo[NR];
 #pragma unroll
-  for (int j = 0; j < NR; ++j) xp[sl * NR + j] = Ar<FMT>::from_d(x[i + j * ldx]);
+  for (int j = 0; j < NR; ++j) {
+    go[j] = false;
+    be[j] = 0.0;
+  }
+  if (!in.r) return;
+  const int j = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (j < NR) {
+    const double* part = in.prr + j * CG_PARTS;
+    CGState* st = in.st + j;
+    const int stopped = st->stopped;
+    const double rho = st->rho[in.par], thresh = st->thresh;
+    double rn = 0.0;
+    for (int i = lane; i < in.np; i += 32) rn += part[i];
+    for (int o = 16; o > 0; o >>= 1) rn += __shfl_xor_sync(0xffffffffu, rn, o);
+    if (lane == 0) {
+      const bool stop = stopped || rn <= thresh;
+      sgo[j] = !stop;
+      sbe[j] = stop ? 0.0 : rn / rho;
+      if (blockIdx.x == 0) {
+        if (stop)
+          st->stopped = 1;
+        else
+          st->rho[in.par ^ 1] = rn;
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < NR; ++q) {
+    go[q] = sgo[q] != 0;
+    be[q] = sbe[q];
+  }
+}
+__device__ __forceinline__ double cg_value(const VecIn& in, int64_t i, bool go, double be) {
+  double v = in.x[i];
+  if (go) {
+    v = fma(be, v, in.r[i]);
+    const_cast<double*>(in.x)[i] = v;
+  }
+  return v;
+}
+__device__ __forceinline__ void clear_regions(const VecIn& in) {
+#pragma unroll
+  for (int z = 0; z < 3; ++z)
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < in.nzero[z];
+         i += (int64_t)gridDim.x * blockDim.x)
+      in.zero[z][i] = make_uint4(0, 0, 0, 0);
 }
 
-// coefficient vectors (float64, KC per cluster, column j at x + j*ldx) -> interleaved
+// coefficient vectors (KC per cluster) -> interleaved, for operators without transfers
 template <int FMT, int NR>
-__global__ void k_coef_in(const double* __restrict__ x, int64_t ldx, int64_t n,
-                          typename Ar<FMT>::vec_t* __restrict__ xc) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+__global__ void __launch_bounds__(256) k_coef_in(VecIn in, int64_t n, typename Ar<FMT>::vec_t* __restrict__ xc) {
+  bool go[NR];
+  double be[NR];
+  cg_beta<NR>(in, go, be);
+  clear_regions(in);
+  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256)
 #pragma unroll
-  for (int j = 0; j < NR; ++j) xc[i * NR + j] = Ar<FMT>::from_d(x[i + j * ldx]);
+    for (int j = 0; j < NR; ++j) xc[i * NR + j] = Ar<FMT>::from_d(cg_value(in, i + j * in.ldx, go[j], be[j]));
 }
 
-// x_hat(leaf l)[b] = sum_i U_l[i, b] x_l[i]   (UT = U^T, KC x KD column-major)
+// Float -> double by moving the bits: the conversion instruction runs at the float64 rate (2
+// per clock and SM), as many as the products it feeds. Subnormals become zero.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f), m = u & 0x7FFFFFFFu;
+  return m < 0x00800000u ? 0.0 : __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double d) { return d; }
+
+// Values of the leaf kernels: float64, or double-double.
+template <int FMT>
+struct LeafVal {
+  using t = double;
+  __device__ static t zero() { return 0.0; }
+  __device__ static void fma(t& a, double u, t x) { a = ::fma(u, x, a); }
+  __device__ static void add(t& a, t b) { a += b; }
+  __device__ static t in(typename Ar<FMT>::vec_t v) { return Ar<FMT>::to_d(v); }
+  __device__ static typename Ar<FMT>::vec_t out(t a) { return Ar<FMT>::from_d(a); }
+  __device__ static t row(typename Ar<FMT>::yo_t v) { return (double)v; }
+  __device__ static double val(t a) { return a; }
+};
+template <>
+struct LeafVal<FMT_DD> {
+  using t = double2;
+  __device__ static t zero() { return make_double2(0.0, 0.0); }
+  __device__ static void fma(t& a, double u, t x) { dd_fma(a.x, a.y, u, x.x, x.y); }
+  __device__ static void add(t& a, t b) { dd_add(a.x, a.y, b.x, b.y); }
+  __device__ static t in(double2 v) { return v; }
+  __device__ static double2 out(t a) {
+    dd_norm(a.x, a.y);
+    return a;
+  }
+  __device__ static t row(double2 v) { return v; }
+  __device__ static double val(t a) { return a.x + a.y; }
+};
+
+constexpr int LEAF_CTAS = CG_PARTS;   // the leaf kernels' grids: one partial per CTA at most
+
+// Point vectors (user order) -> padded tree slots, zero in the padding, and, with a far
+// field, x_hat(leaf l)[b] = sum_i U_l[i, b] x_l[i] (UT = U^T, KC x KD column-major): 256 / KC
+// threads share each sum.
 template <int FMT, class BT, int NR>
-__global__ void k_up_leaf(const BT* __restrict__ UT, int KD, int KC,
-                          const typename Ar<FMT>::vec_t* __restrict__ xp,
-                          typename Ar<FMT>::vec_t* __restrict__ xc) {
-  int l = blockIdx.x;
-  const BT* Ul = UT + (int64_t)l * KD * KC;
-  if constexpr (FMT == FMT_DD) {   // double-double coefficients
-    __shared__ double2 xd[64 * NR];
-    for (int i = threadIdx.x; i < KD * NR; i += blockDim.x) xd[i] = xp[(int64_t)l * KD * NR + i];
-    __syncthreads();
-    for (int b = threadIdx.x; b < KC; b += blockDim.x) {
-      double2 acc[NR];
+__global__ void __launch_bounds__(256) k_leaf_in(VecIn in, const BT* __restrict__ UT, int KD, int KC, int nleaf,
+                                                 const int* __restrict__ leafoff, const int* __restrict__ perm,
+                                                 typename Ar<FMT>::vec_t* __restrict__ xp,
+                                                 typename Ar<FMT>::vec_t* __restrict__ xc) {
+  using V = LeafVal<FMT>;
+  using v_t = typename V::t;
+  __shared__ v_t xs[64 * NR];
+  __shared__ v_t red[256 * NR];
+  bool go[NR];
+  double be[NR];
+  cg_beta<NR>(in, go, be);
+  clear_regions(in);
+  const int b = threadIdx.x % KC, part = threadIdx.x / KC, parts = 256 / KC;
+  for (int l = blockIdx.x; l < nleaf; l += gridDim.x) {
+    const int p0 = leafoff[l], nl = leafoff[l + 1] - p0;
+    for (int e = threadIdx.x; e < KD * NR; e += 256) {
+      const int i = e % KD, j = e / KD;
+      typename Ar<FMT>::vec_t v = Ar<FMT>::from_d(0.0);
+      if (i < nl) {
+        const int64_t o = perm[p0 + i] + j * in.ldx;
+        bool g = go[0];
+        double f = be[0];
 #pragma unroll
-      for (int j = 0; j < NR; ++j) acc[j] = make_double2(0.0, 0.0);
-      for (int i = 0; i < KD; ++i) {
-        const double u = (double)Ul[b + i * KC];
-#pragma unroll
-        for (int j = 0; j < NR; ++j) dd_fma(acc[j].x, acc[j].y, u, xd[i * NR + j].x, xd[i * NR + j].y);
+        for (int q = 1; q < NR; ++q)
+          if (j == q) {
+            g = go[q];
+            f = be[q];
+          }
+        v = Ar<FMT>::from_d(cg_value(in, o, g, f));
       }
-#pragma unroll
-      for (int j = 0; j < NR; ++j) {
-        dd_norm(acc[j].x, acc[j].y);
-        xc[((int64_t)l * KC + b) * NR + j] = acc[j];
-      }
+      xp[((int64_t)l * KD + i) * NR + j] = v;
+      xs[i * NR + j] = V::in(v);
     }
-  } else {
-    __shared__ double xs[64 * NR];
-    for (int i = threadIdx.x; i < KD * NR; i += blockDim.x) xs[i] = Ar<FMT>::to_d(xp[(int64_t)l * KD * NR + i]);
+    if (!UT) continue;
     __syncthreads();
-    for (int b = threadIdx.x; b < KC; b += blockDim.x) {
-      double acc[NR];
+    const BT* Ul = UT + (int64_t)l * KD * KC + b;
+    v_t acc[NR];
 #pragma unroll
-      for (int j = 0; j < NR; ++j) acc[j] = 0.0;
-      for (int i = 0; i < KD; ++i) {
-        double u = (double)Ul[b + i * KC];
+    for (int j = 0; j < NR; ++j) acc[j] = V::zero();
+#pragma unroll 4
+    for (int i = part; i < KD; i += parts) {
+      const double u = widen(Ul[i * KC]);
 #pragma unroll
-        for (int j = 0; j < NR; ++j) acc[j] += u * xs[i * NR + j];
-      }
-#pragma unroll
-      for (int j = 0; j < NR; ++j) xc[((int64_t)l * KC + b) * NR + j] = Ar<FMT>::from_d(acc[j]);
+      for (int j = 0; j < NR; ++j) V::fma(acc[j], u, xs[i * NR + j]);
     }
+#pragma unroll
+    for (int j = 0; j < NR; ++j) red[(part * KC + b) * NR + j] = acc[j];
+    __syncthreads();
+    for (int e = threadIdx.x; e < KC * NR; e += 256) {
+      v_t t = red[e];
+      for (int q = 1; q < parts; ++q) V::add(t, red[q * KC * NR + e]);
+      xc[(int64_t)l * KC * NR + e] = V::out(t);
+    }
+    __syncthreads();
   }
 }
 
@@ -798,11 +921,10 @@ __global__ void k_up_leaf(const BT* __restrict__ UT, int KD, int KC,
 // the upward pass uses the transposed product E'_c^T x_c (reduce-scatter over the
 // lanes that share a column), the downward pass the row product E'_c y_parent.
 //
-// One launch covers up to 3 (upward) or 4 (downward) consecutive tree levels: a CTA
-// owns a subtree (8 clusters of the bottom level going up; one cluster of the top
-// level and its descendants going down), keeps the intermediate coefficients in
-// shared memory and writes every level's coefficients to global memory, since the
-// coupling products and the next launch read them.
+// The upward pass is one launch: a CTA owns two siblings of the bottom level, and of the two
+// CTAs below a cluster the one that comes second goes on with it (k_up_tree). The downward
+// pass covers up to five levels per launch: a CTA owns 4 (or 2) clusters of the bottom level
+// and recomputes the path of their ancestors, one transfer per level (k_down_tree).
 
 // v = E'^T x over the TPW tiles starting at tile t0 of one K x K transfer at B
 // (warp-wide; x: K*NR values, any address space). A tile covers CPP whole columns of
@@ -933,101 +1055,158 @@ __device__ __forceinline__ void warp_transfer(const void* __restrict__ Bv, const
       for (int j = 0; j < NR; ++j) s[(rb + r) * NR + j] = ya[r][j];
 }
 
-// Levels of one pass launch: step k works on tree level `lev[k]`.
-struct PassLevels {
-  const void* E[4];   // transfer pool of the (child) clusters of step k (nullptr: top level, no parent)
-  void* out[4];       // up: parent coefficients of step k; down: coefficients of step k's clusters
-  int slot[4];        // down: first slot of step k's level (row buffer index)
-  int n[4];           // clusters of step k's level
-};
-
-// Upward pass over `steps` levels: step k maps the children (level lc - k) of this
-// CTA's subtree to their parents. x_bottom: coefficients of level lc. At step k the
-// 8 >> k children of the CTA share its 8 warps (1 << k warps per transfer).
+// Upward pass from level `lb` (2^lb clusters, coefficients xc + slot0(lb) ..) to level `lt`,
+// in one launch: CTA b maps clusters 2b and 2b + 1 of level lb to their parent; then one
+// ticket per parent pair decides which CTA goes on: the first to arrive leaves its result in
+// xc and ends, the second reads it and maps both to the next level. No CTA waits for another.
+// A level takes two transfers on 8 warps (4 per transfer); eight clusters per CTA with a warp
+// each, as before, kept 64 of the 152 SMs busy for 512 clusters and took a second launch.
+// Bound by latency, about 2 us per level: 512 clusters of 64 over four levels (FP32, one
+// column) 16 -> 10 us.
+// With in.x the bottom coefficients come from the float64 input vector: the CTA writes them
+// to xc for the block product and does the rest of VecIn's work. The tickets are zero
+// between launches: the second arrival resets its own.
 template <int K, int FMT, int NR>
-__global__ void __launch_bounds__(256) k_up_multi(PassLevels pl, int steps,
-                                                  const typename Ar<FMT>::vec_t* __restrict__ xbottom) {
+__global__ void __launch_bounds__(256) k_up_tree(const char* __restrict__ epool, VecIn in,
+                                                 typename Ar<FMT>::vec_t* __restrict__ xc, int lb, int lt, int ts,
+                                                 unsigned* __restrict__ ticket) {
   using A = Ar<FMT>;
   using vec_t = typename A::vec_t;
   using acc_t = typename A::acc_t;
   constexpr size_t kBlk = (size_t)K * K * (FMT == FMT_F32 ? 4 : 8);
-  __shared__ acc_t v[8][K * NR];
-  __shared__ vec_t xin[4][K * NR];
+  __shared__ acc_t v[2][K * NR];
+  __shared__ vec_t xin[2][K * NR];
+  __shared__ unsigned second;
   const int w = threadIdx.x >> 5;
-  for (int k = 0; k < steps; ++k) {
-    const int per = 8 >> k;                 // children of this CTA at step k
-    const int b = w >> k, sub = w & ((1 << k) - 1);
-    const int c = blockIdx.x * per + b;     // child index within its level
-    if (c < pl.n[k]) {
-      const vec_t* x = (k == 0) ? xbottom + (int64_t)c * K * NR : xin[b];
-      warp_transfer_t_part<K, FMT, NR>((const char*)pl.E[k] + (size_t)c * kBlk, x, v[b], 1 << k, sub);
+  auto slot0 = [&](int l) { return (int64_t)((1 << l) - (1 << ts)); };
+  int idx = blockIdx.x;                       // parent at level l - 1
+  vec_t* xb = xc + (slot0(lb) + 2 * (int64_t)idx) * K * NR;
+  if (in.x) {
+    bool go[NR];
+    double be[NR];
+    cg_beta<NR>(in, go, be);
+    clear_regions(in);
+#pragma unroll
+    for (int j = 0; j < NR; ++j)
+      for (int e = threadIdx.x; e < 2 * K; e += 256) {
+        const int64_t i = 2 * (int64_t)idx * K + e;
+        const vec_t o = A::from_d(cg_value(in, i + j * in.ldx, go[j], be[j]));
+        xin[e / K][(e % K) * NR + j] = o;
+        xb[e * NR + j] = o;
+      }
+  } else {
+    for (int e = threadIdx.x; e < 2 * K * NR; e += 256) xin[e / (K * NR)][e % (K * NR)] = xb[e];
+  }
+  __syncthreads();
+  for (int l = lb;; --l) {
+    const int b = w >> 2;
+    warp_transfer_t_part<K, FMT, NR>(epool + (size_t)(slot0(l) + 2 * (int64_t)idx + b) * kBlk, xin[b], v[b], 4, w & 3);
+    __syncthreads();
+    vec_t* out = xc + slot0(l - 1) * K * NR;
+    for (int i = threadIdx.x; i < K * NR; i += 256) {
+      acc_t t = v[0][i];
+      A::add(t, v[1][i]);
+      const vec_t o = A::out(t);
+      out[(int64_t)idx * K * NR + i] = o;
+      xin[idx & 1][i] = o;
+    }
+    if (l - 1 == lt) return;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      unsigned* t = ticket + slot0(l - 1) + (idx & ~1);
+      second = atomicAdd(t, 1);
+      if (second) *t = 0;
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < (per / 2) * K * NR; idx += blockDim.x) {
-      const int pb = idx / (K * NR), i = idx % (K * NR);
-      const int c0 = blockIdx.x * per + 2 * pb;
-      if (c0 < pl.n[k]) {
-        acc_t t = v[2 * pb][i];
-        A::add(t, v[2 * pb + 1][i]);
-        const vec_t o = A::out(t);
-        ((vec_t*)pl.out[k])[(int64_t)(c0 >> 1) * K * NR + i] = o;
-        xin[pb][i] = o;
-      }
-    }
+    if (!second) return;
+    __threadfence();
+    const int sib = idx ^ 1;
+    for (int i = threadIdx.x; i < K * NR; i += 256) xin[sib & 1][i] = load_cg(out + (int64_t)sib * K * NR + i);
+    idx >>= 1;
     __syncthreads();
   }
 }
 
-// Downward pass over `steps` levels from this CTA's top cluster (level lt): step k
-// forms y_c = yrow_c + E'_c y_parent(c) for the 2^k descendants at level lt + k
-// (no transfer term at the coupling top level), the CTA's 8 warps sharing each
-// transfer's tiles (8 >> k warps per transfer). ypar: coefficients of level lt - 1.
-// On the last step of the last launch the result goes to yout (float64, column j at
-// yout + j * ldo) instead of the coefficient buffer, when yout is given.
-template <int K, int FMT, int NR>
-__global__ void __launch_bounds__(256) k_down_multi(PassLevels pl, int steps,
-                                                    const typename Ar<FMT>::yo_t* __restrict__ yrow,
-                                                    const typename Ar<FMT>::vec_t* __restrict__ ypar,
-                                                    double* __restrict__ yout, int64_t ldo) {
+// part[j * CG_PARTS + CTA] = sum of v over the threads with threadIdx.x % NR == j (256 threads).
+template <int NR>
+__device__ __forceinline__ void column_partials(double v, double* __restrict__ part) {
+  __shared__ double sh[8][NR];
+  for (int o = 16; o >= NR; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) < NR) sh[threadIdx.x >> 5][threadIdx.x & 31] = v;
+  __syncthreads();
+  if (threadIdx.x < NR) {
+    double s = 0.0;
+    for (int w = 0; w < 8; ++w) s += sh[w][threadIdx.x];
+    part[threadIdx.x * CG_PARTS + blockIdx.x] = s;
+  }
+}
+
+// Downward pass from level lt to level lb (at most 5 levels): y_c = yrow_c + E'_c y_parent(c)
+// (no transfer term at the coupling top level ts). A CTA owns S clusters of level lb; above
+// the levels where they are S and S/2 clusters it follows one cluster per level, which the
+// CTAs below that cluster all compute: one transfer on 8 warps is a step of about a
+// microsecond, while a CTA per top cluster left most SMs idle (512 clusters, five levels:
+// 17 -> 9 us; S = 4 only where S = 2 gives every SM several CTAs). ypar: coefficients of level
+// lt - 1. The last level goes to yout (float64, column j at yout + j * ldo), when given, with
+// the CTA's partial of pdot_j^T yout_j (leading dimension ldo) in part[j * CG_PARTS + CTA],
+// else to yc.
+template <int K, int FMT, int NR, int S>
+__global__ void __launch_bounds__(256) k_down_tree(const char* __restrict__ epool,
+                                                   const typename Ar<FMT>::yo_t* __restrict__ yrow,
+                                                   const typename Ar<FMT>::vec_t* __restrict__ ypar,
+                                                   typename Ar<FMT>::vec_t* __restrict__ yc, int lt, int lb, int ts,
+                                                   double* __restrict__ yout, int64_t ldo,
+                                                   const double* __restrict__ pdot, double* __restrict__ part) {
   using A = Ar<FMT>;
   using vec_t = typename A::vec_t;
   using acc_t = typename A::acc_t;
   constexpr size_t kBlk = (size_t)K * K * (FMT == FMT_F32 ? 4 : 8);
   constexpr int T = K * K / 256;
   __shared__ acc_t sv[8][K * NR];
-  __shared__ vec_t ys[8][K * NR];
+  __shared__ vec_t ys[2][S][K * NR];            // this level's and the parents' coefficients
   const int w = threadIdx.x >> 5;
-  for (int k = 0; k < steps; ++k) {
-    const int per = 1 << k;                       // clusters of this CTA at step k
-    const int wpb = 8 >> k;                       // warps per transfer
-    const int wpe = wpb < T ? wpb : T;            // of which hold tiles
-    const int b = w / wpb, sub = w % wpb;
-    const int c = blockIdx.x * per + b;           // cluster index within its level
-    if (pl.E[k] && c < pl.n[k] && sub < wpe) {
-      const vec_t* yp = (k == 0) ? ypar + (int64_t)(c >> 1) * K * NR : ys[b >> 1];
-      const int tpw = T / wpe;
-      warp_transfer<K, FMT, NR>((const char*)pl.E[k] + (size_t)c * kBlk, yp, sv[w], sub * tpw, (sub + 1) * tpw);
-    }
-    __syncthreads();   // every parent value and partial of this step is in place
-    const bool last = (k == steps - 1) && yout;
-    for (int idx = threadIdx.x; idx < per * K * NR; idx += blockDim.x) {
-      const int bb = idx / (K * NR), i = idx % (K * NR);
-      const int cc = blockIdx.x * per + bb;
-      if (cc >= pl.n[k]) continue;
-      acc_t acc = A::from_yo(yrow[(int64_t)(pl.slot[k] + cc) * K * NR + i]);
-      if (pl.E[k])
-        for (int q = 0; q < wpe; ++q) A::add(acc, sv[bb * wpb + q][i]);
-      const vec_t o = A::out(acc);
-      if (last) {
-        const int a = i / NR, j = i % NR;
-        yout[(int64_t)cc * K + a + j * ldo] = A::to_d(o);
-      } else {
-        ((vec_t*)pl.out[k])[(int64_t)cc * K * NR + i] = o;
-        ys[bb][i] = o;
+  auto slot0 = [&](int l) { return (int64_t)((1 << l) - (1 << ts)); };
+  double dot = 0.0;
+  const int nb = 1 << lb;
+  for (int c0 = blockIdx.x * S; c0 < nb; c0 += gridDim.x * S)
+    for (int l = lt; l <= lb; ++l) {
+      const int first = c0 >> (lb - l);                            // clusters first .. first + per - 1
+      const int per = max(1, min(S >> (lb - l), (1 << l) - first));
+      const int share = per <= 1 ? 8 : (per == 2 ? 4 : 2);         // warps per transfer,
+      const int hold = share < T ? share : T;                      // of which hold tiles
+      vec_t(*cur)[K * NR] = ys[l & 1];
+      vec_t(*par)[K * NR] = ys[(l & 1) ^ 1];
+      const int b = w / share, sub = w % share;
+      if (l > ts && b < per && sub < hold) {
+        const int c = first + b, tpw = T / hold;
+        const vec_t* yp = l == lt ? ypar + (int64_t)(c >> 1) * K * NR : par[(c >> 1) - (first >> 1)];
+        warp_transfer<K, FMT, NR>(epool + (size_t)(slot0(l) + c) * kBlk, yp, sv[w], sub * tpw, (sub + 1) * tpw);
       }
+      __syncthreads();   // every parent value and partial of this level is in place
+      const bool last = l == lb;
+      for (int e = threadIdx.x; e < per * K * NR; e += 256) {
+        const int bb = e / (K * NR), i = e % (K * NR);
+        const int c = first + bb;
+        acc_t acc = A::from_yo(yrow[(slot0(l) + c) * K * NR + i]);
+        if (l > ts)
+          for (int q = 0; q < hold; ++q) A::add(acc, sv[bb * share + q][i]);
+        const vec_t o = A::out(acc);
+        if (!last) {
+          cur[bb][i] = o;
+        } else if (yout) {
+          const int a = i / NR, j = i % NR;      // j is the same for all of a thread's e: NR divides 256
+          const int64_t at = (int64_t)c * K + a + j * ldo;
+          const double q = A::to_d(o);
+          yout[at] = q;
+          if (pdot) dot = fma(pdot[at], q, dot);
+        } else {
+          yc[(slot0(l) + c) * K * NR + i] = o;
+        }
+      }
+      __syncthreads();
     }
-    __syncthreads();
-  }
+  if (pdot) column_partials<NR>(dot, part);
 }
 
 // natural column-major K x K blocks (float64) -> swizzled blocks in a format
@@ -1051,58 +1230,54 @@ __global__ void k_swizzle_blocks(const double* __restrict__ in, int K, void* __r
   }
 }
 
-// y(point) = yrowD + U y_hat(leaf), scattered to user order (column j at y + j*ldy).
+// y(point) = yrowD + U y_hat(leaf), scattered to user order (column j at y + j*ldy), and, with
+// pdot given, the CTA's partial of pdot_j^T y_j (as in k_down_tree). 256 / KD threads share
+// each sum.
 template <int FMT, class BT, int NR>
-__global__ void k_leaf_final(int KD, int KC, const typename Ar<FMT>::yo_t* __restrict__ yrow,
-                             const BT* __restrict__ U, const typename Ar<FMT>::vec_t* __restrict__ yleaf,
-                             const int* __restrict__ leafoff, const int* __restrict__ perm,
-                             double* __restrict__ y, int64_t ldy) {
-  using A = Ar<FMT>;
-  int l = blockIdx.x;
-  int p0 = leafoff[l], nl = leafoff[l + 1] - p0;
-  if constexpr (FMT == FMT_DD) {   // double-double sums, rounded to float64 on output
-    __shared__ double2 pd[64 * NR];
-    if (U)
-      for (int i = threadIdx.x; i < KC * NR; i += blockDim.x) pd[i] = yleaf[(int64_t)l * KC * NR + i];
-    __syncthreads();
-    for (int i = threadIdx.x; i < nl; i += blockDim.x) {
-      double2 v[NR];
+__global__ void __launch_bounds__(256) k_leaf_final(int KD, int KC, int nleaf,
+                                                    const typename Ar<FMT>::yo_t* __restrict__ yrow,
+                                                    const BT* __restrict__ U,
+                                                    const typename Ar<FMT>::vec_t* __restrict__ yleaf,
+                                                    const int* __restrict__ leafoff, const int* __restrict__ perm,
+                                                    double* __restrict__ y, int64_t ldy,
+                                                    const double* __restrict__ pdot, double* __restrict__ part) {
+  using V = LeafVal<FMT>;
+  using v_t = typename V::t;
+  __shared__ v_t ps[64 * NR];
+  __shared__ v_t red[256 * NR];
+  const int i = threadIdx.x % KD, pt = threadIdx.x / KD, parts = 256 / KD;
+  double dot = 0.0;
+  for (int l = blockIdx.x; l < nleaf; l += gridDim.x) {
+    const int p0 = leafoff[l], nl = leafoff[l + 1] - p0;
+    if (U) {
+      for (int e = threadIdx.x; e < KC * NR; e += 256) ps[e] = V::in(yleaf[(int64_t)l * KC * NR + e]);
+      __syncthreads();
+      const BT* Ul = U + (int64_t)l * KD * KC + i;
+      v_t acc[NR];
 #pragma unroll
-      for (int j = 0; j < NR; ++j) v[j] = yrow[((int64_t)l * KD + i) * NR + j];
-      if (U) {
-        const BT* Ul = U + (int64_t)l * KD * KC;
-        for (int b = 0; b < KC; ++b) {
-          const double u = (double)Ul[i + b * KD];
+      for (int j = 0; j < NR; ++j) acc[j] = V::zero();
+#pragma unroll 4
+      for (int b = pt; b < KC; b += parts) {
+        const double u = widen(Ul[b * KD]);
 #pragma unroll
-          for (int j = 0; j < NR; ++j) dd_fma(v[j].x, v[j].y, u, pd[b * NR + j].x, pd[b * NR + j].y);
-        }
+        for (int j = 0; j < NR; ++j) V::fma(acc[j], u, ps[b * NR + j]);
       }
-      const int64_t o = perm[p0 + i];
 #pragma unroll
-      for (int j = 0; j < NR; ++j) y[o + j * ldy] = v[j].x + v[j].y;
+      for (int j = 0; j < NR; ++j) red[(pt * KD + i) * NR + j] = acc[j];
+      __syncthreads();
     }
-  } else {
-    __shared__ double ps[64 * NR];
-    if (U)
-      for (int i = threadIdx.x; i < KC * NR; i += blockDim.x) ps[i] = A::to_d(yleaf[(int64_t)l * KC * NR + i]);
+    for (int e = threadIdx.x; e < nl * NR; e += 256) {
+      v_t v = V::row(yrow[(int64_t)l * KD * NR + e]);
+      if (U)
+        for (int q = 0; q < parts; ++q) V::add(v, red[q * KD * NR + e]);
+      const int64_t o = perm[p0 + e / NR] + (e % NR) * ldy;
+      const double r = V::val(v);
+      y[o] = r;
+      if (pdot) dot = fma(pdot[o], r, dot);
+    }
     __syncthreads();
-    for (int i = threadIdx.x; i < nl; i += blockDim.x) {
-      double v[NR];
-#pragma unroll
-      for (int j = 0; j < NR; ++j) v[j] = (double)yrow[((int64_t)l * KD + i) * NR + j];
-      if (U) {
-        const BT* Ul = U + (int64_t)l * KD * KC;
-        for (int b = 0; b < KC; ++b) {
-          double u = (double)Ul[i + b * KD];
-#pragma unroll
-          for (int j = 0; j < NR; ++j) v[j] += u * ps[b * NR + j];
-        }
-      }
-      const int64_t o = perm[p0 + i];
-#pragma unroll
-      for (int j = 0; j < NR; ++j) y[o + j * ldy] = v[j];
-    }
   }
+  if (pdot) column_partials<NR>(dot, part);
 }
 
 __global__ void k_transpose_blocks(const double* __restrict__ in, int R, int C, double* __restrict__ out) {
@@ -1299,6 +1474,7 @@ void setup_operators(Matrix& M) {
   // product workspaces hold up to NRMAX interleaved columns
   size_t ncoef = (size_t)std::max(M.nslots(), 1) * M.KC * NRMAX;
   size_t npts = (size_t)(1 << L) * M.KD * NRMAX;
+  M.d_ticket = (unsigned*)M.alloc(sizeof(unsigned) * std::max(M.nslots(), 1));
   M.wx.p = M.alloc(8 * ncoef);
   M.wyrow.p = M.alloc(8 * ncoef);
   M.wyc.p = M.alloc(8 * ncoef);
@@ -1349,11 +1525,10 @@ static void allow_fx_smem() {
 
 template <int FMT, int NR>
 static void launch_bsgemv(Matrix& M, const SymOp& op, bool f32, const void* x, void* yrow, cudaStream_t s,
-                          int force_split = 0) {
+                          int force_split = 0) {   // yrow: cleared by the caller
   using vt = typename Ar<FMT>::vec_t;
   using yt = typename Ar<FMT>::yo_t;
   if (op.nrows == 0) return;
-  H2_CUDA(cudaMemsetAsync(yrow, 0, sizeof(yt) * (size_t)op.nrows * op.K * NR, s));
   // CTAs per block row: the autotuner's choice, else enough CTAs to fill the GPU when
   // the operator has few block rows
   const int tuned = op.split[FMT == FMT_DD ? FMT_F64 : FMT][nr_index(NR)];
@@ -1409,68 +1584,72 @@ static void launch_bsgemv(Matrix& M, const SymOp& op, bool f32, const void* x, v
   }
 }
 
-// Upward pass from tree level `lb` (coefficients at xc + cslot(lb)) to level `ltop`:
-// children of level l + 1 -> parents of level l, up to 3 levels per launch.
+// Upward pass from tree level `lb` to level `ts`. `in` (optional): the work of the product's
+// first kernel, which this launch takes over.
 template <int FMT, int NR>
-static void pass_up(const Matrix& M, const char* epool, size_t eb, void* xc, int lb, int ltop, cudaStream_t s) {
+static void pass_up(const Matrix& M, const char* epool, void* xc, int lb, int ts, unsigned* ticket, cudaStream_t s,
+                    const VecIn* in = nullptr) {
   using vt = typename Ar<FMT>::vec_t;
   const int KC = M.KC;
-  auto cslot = [&](int ell) { return (vt*)xc + (size_t)M.slot0(ell) * KC * NR; };
-  for (int lc = lb; lc > ltop;) {
-    const int steps = std::min(3, lc - ltop);
-    PassLevels pl{};
-    for (int k = 0; k < steps; ++k) {
-      pl.E[k] = epool + (size_t)M.slot0(lc - k) * KC * KC * eb;
-      pl.out[k] = cslot(lc - k - 1);
-      pl.n[k] = 1 << (lc - k);
-    }
-    const int grid = ceil_div(1 << lc, 8);
-    switch (KC) {
-      case 16: { k_up_multi<16, FMT, NR><<<grid, 256, 0, s>>>(pl, steps, cslot(lc)); ::h2mg::count_launch(); } break;
-      case 32: { k_up_multi<32, FMT, NR><<<grid, 256, 0, s>>>(pl, steps, cslot(lc)); ::h2mg::count_launch(); } break;
-      default: { k_up_multi<64, FMT, NR><<<grid, 256, 0, s>>>(pl, steps, cslot(lc)); ::h2mg::count_launch(); } break;
-    }
+  vt* x = (vt*)xc;
+  if (lb == ts) {
+    if (!in) return;
+    const int64_t n = (int64_t)(1 << lb) * KC;
+    { k_coef_in<FMT, NR><<<std::min(ceil_div(n, 256), 1024), 256, 0, s>>>(*in, n, x); ::h2mg::count_launch(); }
     H2_LAUNCH_CHECK();
-    lc -= steps;
+    return;
   }
+  const VecIn vi = in ? *in : VecIn{};
+  const int grid = 1 << (lb - 1);
+  switch (KC) {
+    case 16: { k_up_tree<16, FMT, NR><<<grid, 256, 0, s>>>(epool, vi, x, lb, ts, ts, ticket); ::h2mg::count_launch(); } break;
+    case 32: { k_up_tree<32, FMT, NR><<<grid, 256, 0, s>>>(epool, vi, x, lb, ts, ts, ticket); ::h2mg::count_launch(); } break;
+    default: { k_up_tree<64, FMT, NR><<<grid, 256, 0, s>>>(epool, vi, x, lb, ts, ts, ticket); ::h2mg::count_launch(); } break;
+  }
+  H2_LAUNCH_CHECK();
 }
 
-// Downward pass from the coupling top level ts to level `lbot`, up to 4 levels per
-// launch; the last level goes to yout (when given) instead of the coefficient buffer.
+// Downward pass from the coupling top level ts to level `lbot`, up to 5 levels per
+// launch (the first launch takes the odd ones); the last level goes to yout (when given)
+// instead of the coefficient buffer, with partials of pdot^T yout. Returns the last launch's
+// CTAs. Two clusters per CTA where four would leave SMs without one.
+constexpr int DOWN_LEVELS = 5;
 template <int FMT, int NR>
-static void pass_down(const Matrix& M, const char* epool, size_t eb, const void* yrow, void* yc, int ts, int lbot,
-                      double* yout, int64_t ldo, cudaStream_t s) {
+static int pass_down(const Matrix& M, const char* epool, const void* yrow, void* yc, int ts, int lbot, double* yout,
+                     int64_t ldo, const double* pdot, double* part, cudaStream_t s) {
   using vt = typename Ar<FMT>::vec_t;
   using yt = typename Ar<FMT>::yo_t;
   const int KC = M.KC;
-  auto cslot = [&](int ell) { return (vt*)yc + (size_t)M.slot0(ell) * KC * NR; };
+  int grid = 0;
   for (int lt = ts; lt <= lbot;) {
-    const int steps = std::min(4, lbot - lt + 1);
-    PassLevels pl{};
-    for (int k = 0; k < steps; ++k) {
-      const int ell = lt + k;
-      pl.E[k] = ell > ts ? epool + (size_t)M.slot0(ell) * KC * KC * eb : nullptr;
-      pl.out[k] = cslot(ell);
-      pl.slot[k] = M.slot0(ell);
-      pl.n[k] = 1 << ell;
-    }
-    const vt* ypar = lt > ts ? cslot(lt - 1) : nullptr;
-    double* yo = (lt + steps - 1 == lbot) ? yout : nullptr;
-    const int grid = 1 << lt;
+    const int lb = lt + (lbot - lt) % DOWN_LEVELS;
+    const vt* ypar = lt > ts ? (const vt*)yc + (size_t)M.slot0(lt - 1) * KC * NR : nullptr;
+    const bool last = lb == lbot;
+    double* yo = last ? yout : nullptr;
+    const double* pd = last ? pdot : nullptr;
+    const int S = (1 << lb) >= 4 * 152 ? 4 : 2;
+    grid = std::min(std::max(1, (1 << lb) / S), CG_PARTS);
+    auto go = [&](auto kernel) {
+      kernel<<<grid, 256, 0, s>>>(epool, (const yt*)yrow, ypar, (vt*)yc, lt, lb, ts, yo, ldo, pd, part);
+      ::h2mg::count_launch();
+    };
     switch (KC) {
-      case 16: { k_down_multi<16, FMT, NR><<<grid, 256, 0, s>>>(pl, steps, (const yt*)yrow, ypar, yo, ldo); ::h2mg::count_launch(); } break;
-      case 32: { k_down_multi<32, FMT, NR><<<grid, 256, 0, s>>>(pl, steps, (const yt*)yrow, ypar, yo, ldo); ::h2mg::count_launch(); } break;
-      default: { k_down_multi<64, FMT, NR><<<grid, 256, 0, s>>>(pl, steps, (const yt*)yrow, ypar, yo, ldo); ::h2mg::count_launch(); } break;
+      case 16: S == 4 ? go(k_down_tree<16, FMT, NR, 4>) : go(k_down_tree<16, FMT, NR, 2>); break;
+      case 32: S == 4 ? go(k_down_tree<32, FMT, NR, 4>) : go(k_down_tree<32, FMT, NR, 2>); break;
+      default: S == 4 ? go(k_down_tree<64, FMT, NR, 4>) : go(k_down_tree<64, FMT, NR, 2>); break;
     }
     H2_LAUNCH_CHECK();
-    lt += steps;
+    lt = lb + 1;
   }
+  return grid;
 }
 
-// y = A_i x for NR columns (x, y column-major with leading dimensions ldx, ldy).
+// y = A_i x for NR columns (x, y column-major with leading dimensions ldx, ldy). With `cg`,
+// x is the CG direction, formed by the first kernel, and the last one leaves partials of
+// x^T y: returns their number.
 template <int FMT, class BT, int NR>
-static void apply_impl(Matrix& M, int i, const double* x, int64_t ldx, double* y, int64_t ldy, cudaStream_t s,
-                       const BT* U, const BT* UT, const ApplyWork* ws = nullptr) {
+static int apply_impl(Matrix& M, int i, const double* x, int64_t ldx, double* y, int64_t ldy, cudaStream_t s,
+                      const BT* U, const BT* UT, const ApplyWork* ws = nullptr, const CgStep* cg = nullptr) {
   using vt = typename Ar<FMT>::vec_t;
   using yt = typename Ar<FMT>::yo_t;
   const int L = M.L, KC = M.KC, KD = M.KD, ts = M.tstar;
@@ -1479,77 +1658,106 @@ static void apply_impl(Matrix& M, int i, const double* x, int64_t ldx, double* y
   yt* yr = (yt*)(ws ? ws->yr : M.wyrow.p);
   vt* yc = (vt*)(ws ? ws->yc : M.wyc.p);
   const char* epool = (const char*)(FMT == FMT_F32 ? M.poolE32.p : M.poolE.p);
-  const size_t eb = FMT == FMT_F32 ? 4 : 8;
   auto cslot = [&](int ell) { return (size_t)M.slot0(ell) * KC * NR; };   // first element of a level
+  VecIn in{};
+  in.x = x;
+  in.ldx = ldx;
+  const double* pdot = nullptr;
+  double* part = nullptr;
+  if (cg) {
+    in.r = cg->r;             // null: x is the direction already
+    in.prr = cg->prr;
+    in.np = cg->nprr;
+    in.par = cg->par;
+    in.st = cg->st;
+    pdot = x;
+    part = cg->ppq;
+  }
+  // the row sums of the levels in use: K * NR elements of 4, 8 or 16 bytes per slot
+  if (ts >= 0) {
+    in.zero[0] = (uint4*)yr;
+    in.nzero[0] = (int64_t)((1 << ((i == 1 ? L : L - i + 2) + 1)) - (1 << ts)) * KC * NR * sizeof(yt) / 16;
+  }
   if (i == 1) {
     vt* xp = (vt*)(ws ? ws->xp : M.wxp.p);
     yt* yp = (yt*)(ws ? ws->yp : M.wyp.p);
-    // padded slots must read as zero: the buffer is shared by every format and column
-    // count, so whatever an earlier product left there (possibly the halves of float64
-    // values, which as floats can be NaN) is cleared first
-    H2_CUDA(cudaMemsetAsync(xp, 0, sizeof(vt) * (size_t)(1 << L) * KD * NR, s));
-    { k_pts_in<FMT, NR><<<ceil_div(M.n, 256), 256, 0, s>>>(x, ldx, M.d_slot_of, M.n, xp); ::h2mg::count_launch(); }
+    in.zero[1] = (uint4*)yp;
+    in.nzero[1] = (int64_t)(1 << L) * KD * NR * sizeof(yt) / 16;
+    // level 1 keeps the upward pass's tickets in the downward pass's buffer, which is idle
+    // until then, so that a product in a caller's workspace uses nothing of the handle
+    unsigned* ticket = (unsigned*)yc;
+    in.zero[2] = (uint4*)ticket;
+    in.nzero[2] = ts >= 0 ? ((int64_t)M.nslots() * sizeof(unsigned) + 15) / 16 : 0;
+    const int grid = std::min(1 << L, LEAF_CTAS);
+    { k_leaf_in<FMT, BT, NR><<<grid, 256, 0, s>>>(in, ts >= 0 ? UT : nullptr, KD, KC, 1 << L, M.d_leafoff, M.d_perm, xp,
+                                                  ts >= 0 ? xc + cslot(L) : nullptr); ::h2mg::count_launch(); }
     H2_LAUNCH_CHECK();
-    if (ts >= 0) {
-      { k_up_leaf<FMT, BT, NR><<<1 << L, std::max(KC, 32), 0, s>>>(UT, KD, KC, xp, xc + cslot(L)); ::h2mg::count_launch(); }
-      H2_LAUNCH_CHECK();
-      pass_up<FMT, NR>(M, epool, eb, xc, L, ts, s);
-    }
+    if (ts >= 0) pass_up<FMT, NR>(M, epool, xc, L, ts, ticket, s);
     launch_bsgemv<FMT, NR>(M, M.opD, f32, xp, yp, s);
     if (ts >= 0) {
       launch_bsgemv<FMT, NR>(M, M.opC[1], f32, xc, yr, s);
-      pass_down<FMT, NR>(M, epool, eb, yr, yc, ts, L, nullptr, 0, s);
+      pass_down<FMT, NR>(M, epool, yr, yc, ts, L, nullptr, 0, nullptr, nullptr, s);
     }
-    { k_leaf_final<FMT, BT, NR><<<1 << L, std::max(KD, 32), 0, s>>>(
-        KD, KC, yp, ts >= 0 ? U : nullptr, ts >= 0 ? yc + cslot(L) : nullptr, M.d_leafoff, M.d_perm, y, ldy);
+    { k_leaf_final<FMT, BT, NR><<<grid, 256, 0, s>>>(KD, KC, 1 << L, yp, ts >= 0 ? U : nullptr,
+                                                     ts >= 0 ? yc + cslot(L) : nullptr, M.d_leafoff, M.d_perm, y, ldy,
+                                                     pdot, part);
       ::h2mg::count_launch(); }
     H2_LAUNCH_CHECK();
-    return;
+    return grid;
   }
   const int m = L - i + 2;
-  const int64_t nm = (int64_t)(1 << m) * KC;
-  { k_coef_in<FMT, NR><<<ceil_div(nm, 256), 256, 0, s>>>(x, ldx, nm, xc + cslot(m)); ::h2mg::count_launch(); }
-  H2_LAUNCH_CHECK();
-  pass_up<FMT, NR>(M, epool, eb, xc, m, ts, s);
+  pass_up<FMT, NR>(M, epool, xc, m, ts, M.d_ticket, s, &in);
   launch_bsgemv<FMT, NR>(M, M.opC[i], f32, xc, yr, s);
-  pass_down<FMT, NR>(M, epool, eb, yr, yc, ts, m, y, ldy, s);
+  return pass_down<FMT, NR>(M, epool, yr, yc, ts, m, y, ldy, pdot, part, s);
 }
 
 template <int FMT, class BT>
-static void apply_cols(Matrix& M, int i, const double* x, int64_t ldx, double* y, int64_t ldy, int nr,
-                       cudaStream_t s, const BT* U, const BT* UT) {
-  int c = 0;
+static int apply_cols(Matrix& M, int i, const double* x, int64_t ldx, double* y, int64_t ldy, int nr,
+                      cudaStream_t s, const BT* U, const BT* UT, const CgStep* cg) {
+  int c = 0, np = 0;
   while (c < nr) {
     int left = nr - c;
+    CgStep g{};
+    if (cg) g = cg->columns_from(c, ldx);
+    const CgStep* gp = cg ? &g : nullptr;
     if constexpr (FMT == FMT_F32) {
       if (left >= 4) {
-        apply_impl<FMT, BT, 4>(M, i, x + c * ldx, ldx, y + c * ldy, ldy, s, U, UT);
+        np = apply_impl<FMT, BT, 4>(M, i, x + c * ldx, ldx, y + c * ldy, ldy, s, U, UT, nullptr, gp);
         c += 4;
         continue;
       }
     }
     if (left >= 2) {
-      apply_impl<FMT, BT, 2>(M, i, x + c * ldx, ldx, y + c * ldy, ldy, s, U, UT);
+      np = apply_impl<FMT, BT, 2>(M, i, x + c * ldx, ldx, y + c * ldy, ldy, s, U, UT, nullptr, gp);
       c += 2;
     } else {
-      apply_impl<FMT, BT, 1>(M, i, x + c * ldx, ldx, y + c * ldy, ldy, s, U, UT);
+      np = apply_impl<FMT, BT, 1>(M, i, x + c * ldx, ldx, y + c * ldy, ldy, s, U, UT, nullptr, gp);
       c += 1;
     }
   }
+  return np;
+}
+
+static int apply_any(Matrix& M, int i, bool f32, const double* x, int64_t ldx, double* y, int64_t ldy, int nr,
+                     cudaStream_t s, const CgStep* cg) {
+  if (f32) {
+    H2_REQUIRE(M.with_f32, H2MG_ERR_INVALID_ARG, "matrix was built without an FP32 copy");
+    return apply_cols<FMT_F32, float>(M, i, x, ldx, y, ldy, nr, s, M.d_U32, M.d_UT32, cg);
+  }
+  if (M.fmt == FMT_DF) return apply_cols<FMT_DF, double>(M, i, x, ldx, y, ldy, nr, s, M.d_U, M.d_UT, cg);
+  return apply_cols<FMT_F64, double>(M, i, x, ldx, y, ldy, nr, s, M.d_U, M.d_UT, cg);
 }
 
 // Y = A_i X for nr columns; columns go through the block products NR at a time
 // (4 for the FP32 copy, 2 for float64 / double-float), each block read once per group.
 void apply_level_multi(Matrix& M, int i, bool f32, const double* x, int64_t ldx, double* y, int64_t ldy, int nr,
                        cudaStream_t s) {
-  if (f32) {
-    H2_REQUIRE(M.with_f32, H2MG_ERR_INVALID_ARG, "matrix was built without an FP32 copy");
-    apply_cols<FMT_F32, float>(M, i, x, ldx, y, ldy, nr, s, M.d_U32, M.d_UT32);
-  } else if (M.fmt == FMT_DF) {
-    apply_cols<FMT_DF, double>(M, i, x, ldx, y, ldy, nr, s, M.d_U, M.d_UT);
-  } else {
-    apply_cols<FMT_F64, double>(M, i, x, ldx, y, ldy, nr, s, M.d_U, M.d_UT);
-  }
+  apply_any(M, i, f32, x, ldx, y, ldy, nr, s, nullptr);
+}
+
+int apply_cg_step(Matrix& M, int i, bool f32, double* p, double* q, int64_t ld, int nr, const CgStep& cg,
+                  cudaStream_t s) {
+  return apply_any(M, i, f32, p, ld, q, ld, nr, s, &cg);
 }
 
 void apply_level(Matrix& M, int i, bool f32, const double* x, double* y, cudaStream_t s) {
@@ -1589,6 +1797,7 @@ static float time_product(Matrix& M, SymOp& op, bool pts, int split, int reps, c
   const bool f32 = FMT == FMT_F32;
   void* x = pts ? M.wxp.p : M.wx.p;
   void* y = pts ? M.wyp.p : M.wyrow.p;
+  H2_CUDA(cudaMemsetAsync(y, 0, sizeof(typename Ar<FMT>::yo_t) * (size_t)op.nrows * op.K * NR, s));
   launch_bsgemv<FMT, NR>(M, op, f32, x, y, s, split);   // warm-up
   H2_CUDA(cudaEventRecord(e0, s));
   for (int r = 0; r < reps; ++r) launch_bsgemv<FMT, NR>(M, op, f32, x, y, s, split);

@@ -152,6 +152,7 @@ struct Matrix {
   DevBuf wcoarse;               // three vectors of the coarse size (triangular solves)
   DevBuf wfcg;                  // five point vectors of the flexible-CG outer loop
   int* d_flag = nullptr;        // device error flags
+  unsigned* d_ticket = nullptr; // upward pass: arrivals per pair of clusters (slots), zero between launches
 
   Profile prof;
   GraphSet* graphs = nullptr;   // captured V-cycle graphs, by solve settings
@@ -178,6 +179,29 @@ void build_dense_coarse(Matrix& M);
 void coarse_solve(Matrix& M, const double* r, double* e, cudaStream_t s);
 void coarse_solve_multi(Matrix& M, const double* r, double* e, int nr, cudaStream_t s);
 // ---- apply.cu
+// State of one column of a smoother's CG, in device memory.
+struct CGState {
+  double rho[2];   // r^T r, double-buffered by iteration parity
+  double thresh;
+  int stopped;
+};
+constexpr int CG_PARTS = 2048;    // partials of one dot product of a column, at most
+// One CG step's product q = A_i p with what surrounds it: r (null in the first step: p is the
+// direction already) with the partials of r^T r gives the direction p = r + beta p before the
+// product, and ppq receives partials of p^T q. Arrays of nr columns (partials: CG_PARTS each).
+struct CgStep {
+  const double* r;
+  const double* prr;
+  int nprr, par;
+  CGState* st;
+  double* ppq;
+  CgStep columns_from(int c, int64_t ld) const {
+    return {r ? r + c * ld : nullptr, prr + (int64_t)c * CG_PARTS, nprr, par, st + c, ppq + (int64_t)c * CG_PARTS};
+  }
+};
+// Returns the number of partials in ppq per column.
+int apply_cg_step(Matrix& M, int i, bool f32, double* p, double* q, int64_t ld, int nr, const CgStep& cg,
+                  cudaStream_t s);
 struct ApplyWork {                // workspace of one product (see apply_impl)
   void *xc, *yr, *yc, *xp, *yp;
 };

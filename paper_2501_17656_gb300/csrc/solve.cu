@@ -14,12 +14,7 @@
 namespace h2mg {
 
 // ----------------------------------------------------------------------------- reductions
-constexpr int NPART = 256;
-struct CGState {
-  double rho[2];   // r^T r, double-buffered by iteration parity
-  double thresh;
-  int stopped;
-};
+constexpr int NPART = 256;       // partials of the outer loops' dot products
 
 __device__ double block_reduce_sum(double v) {
   __shared__ double sh[32];
@@ -46,30 +41,13 @@ __global__ void k_dot_part(const double* __restrict__ a, const double* __restric
   if (threadIdx.x == 0) part[blockIdx.y * NPART + blockIdx.x] = s;
 }
 
-__device__ double sum_parts(const double* part, int np) {
-  double s = 0.0;
-  for (int i = 0; i < np; ++i) s += part[i];
-  return s;
-}
-
 static int part_grid(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>(NPART, (n + 1023) / 1024)); }
 
-// per column (thread c): rho = r.r, thresh = (1e-30 |f|)^2
-__global__ void k_cg_init(const double* __restrict__ prr, const double* __restrict__ pff, int np, int nr,
-                          CGState* st) {
-  const int c = threadIdx.x;
-  if (c >= nr) return;
-  double rr = sum_parts(prr + c * NPART, np), ff = sum_parts(pff + c * NPART, np);
-  double t = 1e-30 * sqrt(ff);
-  st[c].rho[0] = rr;
-  st[c].thresh = t * t;
-  st[c].stopped = 0;
-}
-
-// Sum of np (<= 256) partials, by every CTA (blockDim 256).
+// Sum of np partials, by every CTA (blockDim 256).
 __device__ double cta_sum_parts(const double* __restrict__ part, int np) {
   __shared__ double sh[8];
-  double v = threadIdx.x < np ? part[threadIdx.x] : 0.0;
+  double v = 0.0;
+  for (int i = threadIdx.x; i < np; i += 256) v += part[i];
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
   __syncthreads();
@@ -79,57 +57,88 @@ __device__ double cta_sum_parts(const double* __restrict__ part, int np) {
   return s;
 }
 
+// Start of a CG: r = f - q (q null: r = f, and x = 0), p = r, partials of r^T r and f^T f.
+__global__ void __launch_bounds__(256) k_cg_start(const double* __restrict__ f, const double* __restrict__ q,
+                                                  int64_t n, double* __restrict__ x, double* __restrict__ r,
+                                                  double* __restrict__ p, double* __restrict__ prr,
+                                                  double* __restrict__ pff) {
+  const int64_t c = blockIdx.y * n;
+  double rr = 0.0, ff = 0.0;
+  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+    const double fi = f[c + i], ri = q ? fi - q[c + i] : fi;
+    if (!q) x[c + i] = 0.0;
+    r[c + i] = ri;
+    p[c + i] = ri;
+    rr = fma(ri, ri, rr);
+    ff = fma(fi, fi, ff);
+  }
+  rr = block_reduce_sum(rr);
+  ff = block_reduce_sum(ff);
+  if (threadIdx.x == 0) {
+    prr[blockIdx.y * CG_PARTS + blockIdx.x] = rr;
+    pff[blockIdx.y * CG_PARTS + blockIdx.x] = ff;
+  }
+}
+
+// per column (CTA c): rho = r.r, thresh = (1e-30 |f|)^2
+__global__ void __launch_bounds__(256) k_cg_init(const double* __restrict__ prr, const double* __restrict__ pff,
+                                                 int np, CGState* st) {
+  const int c = blockIdx.x;
+  const double rr = cta_sum_parts(prr + c * CG_PARTS, np), ff = cta_sum_parts(pff + c * CG_PARTS, np);
+  if (threadIdx.x == 0) {
+    const double t = 1e-30 * sqrt(ff);
+    st[c].rho[0] = rr;
+    st[c].thresh = t * t;
+    st[c].stopped = 0;
+  }
+}
+
 // alpha = rho / p^T q (stop before the update if p^T q <= 0); x += alpha p;
 // r -= alpha q; partials of r^T r. Every CTA of a column (blockIdx.y) takes the same
-// decision from the same partials.
+// decision from the same partials. The new direction p = r + (rho' / rho) p is formed by the
+// next step's product (VecIn in apply.cu).
 __global__ void __launch_bounds__(256) k_cg_update(double* __restrict__ x, double* __restrict__ r,
                                                    const double* __restrict__ p, const double* __restrict__ q,
-                                                   int64_t n, int64_t ld, CGState* st,
-                                                   const double* __restrict__ ppq, int np, int par,
-                                                   double* __restrict__ part) {
+                                                   int64_t n, CGState* st, const double* __restrict__ ppq, int np,
+                                                   int par, double* __restrict__ part) {
   const int c = blockIdx.y;
-  x += c * ld;
-  r += c * ld;
-  p += c * ld;
-  q += c * ld;
-  const double pq = cta_sum_parts(ppq + c * NPART, np);
-  bool go = !st[c].stopped;
-  if (go && !(pq > 0.0)) {
-    go = false;
-    if (blockIdx.x == 0 && threadIdx.x == 0) st[c].stopped = 1;
+  x += c * n;
+  r += c * n;
+  p += c * n;
+  q += c * n;
+  // the first element's loads are under way while the partials are summed
+  int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  double ri = 0.0, pi = 0.0, qi = 0.0, xi = 0.0;
+  if (i < n) {
+    ri = r[i];
+    pi = p[i];
+    qi = q[i];
+    xi = x[i];
   }
-  const double al = go ? st[c].rho[par] / pq : 0.0;
+  const int stopped = st[c].stopped;
+  const double rho = st[c].rho[par];
+  const double pq = cta_sum_parts(ppq + c * CG_PARTS, np);
+  const bool go = !stopped && pq > 0.0;
+  if (!stopped && !go && blockIdx.x == 0 && threadIdx.x == 0) st[c].stopped = 1;
+  const double al = go ? rho / pq : 0.0;
   double s = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    double ri = r[i];
+  while (i < n) {
     if (go) {
-      x[i] = fma(al, p[i], x[i]);
-      ri = fma(-al, q[i], ri);
+      x[i] = fma(al, pi, xi);
+      ri = fma(-al, qi, ri);
       r[i] = ri;
     }
     s = fma(ri, ri, s);
+    i += (int64_t)gridDim.x * 256;
+    if (i < n) {
+      ri = r[i];
+      pi = p[i];
+      qi = q[i];
+      xi = x[i];
+    }
   }
   s = block_reduce_sum(s);
-  if (threadIdx.x == 0) part[c * NPART + blockIdx.x] = s;
-}
-
-// rho' = r^T r; stop (after the update) if rho' <= thresh; else p = r + (rho'/rho) p.
-__global__ void __launch_bounds__(256) k_cg_p(double* __restrict__ p, const double* __restrict__ r, int64_t n,
-                                              int64_t ld, CGState* st, const double* __restrict__ prr, int np,
-                                              int par) {
-  const int c = blockIdx.y;
-  p += c * ld;
-  r += c * ld;
-  const double rn = cta_sum_parts(prr + c * NPART, np);
-  if (st[c].stopped) return;
-  if (rn <= st[c].thresh) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) st[c].stopped = 1;
-    return;
-  }
-  const double be = rn / st[c].rho[par];
-  if (blockIdx.x == 0 && threadIdx.x == 0) st[c].rho[par ^ 1] = rn;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    p[i] = fma(be, p[i], r[i]);
+  if (threadIdx.x == 0) part[c * CG_PARTS + blockIdx.x] = s;
 }
 
 // y_c += a[c] x_c for every column c = blockIdx.y (a in device memory)
@@ -263,7 +272,7 @@ static Work work(Matrix& M) {
   if (!M.wvec.p) {
     M.wvec.bytes = sizeof(double) * tot * NRMAX;
     M.wvec.p = M.alloc(M.wvec.bytes);
-    M.wred.bytes = sizeof(double) * (2 * NPART + 8) * NRMAX + sizeof(CGState) * NRMAX + 64;
+    M.wred.bytes = sizeof(double) * (2 * CG_PARTS + 8) * NRMAX + sizeof(CGState) * NRMAX + 64;
     M.wred.p = M.alloc(M.wred.bytes);
     M.wfcg.bytes = sizeof(double) * 4 * (size_t)M.n * NRMAX;   // flexible-CG directions
     M.wfcg.p = M.alloc(M.wfcg.bytes);
@@ -281,8 +290,8 @@ static Work work(Matrix& M) {
   W.t1 = p; p += nmax * NRMAX;
   W.t2 = p; p += nmax * NRMAX;
   W.pa = (double*)M.wred.p;
-  W.pb = W.pa + NPART * NRMAX;
-  W.scal = W.pb + NPART * NRMAX;
+  W.pb = W.pa + CG_PARTS * NRMAX;
+  W.scal = W.pb + CG_PARTS * NRMAX;
   W.st = (CGState*)(W.scal + 8 * NRMAX);
   return W;
 }
@@ -296,6 +305,12 @@ static void dot_part(const double* a, const double* b, int64_t n, int64_t ld, in
   H2_LAUNCH_CHECK();
 }
 
+// Four launches per step (on level 1, two more for the leaves and one for the close blocks):
+// the product's first kernel forms the direction and its last one the partials of p^T q.
+// Nine or ten launches, with vectors converted, cleared and reduced in kernels of their own,
+// took 196 us per step on level 2 of 30011 points in the cube (FP32; the blocks alone 128)
+// and 87 us on the 1024 unknowns of level 2 of 4096 points (F64); now 165 and 29.
+//
 // n CG iterations on A_i X = F from X0 (nullptr: zero) for nr columns of length N_i.
 // X receives the iterates; R (if not null) the recurrence residuals. Hestenes-Stiefel
 // with, per column, the breakdown guard p^T A p <= 0 and the stop r^T r <= (1e-30 |f|)^2.
@@ -305,33 +320,28 @@ void smooth_multi(Matrix& M, int i, bool f32, const double* f, const double* x0,
   Work W = work(M);
   const int64_t N = level_size(M, i), tot = N * nr;
   double* rr = r ? r : W.cr;
-  const int g = vec_grid(N), np = part_grid(N);
   if (n == 0 && x0 != nullptr && r == nullptr) {   // no iteration, residual not wanted
     if (x != x0) H2_CUDA(cudaMemcpyAsync(x, x0, sizeof(double) * tot, cudaMemcpyDeviceToDevice, s));
     return;
   }
-  if (x0 == nullptr) {
-    H2_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * tot, s));
-    H2_CUDA(cudaMemcpyAsync(rr, f, sizeof(double) * tot, cudaMemcpyDeviceToDevice, s));
-    if (n == 0) return;
-  } else {
+  const double* q0 = nullptr;
+  if (x0 != nullptr) {
     if (x != x0) H2_CUDA(cudaMemcpyAsync(x, x0, sizeof(double) * tot, cudaMemcpyDeviceToDevice, s));
     apply_level_multi(M, i, f32, x, N, W.cq, N, nr, s);
-    { k_sub<<<vec_grid(tot), 256, 0, s>>>(f, W.cq, rr, tot); ::h2mg::count_launch(); }
-    H2_LAUNCH_CHECK();
+    q0 = W.cq;
   }
-  H2_CUDA(cudaMemcpyAsync(W.cp, rr, sizeof(double) * tot, cudaMemcpyDeviceToDevice, s));
-  dot_part(rr, rr, N, N, nr, W.pa, s);
-  dot_part(f, f, N, N, nr, W.pb, s);
-  { k_cg_init<<<1, 32, 0, s>>>(W.pa, W.pb, np, nr, W.st); ::h2mg::count_launch(); }
+  // one element per thread where the vector is short: the steps are latency, not bandwidth
+  const int g = (int)std::max<int64_t>(1, std::min<int64_t>(2 * 152, (N + 255) / 256));
+  { k_cg_start<<<dim3(g, nr), 256, 0, s>>>(f, q0, N, x, rr, W.cp, W.pb, W.pa); ::h2mg::count_launch(); }
+  H2_LAUNCH_CHECK();
+  if (n == 0) return;
+  { k_cg_init<<<nr, 256, 0, s>>>(W.pb, W.pa, g, W.st); ::h2mg::count_launch(); }
   H2_LAUNCH_CHECK();
   for (int it = 0; it < n; ++it) {
-    const int par = it & 1;
-    apply_level_multi(M, i, f32, W.cp, N, W.cq, N, nr, s);
-    dot_part(W.cp, W.cq, N, N, nr, W.pa, s);
-    { k_cg_update<<<dim3(np, nr), 256, 0, s>>>(x, rr, W.cp, W.cq, N, N, W.st, W.pa, np, par, W.pb); ::h2mg::count_launch(); }
-    H2_LAUNCH_CHECK();
-    { k_cg_p<<<dim3(g, nr), 256, 0, s>>>(W.cp, rr, N, N, W.st, W.pb, np, par); ::h2mg::count_launch(); }
+    // the direction of step `it` comes from step it - 1's residual: rho' and rho there
+    const CgStep cg{it > 0 ? rr : nullptr, W.pb, g, (it - 1) & 1, W.st, W.pa};
+    const int np = apply_cg_step(M, i, f32, W.cp, W.cq, N, nr, cg, s);
+    { k_cg_update<<<dim3(g, nr), 256, 0, s>>>(x, rr, W.cp, W.cq, N, W.st, W.pa, np, it & 1, W.pb); ::h2mg::count_launch(); }
     H2_LAUNCH_CHECK();
   }
 }
