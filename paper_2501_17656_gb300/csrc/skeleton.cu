@@ -18,9 +18,11 @@
 //     of sigma''s two children concatenated and thinned to every s-th entry from the
 //     first, s = ceil(count / 128);
 //  2. R0 = the R factor of W = A(F_tau, candidates): the sampled rows are generated
-//     in chunks of 32 and folded into an upper-triangular R in shared memory by
+//     in chunks of 128 and folded into an upper-triangular R in shared memory by
 //     Householder reflections that touch only row j of R and the chunk (a
-//     tall-skinny QR; W itself is never stored);
+//     tall-skinny QR; W itself is never stored). Where a level has fewer clusters than
+//     the GPU has room for, several CTAs fold parts of a cluster's rows and their R
+//     factors are folded together;
 //  3. greedy column-pivoted Householder QR of R0 (the column of largest remaining
 //     norm; columns within a relative 1e-10 of the largest squared norm are tied and
 //     the lowest index wins), stopped at rank_max, at min(rows, candidates), or once
@@ -36,24 +38,19 @@
 namespace h2mg {
 
 constexpr int SK_CAND = 128;        // candidates of a cluster at most (two skeletons of <= 64)
-constexpr int SK_CHUNK = 32;        // sampled rows folded into R at a time (one per lane)
+constexpr int SK_CHUNK = 128;       // sampled rows folded into R at a time
+constexpr int SK_OWN = 32;          // of which a thread holds a quarter, for one column, in registers
 constexpr int SK_SAMPLE_CAP = 128;  // points kept per far partner of the parent
 constexpr double SK_TIE = 1e-10;    // relative tie band of the pivot choice
 
-// Sum over the 32 lanes of a warp.
-__device__ __forceinline__ double warp_sum(double v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Block-wide max / min helpers (blockDim.x == 256); red has >= 8 entries.
+// Block-wide max / min helpers; red has one entry per warp.
 __device__ double block_max(double v, double* red) {
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
   __syncthreads();
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
   double m = red[0];
-  for (int i = 1; i < 8; ++i) m = fmax(m, red[i]);
+  for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = fmax(m, red[i]);
   __syncthreads();
   return m;
 }
@@ -63,90 +60,192 @@ __device__ int block_min_int(int v, int* red) {
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
   int m = red[0];
-  for (int i = 1; i < 8; ++i) m = min(m, red[i]);
+  for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = min(m, red[i]);
   __syncthreads();
   return m;
 }
 
-// One CTA (256 threads) per cluster of the level.
+// Shared memory of k_skeletonize<NC> (NC candidates at most, 4 NC threads). R is
+// column-major with ld NC + 1: rows and columns are both read without bank conflicts.
+template <int NC>
+struct SkelSmem {
+  double R[NC * (NC + 1)];
+  double stage[SK_CHUNK / 4 * NC];   // kernel values on their way into the owning thread's registers
+  double v[2][SK_CHUNK];             // column j of the chunk (double-buffered over j)
+  double part[4][NC];                // partial dot products of the row quarters
+  double sig[4];
+  double sc[3];                      // beta, tau, scale of the reflector
+  double nrm[NC];
+  double red[16];
+  double bcast[3];
+  int piv[NC];
+  int ired[16];
+};
+
+// Folds a chunk of 128 rows into R: thread (k, q) holds c[SK_OWN], quarter q of the rows, of
+// column k. Reflector j: v = (1, column j of the chunk / (alpha - beta)), alpha = R_jj. Warps
+// are numbered so that every scheduler holds one quarter of each group of 32 columns: their
+// load stays even as the leading columns finish. Bound by the float64 pipe: 2 FMAs per row
+// and pair of columns, the minimum of Householder's method, in 70 operations of which 64 are
+// those FMAs (a warp per column with 32 rows took 8 operations for 2, most of them in
+// warp-wide sums). Whole builds: 8192 points 296 -> 99 ms, 16384 points 660 -> 225 ms.
+template <int NC>
+__device__ __forceinline__ void fold_chunk(SkelSmem<NC>& sm, int nc, int k, int q, double (&c)[SK_OWN]) {
+  auto publish = [&](int j) {          // column j's threads hand out the column and its partial norm
+    if (k == j) {
+      double s = 0.0;
+#pragma unroll
+      for (int i = 0; i < SK_OWN; ++i) {
+        sm.v[j & 1][q * SK_OWN + i] = c[i];
+        s = fma(c[i], c[i], s);
+      }
+      sm.sig[q] = s;
+    }
+  };
+  publish(0);
+  __syncthreads();
+  for (int j = 0; j < nc; ++j) {
+    const double2* v = reinterpret_cast<const double2*>(sm.v[j & 1] + q * SK_OWN);
+    const bool active = k > j && k < nc;
+    if (threadIdx.x == 0) {
+      const double sigma = (sm.sig[0] + sm.sig[1]) + (sm.sig[2] + sm.sig[3]);
+      const double alpha = sm.R[j + j * (NC + 1)];
+      double beta = alpha, tau = 0.0, scale = 0.0;
+      if (sigma > 0.0) {
+        beta = -copysign(sqrt(fma(alpha, alpha, sigma)), alpha);
+        tau = (beta - alpha) / beta;
+        scale = 1.0 / (alpha - beta);
+      }
+      sm.sc[0] = beta;
+      sm.sc[1] = tau;
+      sm.sc[2] = scale;
+    }
+    if (active) {
+      double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+      for (int i = 0; i < SK_OWN / 2; ++i) {
+        const double2 x = v[i];
+        s0 = fma(c[2 * i], x.x, s0);
+        s1 = fma(c[2 * i + 1], x.y, s1);
+      }
+      sm.part[q][k] = s0 + s1;
+    }
+    __syncthreads();
+    const double tau = sm.sc[1], scale = sm.sc[2];
+    if (tau != 0.0 && active) {
+      const double d = (sm.part[0][k] + sm.part[1][k]) + (sm.part[2][k] + sm.part[3][k]);
+      double* r = sm.R + j + k * (NC + 1);
+      const double wk = tau * fma(scale, d, *r), f = -wk * scale;
+#pragma unroll
+      for (int i = 0; i < SK_OWN / 2; ++i) {
+        const double2 x = v[i];
+        c[2 * i] = fma(f, x.x, c[2 * i]);
+        c[2 * i + 1] = fma(f, x.y, c[2 * i + 1]);
+      }
+      if (q == 0) sm.nrm[k] = wk;              // R_jk is read by the other quarters: changed after the barrier
+    }
+    publish(j + 1);
+    __syncthreads();
+    if (tau != 0.0) {
+      if (active && q == 0) sm.R[j + k * (NC + 1)] -= sm.nrm[k];
+      if (threadIdx.x == 0) sm.R[j + j * (NC + 1)] = sm.sc[0];
+    }
+  }
+  __syncthreads();
+}
+
+// `parts` CTAs of 4 NC threads per cluster of the level.
 //   cand   [ncl][SK_CAND]: candidate tree positions, ncand[ncl] of them
 //   samp   sampled tree positions of all clusters, cluster c at samp[soff[c] .. soff[c+1])
 //   out:   skel[ncl][64] (tree positions, pivot order), rank[ncl], T[ncl][SK_CAND x 64]
 //          (rows = candidates in their original order, column-major, ld SK_CAND)
-__global__ void __launch_bounds__(256, 1) k_skeletonize(const int* __restrict__ cand, const int* __restrict__ ncand,
-                                                       const int* __restrict__ samp, const int64_t* __restrict__ soff,
-                                                       const double* __restrict__ X, const double* __restrict__ sw,
-                                                       int dim, KernelParams kp, double tol, int rank_max,
-                                                       int* __restrict__ skel, int* __restrict__ rank_out,
-                                                       double* __restrict__ Tout) {
-  extern __shared__ double sm[];
-  double* R = sm;                                  // SK_CAND x SK_CAND, column-major, ld SK_CAND
-  double* C = R + SK_CAND * SK_CAND;               // SK_CHUNK x SK_CAND, column-major, ld SK_CHUNK
-  double* cx = C + SK_CHUNK * SK_CAND;             // candidate coordinates [SK_CAND][3]
-  double* cw = cx + SK_CAND * 3;                   // candidate sqrt(w)
-  double* nrm = cw + SK_CAND;                      // column norms (pivoting)
-  double* red = nrm + SK_CAND;                     // 8 reduction slots
-  double* bcast = red + 8;                         // 4 broadcast slots
-  int* piv = (int*)(bcast + 4);                    // SK_CAND
-  int* ired = piv + SK_CAND;                       // 8
-  const int c = blockIdx.x;
+// With parts > 1 a first launch (finish = 0) leaves the R factor of each part of the rows in
+// Rpart, and a second one, one CTA per cluster (finish = 1), folds them and goes on.
+template <int NC>
+__global__ void __launch_bounds__(4 * NC) k_skeletonize(const int* __restrict__ cand, const int* __restrict__ ncand,
+                                                        const int* __restrict__ samp, const int64_t* __restrict__ soff,
+                                                        const double* __restrict__ X, const double* __restrict__ sw,
+                                                        int dim, KernelParams kp, double tol, int rank_max, int parts,
+                                                        int finish, double* __restrict__ Rpart, int* __restrict__ skel,
+                                                        int* __restrict__ rank_out, double* __restrict__ Tout) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  SkelSmem<NC>& sm = *reinterpret_cast<SkelSmem<NC>*>(dsm);
+  constexpr int LD = NC + 1;
+  double* R = sm.R;
+  double* nrm = sm.nrm;
+  double* red = sm.red;
+  double* bcast = sm.bcast;
+  int* piv = sm.piv;
+  int* ired = sm.ired;
+  const int c = finish ? blockIdx.x : blockIdx.x / parts, part = finish ? 0 : blockIdx.x % parts;
   const int nc = ncand[c];
   const int* cd = cand + (int64_t)c * SK_CAND;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int k = 32 * (w >> 2) + lane, q = w & 3;     // column and row quarter of this thread
   const int64_t s0 = soff[c], s1 = soff[c + 1];
   const int64_t m = s1 - s0;
-  for (int i = threadIdx.x; i < nc; i += blockDim.x) {
-    const int p = cd[i];
-    for (int d = 0; d < dim; ++d) cx[i * 3 + d] = X[(int64_t)p * dim + d];
-    cw[i] = sw[p];
-    piv[i] = i;
-  }
-  for (int i = threadIdx.x; i < SK_CAND * SK_CAND; i += blockDim.x) R[i] = 0.0;
+  for (int i = threadIdx.x; i < nc; i += blockDim.x) piv[i] = i;
+  for (int i = threadIdx.x; i < NC * LD; i += blockDim.x) R[i] = 0.0;
   __syncthreads();
   int r = 0;
   if (m > 0 && nc > 0) {
-    // ---- 2. tall-skinny QR of the sampled rows, SK_CHUNK rows at a time
-    for (int64_t q0 = 0; q0 < m; q0 += SK_CHUNK) {
-      for (int e = threadIdx.x; e < SK_CHUNK * nc; e += blockDim.x) {
-        const int i = e % SK_CHUNK, k = e / SK_CHUNK;
-        double v = 0.0;
-        if (q0 + i < m) {
-          const int f = samp[s0 + q0 + i];
-          v = sw[f] * kernel_eval(kp, X + (int64_t)f * dim, cx + k * 3, dim) * cw[k];
+    // ---- 2. tall-skinny QR of the sampled rows
+    double cc[SK_OWN];
+    if (finish) {
+      const double* P = Rpart + (int64_t)c * parts * NC * NC;
+      for (int p = 0; p < parts; ++p) {
+#pragma unroll
+        for (int i = 0; i < SK_OWN; ++i) {
+          const int row = q * SK_OWN + i;
+          cc[i] = k < nc && row < NC ? P[((int64_t)p * NC + k) * NC + row] : 0.0;
         }
-        C[i + k * SK_CHUNK] = v;
+        fold_chunk<NC>(sm, nc, k, q, cc);
       }
-      __syncthreads();
-      for (int j = 0; j < nc; ++j) {
-        const double cij = C[lane + j * SK_CHUNK];
-        const double sigma = warp_sum(cij * cij);
-        const double alpha = R[j + j * SK_CAND];
-        if (sigma > 0.0) {
-          const double beta = -copysign(sqrt(alpha * alpha + sigma), alpha);
-          const double tau = (beta - alpha) / beta;
-          const double vi = cij / (alpha - beta);
-          for (int k = j + 1 + w; k < nc; k += 8) {
-            const double ck = C[lane + k * SK_CHUNK];
-            const double wk = tau * (R[j + k * SK_CAND] + warp_sum(vi * ck));
-            if (lane == 0) R[j + k * SK_CAND] -= wk;
-            C[lane + k * SK_CHUNK] = ck - wk * vi;
+    } else {
+      double x[3] = {0.0, 0.0, 0.0}, wk = 0.0;
+      if (k < nc) {
+        const int p = cd[k];
+        for (int d = 0; d < dim; ++d) x[d] = X[(int64_t)p * dim + d];
+        wk = sw[p];
+      }
+      const int64_t chunks = (m + SK_CHUNK - 1) / SK_CHUNK;
+      const int64_t ch1 = chunks * (part + 1) / parts;
+      for (int64_t ch = chunks * part / parts; ch < ch1; ++ch) {
+        const int64_t row0 = ch * SK_CHUNK + q * SK_OWN;
+#pragma unroll
+        for (int g = 0; g < SK_OWN / 8; ++g) {
+#pragma unroll 1
+          for (int i = 0; i < 8; ++i) {
+            const int64_t row = row0 + 8 * g + i;
+            double v = 0.0;
+            if (k < nc && row < m) {
+              const int f = samp[s0 + row];
+              v = sw[f] * kernel_eval(kp, X + (int64_t)f * dim, x, dim) * wk;
+            }
+            sm.stage[(q * 8 + i) * NC + k] = v;      // read back by this thread alone
           }
-          __syncthreads();
-          if (threadIdx.x == 0) R[j + j * SK_CAND] = beta;
-        } else {
-          __syncthreads();
+#pragma unroll
+          for (int i = 0; i < 8; ++i) cc[8 * g + i] = sm.stage[(q * 8 + i) * NC + k];
         }
+        fold_chunk<NC>(sm, nc, k, q, cc);
       }
-      __syncthreads();
+    }
+    if (!finish && parts > 1) {
+      double* P = Rpart + ((int64_t)c * parts + part) * NC * NC;
+      for (int e = threadIdx.x; e < NC * NC; e += blockDim.x) {
+        const int i = e % NC, kk = e / NC;
+        P[e] = i <= kk ? R[i + kk * LD] : 0.0;
+      }
+      return;
     }
     // ---- 3. greedy column-pivoted Householder QR of R0 (rows: min(m, nc))
-    const int rows = (int)std::min<int64_t>(m, nc);
+    const int rows = (int)(m < nc ? m : nc);
     const int kmax = min(rank_max, min(rows, nc));
     double first = 0.0;
     for (int j = 0; j < kmax; ++j) {
       for (int k = j + threadIdx.x; k < nc; k += blockDim.x) {
         double s = 0.0;
-        for (int i = j; i < nc; ++i) s = fma(R[i + k * SK_CAND], R[i + k * SK_CAND], s);
+        for (int i = j; i < nc; ++i) s = fma(R[i + k * LD], R[i + k * LD], s);
         nrm[k] = s;
       }
       __syncthreads();
@@ -165,9 +264,9 @@ __global__ void __launch_bounds__(256, 1) k_skeletonize(const int* __restrict__ 
       const int p = block_min_int(cand_k, ired);
       if (p != j) {
         for (int i = threadIdx.x; i < nc; i += blockDim.x) {
-          const double t = R[i + j * SK_CAND];
-          R[i + j * SK_CAND] = R[i + p * SK_CAND];
-          R[i + p * SK_CAND] = t;
+          const double t = R[i + j * LD];
+          R[i + j * LD] = R[i + p * LD];
+          R[i + p * LD] = t;
         }
         if (threadIdx.x == 0) {
           const int t = piv[j];
@@ -177,35 +276,38 @@ __global__ void __launch_bounds__(256, 1) k_skeletonize(const int* __restrict__ 
         __syncthreads();
       }
       // reflector of R[j:, j]
-      if (threadIdx.x == 0) {
-        const double alpha = R[j + j * SK_CAND];
+      if (threadIdx.x < 32) {
+        const double alpha = R[j + j * LD];
         double sigma = 0.0;
-        for (int i = j + 1; i < nc; ++i) sigma = fma(R[i + j * SK_CAND], R[i + j * SK_CAND], sigma);
+        for (int i = j + 1 + lane; i < nc; i += 32) sigma = fma(R[i + j * LD], R[i + j * LD], sigma);
+        for (int o = 16; o > 0; o >>= 1) sigma += __shfl_xor_sync(0xffffffffu, sigma, o);
         double beta = alpha, tau = 0.0, scale = 0.0;
         if (sigma > 0.0) {
           beta = -copysign(sqrt(alpha * alpha + sigma), alpha);
           tau = (beta - alpha) / beta;
           scale = 1.0 / (alpha - beta);
         }
-        bcast[0] = beta;
-        bcast[1] = tau;
-        bcast[2] = scale;
+        if (lane == 0) {
+          bcast[0] = beta;
+          bcast[1] = tau;
+          bcast[2] = scale;
+        }
       }
       __syncthreads();
       const double beta = bcast[0], tau = bcast[1], scale = bcast[2];
       if (tau != 0.0) {
-        for (int i = j + 1 + threadIdx.x; i < nc; i += blockDim.x) R[i + j * SK_CAND] *= scale;
+        for (int i = j + 1 + threadIdx.x; i < nc; i += blockDim.x) R[i + j * LD] *= scale;
         __syncthreads();
         for (int k = j + 1 + threadIdx.x; k < nc; k += blockDim.x) {
-          double wk = R[j + k * SK_CAND];
-          for (int i = j + 1; i < nc; ++i) wk = fma(R[i + j * SK_CAND], R[i + k * SK_CAND], wk);
+          double wk = R[j + k * LD];
+          for (int i = j + 1; i < nc; ++i) wk = fma(R[i + j * LD], R[i + k * LD], wk);
           wk *= tau;
-          R[j + k * SK_CAND] -= wk;
-          for (int i = j + 1; i < nc; ++i) R[i + k * SK_CAND] = fma(-wk, R[i + j * SK_CAND], R[i + k * SK_CAND]);
+          R[j + k * LD] -= wk;
+          for (int i = j + 1; i < nc; ++i) R[i + k * LD] = fma(-wk, R[i + j * LD], R[i + k * LD]);
         }
         __syncthreads();
-        if (threadIdx.x == 0) R[j + j * SK_CAND] = beta;
-        for (int i = j + 1 + threadIdx.x; i < nc; i += blockDim.x) R[i + j * SK_CAND] = 0.0;
+        if (threadIdx.x == 0) R[j + j * LD] = beta;
+        for (int i = j + 1 + threadIdx.x; i < nc; i += blockDim.x) R[i + j * LD] = 0.0;
       }
       __syncthreads();
       r = j + 1;
@@ -215,14 +317,14 @@ __global__ void __launch_bounds__(256, 1) k_skeletonize(const int* __restrict__ 
     if (R[0] != 0.0) {
       for (int b = r + threadIdx.x; b < nc; b += blockDim.x) {
         for (int a = r - 1; a >= 0; --a) {
-          double v = R[a + b * SK_CAND];
-          for (int a2 = a + 1; a2 < r; ++a2) v = fma(-R[a + a2 * SK_CAND], R[a2 + b * SK_CAND], v);
-          R[a + b * SK_CAND] = v / R[a + a * SK_CAND];
+          double v = R[a + b * LD];
+          for (int a2 = a + 1; a2 < r; ++a2) v = fma(-R[a + a2 * LD], R[a2 + b * LD], v);
+          R[a + b * LD] = v / R[a + a * LD];
         }
       }
     } else {
       for (int b = r + threadIdx.x; b < nc; b += blockDim.x)
-        for (int a = 0; a < r; ++a) R[a + b * SK_CAND] = 0.0;
+        for (int a = 0; a < r; ++a) R[a + b * LD] = 0.0;
     }
     __syncthreads();
   } else {
@@ -237,7 +339,7 @@ __global__ void __launch_bounds__(256, 1) k_skeletonize(const int* __restrict__ 
     const int k = e % nc, a = e / nc;   // pivot position k, column a
     double v;
     if (k < r) v = (k == a) ? 1.0 : 0.0;
-    else v = id ? R[a + k * SK_CAND] : 0.0;
+    else v = id ? R[a + k * LD] : 0.0;
     Tc[piv[k] + a * SK_CAND] = v;
   }
   for (int a = threadIdx.x; a < 64; a += blockDim.x) skel[(int64_t)c * 64 + a] = a < r ? cd[piv[a]] : -1;
@@ -306,9 +408,26 @@ __global__ void k_skel_nodes(const int* __restrict__ skel, const int* __restrict
   }
 }
 
-size_t skeleton_smem_bytes() {
-  return sizeof(double) * ((size_t)SK_CAND * SK_CAND + SK_CHUNK * SK_CAND + SK_CAND * 3 + SK_CAND + SK_CAND + 8 + 4) +
-         sizeof(int) * (SK_CAND + 8);
+// Launches one level's clusters. `rows`: sampled rows of the largest cluster. Parts: as many
+// CTAs per cluster as fill the GPU, but no more than the square root of the chunks, since
+// the parts' factors are folded one after the other.
+template <int NC>
+static void skeletonize_level(Matrix& M, int ncl, int64_t rows, const int* cand, const int* ncand, const int* samp,
+                              const int64_t* soff, int* skel, int* rank, double* T) {
+  cudaStream_t s = M.stream;
+  const int smem = (int)sizeof(SkelSmem<NC>), room = NC == 64 ? 2 * 152 : 152;
+  H2_CUDA(cudaFuncSetAttribute(k_skeletonize<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  const int most = (int)std::sqrt((double)((rows + SK_CHUNK - 1) / SK_CHUNK));
+  const int parts = std::max(1, std::min(room / ncl, most));
+  double* Rpart = parts > 1 ? (double*)M.alloc(sizeof(double) * (size_t)ncl * parts * NC * NC) : nullptr;
+  for (int finish = 0; finish < (parts > 1 ? 2 : 1); ++finish) {
+    { k_skeletonize<NC><<<finish ? ncl : ncl * parts, 4 * NC, smem, s>>>(cand, ncand, samp, soff, M.d_X, M.d_sw, M.dim,
+                                                                         M.kp, M.basis_tol, M.k, parts, finish, Rpart,
+                                                                         skel, rank, T);
+      ::h2mg::count_launch(); }
+    H2_LAUNCH_CHECK();
+  }
+  M.free_owned(Rpart);
 }
 
 // Skeletons of every cluster at levels t*..L, bottom-up, into M.d_skel (slot-indexed,
@@ -322,8 +441,6 @@ void build_skeletons(Matrix& M) {
   M.tid.p = M.alloc(M.tid.bytes);
   M.h_rank.assign(nsl, 0);
   M.d_rank = (int*)M.alloc(sizeof(int) * nsl);
-  const size_t smem = skeleton_smem_bytes();
-  H2_CUDA(cudaFuncSetAttribute(k_skeletonize, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   // candidates of two consecutive levels (this one and the one below)
   std::vector<int> ncand_h;                      // of level ell
   int* d_cand = (int*)M.alloc(sizeof(int) * ((size_t)1 << L) * SK_CAND);
@@ -382,11 +499,15 @@ void build_skeletons(Matrix& M) {
         H2_LAUNCH_CHECK();
       }
     }
-    { k_skeletonize<<<ncl, 256, smem, s>>>(d_cand, d_ncand, d_samp, d_soff, M.d_X, M.d_sw, M.dim, M.kp, M.basis_tol,
-                                          M.k, M.d_skel + (size_t)M.slot0(ell) * 64, M.d_rank + M.slot0(ell),
-                                          (double*)M.tid.p + (size_t)M.slot0(ell) * SK_CAND * 64);
-      ::h2mg::count_launch(); }
-    H2_LAUNCH_CHECK();
+    int64_t rows = 0;
+    int most = 0;
+    for (int j = 0; j < ncl; ++j) {
+      rows = std::max(rows, soff[j + 1] - soff[j]);
+      most = std::max(most, ncand_h[j]);
+    }
+    (most <= 64 ? skeletonize_level<64> : skeletonize_level<SK_CAND>)(
+        M, ncl, rows, d_cand, d_ncand, d_samp, d_soff, M.d_skel + (size_t)M.slot0(ell) * 64, M.d_rank + M.slot0(ell),
+        (double*)M.tid.p + (size_t)M.slot0(ell) * SK_CAND * 64);
     H2_CUDA(cudaMemcpyAsync(M.h_rank.data() + M.slot0(ell), M.d_rank + M.slot0(ell), sizeof(int) * ncl,
                             cudaMemcpyDeviceToHost, s));
     H2_CUDA(cudaStreamSynchronize(s));
