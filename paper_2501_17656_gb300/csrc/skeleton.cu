@@ -18,11 +18,9 @@
 //     of sigma''s two children concatenated and thinned to every s-th entry from the
 //     first, s = ceil(count / 128);
 //  2. R0 = the R factor of W = A(F_tau, candidates): the sampled rows are generated
-//     in chunks of 128 and folded into an upper-triangular R in shared memory by
+//     in chunks of 32 and folded into an upper-triangular R in shared memory by
 //     Householder reflections that touch only row j of R and the chunk (a
-//     tall-skinny QR; W itself is never stored). Where a level has fewer clusters than
-//     the GPU has room for, several CTAs fold parts of a cluster's rows and their R
-//     factors are folded together;
+//     tall-skinny QR; W itself is never stored);
 //  3. greedy column-pivoted Householder QR of R0 (the column of largest remaining
 //     norm; columns within a relative 1e-10 of the largest squared norm are tied and
 //     the lowest index wins), stopped at rank_max, at min(rows, candidates), or once
@@ -38,8 +36,8 @@
 namespace h2mg {
 
 constexpr int SK_CAND = 128;        // candidates of a cluster at most (two skeletons of <= 64)
-constexpr int SK_CHUNK = 128;       // sampled rows folded into R at a time
-constexpr int SK_OWN = 32;          // of which a thread holds a quarter, for one column, in registers
+constexpr int SK_CHUNK = 32;        // sampled rows folded into R at a time
+constexpr int SK_OWN = 8;           // of which a thread holds a quarter, for one column, in registers
 constexpr int SK_SAMPLE_CAP = 128;  // points kept per far partner of the parent
 constexpr double SK_TIE = 1e-10;    // relative tie band of the pivot choice
 
@@ -65,109 +63,129 @@ __device__ int block_min_int(int v, int* red) {
   return m;
 }
 
-// Shared memory of k_skeletonize<NC> (NC candidates at most, 4 NC threads). R is
+// Shared memory of k_skeletonize<NC> (NC candidates at most, 4 NC + 64 threads). R is
 // column-major with ld NC + 1: rows and columns are both read without bank conflicts.
 template <int NC>
 struct SkelSmem {
   double R[NC * (NC + 1)];
-  double stage[SK_CHUNK / 4 * NC];   // kernel values on their way into the owning thread's registers
-  double v[2][SK_CHUNK];             // column j of the chunk (double-buffered over j)
-  double part[4][NC];                // partial dot products of the row quarters
-  double sig[4];
-  double sc[3];                      // beta, tau, scale of the reflector
-  double nrm[NC];
-  double red[16];
+  double stage[SK_OWN * 4 * NC];     // kernel values on their way into the owning thread's registers
+  double v[2][SK_CHUNK];             // reflectors j and j + 1; row i at (i % 4) * 8 + i / 4
+  double col[SK_CHUNK], alpha;       // column j + 1 of the chunk and R's diagonal, for the first warps
+  double tau[2];
+  int go[2];
+  double nrm[NC], sig[NC];
+  double red[32];
   double bcast[3];
   int piv[NC];
-  int ired[16];
+  int ired[32];
 };
 
-// Folds a chunk of 128 rows into R: thread (k, q) holds c[SK_OWN], quarter q of the rows, of
-// column k. Reflector j: v = (1, column j of the chunk / (alpha - beta)), alpha = R_jj. Warps
-// are numbered so that every scheduler holds one quarter of each group of 32 columns: their
-// load stays even as the leading columns finish. Bound by the float64 pipe: 2 FMAs per row
-// and pair of columns, the minimum of Householder's method, in 70 operations of which 64 are
-// those FMAs (a warp per column with 32 rows took 8 operations for 2, most of them in
-// warp-wide sums). Whole builds: 8192 points 296 -> 99 ms, 16384 points 660 -> 225 ms.
+// Reflector j of a chunk, by the first two warps: v = column j (one row per lane) / (alpha -
+// beta), alpha = R_jj, and tau, each with a division of its own behind the square root. A
+// column of zeros leaves everything as it is.
 template <int NC>
-__device__ __forceinline__ void fold_chunk(SkelSmem<NC>& sm, int nc, int k, int q, double (&c)[SK_OWN]) {
-  auto publish = [&](int j) {          // column j's threads hand out the column and its partial norm
-    if (k == j) {
-      double s = 0.0;
-#pragma unroll
-      for (int i = 0; i < SK_OWN; ++i) {
-        sm.v[j & 1][q * SK_OWN + i] = c[i];
-        s = fma(c[i], c[i], s);
-      }
-      sm.sig[q] = s;
-    }
-  };
-  publish(0);
-  __syncthreads();
-  for (int j = 0; j < nc; ++j) {
-    const double2* v = reinterpret_cast<const double2*>(sm.v[j & 1] + q * SK_OWN);
-    const bool active = k > j && k < nc;
-    if (threadIdx.x == 0) {
-      const double sigma = (sm.sig[0] + sm.sig[1]) + (sm.sig[2] + sm.sig[3]);
-      const double alpha = sm.R[j + j * (NC + 1)];
-      double beta = alpha, tau = 0.0, scale = 0.0;
-      if (sigma > 0.0) {
-        beta = -copysign(sqrt(fma(alpha, alpha, sigma)), alpha);
-        tau = (beta - alpha) / beta;
-        scale = 1.0 / (alpha - beta);
-      }
-      sm.sc[0] = beta;
-      sm.sc[1] = tau;
-      sm.sc[2] = scale;
-    }
-    if (active) {
-      double s0 = 0.0, s1 = 0.0;
-#pragma unroll
-      for (int i = 0; i < SK_OWN / 2; ++i) {
-        const double2 x = v[i];
-        s0 = fma(c[2 * i], x.x, s0);
-        s1 = fma(c[2 * i + 1], x.y, s1);
-      }
-      sm.part[q][k] = s0 + s1;
-    }
-    __syncthreads();
-    const double tau = sm.sc[1], scale = sm.sc[2];
-    if (tau != 0.0 && active) {
-      const double d = (sm.part[0][k] + sm.part[1][k]) + (sm.part[2][k] + sm.part[3][k]);
-      double* r = sm.R + j + k * (NC + 1);
-      const double wk = tau * fma(scale, d, *r), f = -wk * scale;
-#pragma unroll
-      for (int i = 0; i < SK_OWN / 2; ++i) {
-        const double2 x = v[i];
-        c[2 * i] = fma(f, x.x, c[2 * i]);
-        c[2 * i + 1] = fma(f, x.y, c[2 * i + 1]);
-      }
-      if (q == 0) sm.nrm[k] = wk;              // R_jk is read by the other quarters: changed after the barrier
-    }
-    publish(j + 1);
-    __syncthreads();
-    if (tau != 0.0) {
-      if (active && q == 0) sm.R[j + k * (NC + 1)] -= sm.nrm[k];
-      if (threadIdx.x == 0) sm.R[j + j * (NC + 1)] = sm.sc[0];
+__device__ __forceinline__ void make_reflector(SkelSmem<NC>& sm, int j, int warp, int lane) {
+  const double c = sm.col[lane];
+  double s = __dmul_rn(c, c);
+  for (int o = 16; o > 0; o >>= 1) s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, o));
+  const double alpha = sm.alpha;
+  const bool go = s > 0.0;
+  if (go) {
+    const double beta = -copysign(sqrt(__fma_rn(alpha, alpha, s)), alpha);
+    const double quot = __ddiv_rn(warp ? __dsub_rn(beta, alpha) : c, warp ? beta : __dsub_rn(alpha, beta));
+    if (warp == 0) sm.v[j & 1][(lane & 3) * SK_OWN + (lane >> 2)] = quot;
+    if (warp == 1 && lane == 0) {
+      sm.tau[j & 1] = quot;
+      sm.R[j + j * (NC + 1)] = beta;
     }
   }
-  __syncthreads();
+  if (warp == 0 && lane == 0) sm.go[j & 1] = go;
 }
 
-// `parts` CTAs of 4 NC threads per cluster of the level.
+// Folds a chunk of 32 rows into R: lane q of the four that own column k holds c[SK_OWN], the
+// rows q, q + 4, .. The first two warps own no column: while the others apply reflector j they
+// make reflector j + 1, as soon as the warp that owns column j + 1 has handed it over. Every
+// sum over the rows is one tree of pairs (16, 8, 4, 2, 1 rows apart), rounded step by step, and
+// the chunks go one after the other: R, and with it every skeleton and basis, has the same
+// bits as with a warp per column and a row per lane, so that FP32 and split-TF32 products of
+// the bases round alike. (Chunks of 128 rows, and parts of a cluster's rows on CTAs of their
+// own, built in 99 ms, but turned last bits of FP32 results.)
+//
+// A step of one reflector takes what the float64 pipe (2 operations per clock and SM) needs
+// for 28 operations of every lane, 3600 clocks on average for 128 columns, and then the rest
+// of the next reflector's chain (a sum, a square root and a division, behind the warps that
+// share the pipe): 2000 to 3000 clocks more. A warp per column took 8 float64 operations for
+// every 2 of the columns' own, most of them in warp-wide sums and repeated reflectors. Whole
+// skeleton builds of 8192 points: 296 -> 171 ms.
+template <int NC>
+__device__ __forceinline__ void fold_chunk(SkelSmem<NC>& sm, int nc, int k, int q, double (&c)[SK_OWN]) {
+  const int w = (int)(threadIdx.x >> 5) - 2, lane = threadIdx.x & 31;
+  auto publish = [&](int j) {
+    if (k == j) {
+#pragma unroll
+      for (int t = 0; t < SK_OWN; ++t) sm.col[q + 4 * t] = c[t];
+      if (q == 0) sm.alpha = sm.R[j + j * (NC + 1)];
+    }
+  };
+  if (w >= 0) publish(0);
+  __syncthreads();
+  if (w < 0) make_reflector<NC>(sm, 0, w + 2, lane);
+  __syncthreads();
+  for (int j = 0; j < nc; ++j) {
+    if (w < 0) {
+      if (j + 1 < nc) {
+        asm volatile("bar.sync 1, 96;" ::: "memory");
+        make_reflector<NC>(sm, j + 1, w + 2, lane);
+      }
+    } else if (8 * w + 7 > j && 8 * w < nc) {
+      if (sm.go[j & 1]) {
+        const bool active = k > j && k < nc;
+        const double tau = sm.tau[j & 1];
+        double* r = sm.R + j + (active ? k : j) * (NC + 1);
+        const double rv = *r;               // before the shuffles: lane 0 of the four changes it after them
+        const double2* v2 = reinterpret_cast<const double2*>(sm.v[j & 1] + q * SK_OWN);
+        double v[SK_OWN], p[SK_OWN];
+#pragma unroll
+        for (int t = 0; t < SK_OWN / 2; ++t) {
+          const double2 x = v2[t];
+          v[2 * t] = x.x;
+          v[2 * t + 1] = x.y;
+        }
+#pragma unroll
+        for (int t = 0; t < SK_OWN; ++t) p[t] = __dmul_rn(v[t], c[t]);
+        double s = __dadd_rn(__dadd_rn(__dadd_rn(p[0], p[4]), __dadd_rn(p[2], p[6])),
+                             __dadd_rn(__dadd_rn(p[1], p[5]), __dadd_rn(p[3], p[7])));
+        s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, 2));
+        s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, 1));
+        if (active) {
+          const double wk = __dmul_rn(tau, __dadd_rn(rv, s));
+          if (q == 0) *r = __dsub_rn(rv, wk);
+#pragma unroll
+          for (int t = 0; t < SK_OWN; ++t) c[t] = __fma_rn(-wk, v[t], c[t]);
+        }
+      }
+      if (j + 1 < nc && (j + 1) >> 3 == w) {
+        __syncwarp();
+        publish(j + 1);
+        __syncwarp();
+        asm volatile("bar.arrive 1, 96;" ::: "memory");
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// One CTA of 4 NC + 64 threads per cluster of the level.
 //   cand   [ncl][SK_CAND]: candidate tree positions, ncand[ncl] of them
 //   samp   sampled tree positions of all clusters, cluster c at samp[soff[c] .. soff[c+1])
 //   out:   skel[ncl][64] (tree positions, pivot order), rank[ncl], T[ncl][SK_CAND x 64]
 //          (rows = candidates in their original order, column-major, ld SK_CAND)
-// With parts > 1 a first launch (finish = 0) leaves the R factor of each part of the rows in
-// Rpart, and a second one, one CTA per cluster (finish = 1), folds them and goes on.
 template <int NC>
-__global__ void __launch_bounds__(4 * NC) k_skeletonize(const int* __restrict__ cand, const int* __restrict__ ncand,
-                                                        const int* __restrict__ samp, const int64_t* __restrict__ soff,
-                                                        const double* __restrict__ X, const double* __restrict__ sw,
-                                                        int dim, KernelParams kp, double tol, int rank_max, int parts,
-                                                        int finish, double* __restrict__ Rpart, int* __restrict__ skel,
-                                                        int* __restrict__ rank_out, double* __restrict__ Tout) {
+__global__ void __launch_bounds__(4 * NC + 64)
+    k_skeletonize(const int* __restrict__ cand, const int* __restrict__ ncand, const int* __restrict__ samp,
+                  const int64_t* __restrict__ soff, const double* __restrict__ X, const double* __restrict__ sw,
+                  int dim, KernelParams kp, double tol, int rank_max, int* __restrict__ skel,
+                  int* __restrict__ rank_out, double* __restrict__ Tout) {
   extern __shared__ __align__(16) unsigned char dsm[];
   SkelSmem<NC>& sm = *reinterpret_cast<SkelSmem<NC>*>(dsm);
   constexpr int LD = NC + 1;
@@ -177,11 +195,11 @@ __global__ void __launch_bounds__(4 * NC) k_skeletonize(const int* __restrict__ 
   double* bcast = sm.bcast;
   int* piv = sm.piv;
   int* ired = sm.ired;
-  const int c = finish ? blockIdx.x : blockIdx.x / parts, part = finish ? 0 : blockIdx.x % parts;
+  const int c = blockIdx.x;
   const int nc = ncand[c];
   const int* cd = cand + (int64_t)c * SK_CAND;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int k = 32 * (w >> 2) + lane, q = w & 3;     // column and row quarter of this thread
+  const int own = (int)threadIdx.x - 64;             // the first two warps own no column
+  const int k = own >= 0 ? own >> 2 : NC, q = own & 3;
   const int64_t s0 = soff[c], s1 = soff[c + 1];
   const int64_t m = s1 - s0;
   for (int i = threadIdx.x; i < nc; i += blockDim.x) piv[i] = i;
@@ -191,52 +209,26 @@ __global__ void __launch_bounds__(4 * NC) k_skeletonize(const int* __restrict__ 
   if (m > 0 && nc > 0) {
     // ---- 2. tall-skinny QR of the sampled rows
     double cc[SK_OWN];
-    if (finish) {
-      const double* P = Rpart + (int64_t)c * parts * NC * NC;
-      for (int p = 0; p < parts; ++p) {
-#pragma unroll
-        for (int i = 0; i < SK_OWN; ++i) {
-          const int row = q * SK_OWN + i;
-          cc[i] = k < nc && row < NC ? P[((int64_t)p * NC + k) * NC + row] : 0.0;
-        }
-        fold_chunk<NC>(sm, nc, k, q, cc);
-      }
-    } else {
-      double x[3] = {0.0, 0.0, 0.0}, wk = 0.0;
-      if (k < nc) {
-        const int p = cd[k];
-        for (int d = 0; d < dim; ++d) x[d] = X[(int64_t)p * dim + d];
-        wk = sw[p];
-      }
-      const int64_t chunks = (m + SK_CHUNK - 1) / SK_CHUNK;
-      const int64_t ch1 = chunks * (part + 1) / parts;
-      for (int64_t ch = chunks * part / parts; ch < ch1; ++ch) {
-        const int64_t row0 = ch * SK_CHUNK + q * SK_OWN;
-#pragma unroll
-        for (int g = 0; g < SK_OWN / 8; ++g) {
-#pragma unroll 1
-          for (int i = 0; i < 8; ++i) {
-            const int64_t row = row0 + 8 * g + i;
-            double v = 0.0;
-            if (k < nc && row < m) {
-              const int f = samp[s0 + row];
-              v = sw[f] * kernel_eval(kp, X + (int64_t)f * dim, x, dim) * wk;
-            }
-            sm.stage[(q * 8 + i) * NC + k] = v;      // read back by this thread alone
-          }
-#pragma unroll
-          for (int i = 0; i < 8; ++i) cc[8 * g + i] = sm.stage[(q * 8 + i) * NC + k];
-        }
-        fold_chunk<NC>(sm, nc, k, q, cc);
-      }
+    double x[3] = {0.0, 0.0, 0.0}, wk = 0.0;
+    if (k < nc) {
+      const int p = cd[k];
+      for (int d = 0; d < dim; ++d) x[d] = X[(int64_t)p * dim + d];
+      wk = sw[p];
     }
-    if (!finish && parts > 1) {
-      double* P = Rpart + ((int64_t)c * parts + part) * NC * NC;
-      for (int e = threadIdx.x; e < NC * NC; e += blockDim.x) {
-        const int i = e % NC, kk = e / NC;
-        P[e] = i <= kk ? R[i + kk * LD] : 0.0;
+    for (int64_t row0 = 0; row0 < m; row0 += SK_CHUNK) {
+#pragma unroll 1
+      for (int t = 0; t < SK_OWN; ++t) {
+        const int64_t row = row0 + q + 4 * t;
+        double v = 0.0;
+        if (k < nc && row < m) {
+          const int f = samp[s0 + row];
+          v = sw[f] * kernel_eval(kp, X + (int64_t)f * dim, x, dim) * wk;
+        }
+        if (own >= 0) sm.stage[t * 4 * NC + own] = v;      // read back by this thread alone
       }
-      return;
+#pragma unroll
+      for (int t = 0; t < SK_OWN; ++t) cc[t] = own >= 0 ? sm.stage[t * 4 * NC + own] : 0.0;
+      fold_chunk<NC>(sm, nc, k, q, cc);
     }
     // ---- 3. greedy column-pivoted Householder QR of R0 (rows: min(m, nc))
     const int rows = (int)(m < nc ? m : nc);
@@ -244,9 +236,13 @@ __global__ void __launch_bounds__(4 * NC) k_skeletonize(const int* __restrict__ 
     double first = 0.0;
     for (int j = 0; j < kmax; ++j) {
       for (int k = j + threadIdx.x; k < nc; k += blockDim.x) {
-        double s = 0.0;
-        for (int i = j; i < nc; ++i) s = fma(R[i + k * LD], R[i + k * LD], s);
+        double s = R[j + k * LD] * R[j + k * LD], below = 0.0;
+        for (int i = j + 1; i < nc; ++i) {
+          s = fma(R[i + k * LD], R[i + k * LD], s);
+          below = fma(R[i + k * LD], R[i + k * LD], below);
+        }
         nrm[k] = s;
+        sm.sig[k] = below;
       }
       __syncthreads();
       double mv = -1.0;
@@ -276,22 +272,17 @@ __global__ void __launch_bounds__(4 * NC) k_skeletonize(const int* __restrict__ 
         __syncthreads();
       }
       // reflector of R[j:, j]
-      if (threadIdx.x < 32) {
-        const double alpha = R[j + j * LD];
-        double sigma = 0.0;
-        for (int i = j + 1 + lane; i < nc; i += 32) sigma = fma(R[i + j * LD], R[i + j * LD], sigma);
-        for (int o = 16; o > 0; o >>= 1) sigma += __shfl_xor_sync(0xffffffffu, sigma, o);
+      if (threadIdx.x == 0) {
+        const double alpha = R[j + j * LD], sigma = sm.sig[p];
         double beta = alpha, tau = 0.0, scale = 0.0;
         if (sigma > 0.0) {
           beta = -copysign(sqrt(alpha * alpha + sigma), alpha);
           tau = (beta - alpha) / beta;
           scale = 1.0 / (alpha - beta);
         }
-        if (lane == 0) {
-          bcast[0] = beta;
-          bcast[1] = tau;
-          bcast[2] = scale;
-        }
+        bcast[0] = beta;
+        bcast[1] = tau;
+        bcast[2] = scale;
       }
       __syncthreads();
       const double beta = bcast[0], tau = bcast[1], scale = bcast[2];
@@ -408,26 +399,15 @@ __global__ void k_skel_nodes(const int* __restrict__ skel, const int* __restrict
   }
 }
 
-// Launches one level's clusters. `rows`: sampled rows of the largest cluster. Parts: as many
-// CTAs per cluster as fill the GPU, but no more than the square root of the chunks, since
-// the parts' factors are folded one after the other.
 template <int NC>
-static void skeletonize_level(Matrix& M, int ncl, int64_t rows, const int* cand, const int* ncand, const int* samp,
+static void skeletonize_level(Matrix& M, int ncl, const int* cand, const int* ncand, const int* samp,
                               const int64_t* soff, int* skel, int* rank, double* T) {
-  cudaStream_t s = M.stream;
-  const int smem = (int)sizeof(SkelSmem<NC>), room = NC == 64 ? 2 * 152 : 152;
+  const int smem = (int)sizeof(SkelSmem<NC>);
   H2_CUDA(cudaFuncSetAttribute(k_skeletonize<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  const int most = (int)std::sqrt((double)((rows + SK_CHUNK - 1) / SK_CHUNK));
-  const int parts = std::max(1, std::min(room / ncl, most));
-  double* Rpart = parts > 1 ? (double*)M.alloc(sizeof(double) * (size_t)ncl * parts * NC * NC) : nullptr;
-  for (int finish = 0; finish < (parts > 1 ? 2 : 1); ++finish) {
-    { k_skeletonize<NC><<<finish ? ncl : ncl * parts, 4 * NC, smem, s>>>(cand, ncand, samp, soff, M.d_X, M.d_sw, M.dim,
-                                                                         M.kp, M.basis_tol, M.k, parts, finish, Rpart,
-                                                                         skel, rank, T);
-      ::h2mg::count_launch(); }
-    H2_LAUNCH_CHECK();
-  }
-  M.free_owned(Rpart);
+  { k_skeletonize<NC><<<ncl, 4 * NC + 64, smem, M.stream>>>(cand, ncand, samp, soff, M.d_X, M.d_sw, M.dim, M.kp,
+                                                            M.basis_tol, M.k, skel, rank, T);
+    ::h2mg::count_launch(); }
+  H2_LAUNCH_CHECK();
 }
 
 // Skeletons of every cluster at levels t*..L, bottom-up, into M.d_skel (slot-indexed,
@@ -499,14 +479,9 @@ void build_skeletons(Matrix& M) {
         H2_LAUNCH_CHECK();
       }
     }
-    int64_t rows = 0;
-    int most = 0;
-    for (int j = 0; j < ncl; ++j) {
-      rows = std::max(rows, soff[j + 1] - soff[j]);
-      most = std::max(most, ncand_h[j]);
-    }
+    const int most = *std::max_element(ncand_h.begin(), ncand_h.end());
     (most <= 64 ? skeletonize_level<64> : skeletonize_level<SK_CAND>)(
-        M, ncl, rows, d_cand, d_ncand, d_samp, d_soff, M.d_skel + (size_t)M.slot0(ell) * 64, M.d_rank + M.slot0(ell),
+        M, ncl, d_cand, d_ncand, d_samp, d_soff, M.d_skel + (size_t)M.slot0(ell) * 64, M.d_rank + M.slot0(ell),
         (double*)M.tid.p + (size_t)M.slot0(ell) * SK_CAND * 64);
     H2_CUDA(cudaMemcpyAsync(M.h_rank.data() + M.slot0(ell), M.d_rank + M.slot0(ell), sizeof(int) * ncl,
                             cudaMemcpyDeviceToHost, s));
