@@ -30,6 +30,7 @@
 // candidates with T = [I; 0].
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 
 #include "internal.h"
 
@@ -37,7 +38,6 @@ namespace h2mg {
 
 constexpr int SK_CAND = 128;        // candidates of a cluster at most (two skeletons of <= 64)
 constexpr int SK_CHUNK = 32;        // sampled rows folded into R at a time
-constexpr int SK_OWN = 8;           // of which a thread holds a quarter, for one column, in registers
 constexpr int SK_SAMPLE_CAP = 128;  // points kept per far partner of the parent
 constexpr double SK_TIE = 1e-10;    // relative tie band of the pivot choice
 
@@ -63,129 +63,198 @@ __device__ int block_min_int(int v, int* red) {
   return m;
 }
 
-// Shared memory of k_skeletonize<NC> (NC candidates at most, 4 NC + 64 threads). R is
-// column-major with ld NC + 1: rows and columns are both read without bank conflicts.
+// How a CTA folds the rows of a cluster with at most NC candidates: NG groups of warps, each
+// with a chunk of its own in hand, LPC lanes per column, and two warps per group for the
+// reflectors.
+template <int NC>
+struct Skel {
+  static constexpr int NG = NC == 64 ? 3 : 2, LPC = NC == 64 ? 4 : 2;
+  static constexpr int OWN = SK_CHUNK / LPC;               // rows of a column per lane, in registers
+  static constexpr int CPW = 32 / LPC;                     // columns per warp
+  static constexpr int GROUP = NC * LPC + 64, THREADS = NG * GROUP;
+  static constexpr int FILL = 8;                           // kernel values staged at a time
+};
+
+// What the warps of a group share.
+template <int NC>
+struct SkelGroup {
+  double stage[Skel<NC>::FILL * NC * Skel<NC>::LPC];   // kernel values on their way into the owning thread's registers
+  alignas(16) double v[2][SK_CHUNK]; // reflectors j and j + 1; row i at (i % LPC) * OWN + i / LPC (read in pairs)
+  double col[SK_CHUNK];              // column j + 1 of the chunk, on its way to the first warps
+  double alpha;                      // R's diagonal there
+  double tau[2];
+  int go[2];
+  int done;                          // reflectors applied so far, over all its chunks
+};
+
+// Shared memory of k_skeletonize<NC>. R is column-major with ld NC + 1: rows and columns are
+// both read without bank conflicts.
 template <int NC>
 struct SkelSmem {
   double R[NC * (NC + 1)];
-  double stage[SK_OWN * 4 * NC];     // kernel values on their way into the owning thread's registers
-  double v[2][SK_CHUNK];             // reflectors j and j + 1; row i at (i % 4) * 8 + i / 4
-  double col[SK_CHUNK], alpha;       // column j + 1 of the chunk and R's diagonal, for the first warps
-  double tau[2];
-  int go[2];
+  SkelGroup<NC> g[Skel<NC>::NG];
   double nrm[NC], sig[NC];
   double red[32];
   double bcast[3];
   int piv[NC];
   int ired[32];
+  int late;                          // a wait for another group ran out
 };
 
-// Reflector j of a chunk, by the first two warps: v = column j (one row per lane) / (alpha -
-// beta), alpha = R_jj, and tau, each with a division of its own behind the square root. A
-// column of zeros leaves everything as it is.
+static_assert(offsetof(SkelSmem<64>, g) % 16 == 0 && sizeof(SkelGroup<64>) % 16 == 0 &&
+                  offsetof(SkelGroup<64>, v) % 16 == 0 && offsetof(SkelSmem<128>, g) % 16 == 0 &&
+                  sizeof(SkelGroup<128>) % 16 == 0 && offsetof(SkelGroup<128>, v) % 16 == 0,
+              "reflectors are read 16 bytes at a time");
+
+// Reflector j of a chunk, by the group's first two warps: v = column j (one row per lane) /
+// (alpha - beta), alpha = R_jj, and tau, each with a division of its own behind the square
+// root. A column of zeros leaves everything as it is.
 template <int NC>
-__device__ __forceinline__ void make_reflector(SkelSmem<NC>& sm, int j, int warp, int lane) {
-  const double c = sm.col[lane];
+__device__ __forceinline__ void make_reflector(SkelGroup<NC>& sg, double* R, int j, int warp, int lane) {
+  using K = Skel<NC>;
+  const double c = sg.col[lane];
   double s = __dmul_rn(c, c);
   for (int o = 16; o > 0; o >>= 1) s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, o));
-  const double alpha = sm.alpha;
+  const double alpha = sg.alpha;
   const bool go = s > 0.0;
   if (go) {
     const double beta = -copysign(sqrt(__fma_rn(alpha, alpha, s)), alpha);
     const double quot = __ddiv_rn(warp ? __dsub_rn(beta, alpha) : c, warp ? beta : __dsub_rn(alpha, beta));
-    if (warp == 0) sm.v[j & 1][(lane & 3) * SK_OWN + (lane >> 2)] = quot;
+    if (warp == 0) sg.v[j & 1][(lane % K::LPC) * K::OWN + lane / K::LPC] = quot;
     if (warp == 1 && lane == 0) {
-      sm.tau[j & 1] = quot;
-      sm.R[j + j * (NC + 1)] = beta;
+      sg.tau[j & 1] = quot;
+      R[j + j * (NC + 1)] = beta;
     }
   }
-  if (warp == 0 && lane == 0) sm.go[j & 1] = go;
+  if (warp == 0 && lane == 0) sg.go[j & 1] = go;
 }
 
-// Folds a chunk of 32 rows into R: lane q of the four that own column k holds c[SK_OWN], the
-// rows q, q + 4, .. The first two warps own no column: while the others apply reflector j they
-// make reflector j + 1, as soon as the warp that owns column j + 1 has handed it over. Every
-// sum over the rows is one tree of pairs (16, 8, 4, 2, 1 rows apart), rounded step by step, and
-// the chunks go one after the other: R, and with it every skeleton and basis, has the same
-// bits as with a warp per column and a row per lane, so that FP32 and split-TF32 products of
-// the bases round alike. (Chunks of 128 rows, and parts of a cluster's rows on CTAs of their
-// own, built in 99 ms, but turned last bits of FP32 results.)
+// Waits until a group has applied `want` reflectors, two seconds at most; after a wait that
+// ran out, no wait of the CTA waits any more.
+__device__ __forceinline__ void wait_group(const int* done, int want, int* late) {
+  const volatile int* d = done;
+  if (*d >= want) return;
+  const long long t0 = clock64();
+  while (*d < want && !*(volatile int*)late)
+    if (clock64() - t0 > (1ll << 32)) *(volatile int*)late = 1;
+}
+
+// Folds chunk number `ch` (32 rows) into R: lane q of the LPC that own column k holds c[OWN],
+// the rows q, q + LPC, .. The group's first two warps own no column: while the others apply
+// reflector j they make reflector j + 1, as soon as the warp that owns column j + 1 has handed
+// it over. Chunks go to the groups in turn, and each follows the one before it through the
+// columns: step j waits until that one has finished with row j of R. Every sum over the rows is
+// one tree of pairs (16, 8, 4, 2, 1 rows apart), rounded step by step, and the chunks meet R
+// one after the other: R, and with it every skeleton and basis, has the same bits as with a
+// warp per column and a row per lane, so that FP32 and split-TF32 products of the bases round
+// alike. (Chunks of 128 rows, and parts of a cluster's rows on CTAs of their own, built 8192
+// points in 99 ms, but turned last bits of FP32 results.)
 //
-// A step of one reflector takes what the float64 pipe (2 operations per clock and SM) needs
-// for 28 operations of every lane, 3600 clocks on average for 128 columns, and then the rest
-// of the next reflector's chain (a sum, a square root and a division, behind the warps that
-// share the pipe): 2000 to 3000 clocks more. A warp per column took 8 float64 operations for
-// every 2 of the columns' own, most of them in warp-wide sums and repeated reflectors. Whole
-// skeleton builds of 8192 points: 296 -> 171 ms.
+// A step is the columns' work, 98 float64 operations per column of 32 rows (3700 clocks on
+// average for 128 columns on a pipe of 2 per clock and SM), and the next reflector's chain: a
+// sum, a square root and a division, 4000 clocks. A warp per column spent 8 operations for
+// every 2 of the columns' own, mostly on warp-wide sums and on the reflector in every warp:
+// 8192 points in 296 ms. One group of four lanes per column 171 ms; with the groups, one's
+// chain runs beside another's columns: 138 ms.
 template <int NC>
-__device__ __forceinline__ void fold_chunk(SkelSmem<NC>& sm, int nc, int k, int q, double (&c)[SK_OWN]) {
-  const int w = (int)(threadIdx.x >> 5) - 2, lane = threadIdx.x & 31;
+__device__ __forceinline__ void fold_chunk(SkelSmem<NC>& sm, int nc, int64_t ch, int group, int k, int q,
+                                           double (&c)[Skel<NC>::OWN]) {
+  using K = Skel<NC>;
+  const int w = (int)(threadIdx.x % K::GROUP >> 5) - 2, lane = threadIdx.x & 31;
+  SkelGroup<NC>& sg = sm.g[group];
+  const int before = (int)((ch / K::NG) * nc);                          // of this group's earlier chunks
+  const int* ahead = ch > 0 ? &sm.g[(group + K::NG - 1) % K::NG].done : nullptr;
+  const int ahead0 = ch > 0 ? (int)(((ch - 1) / K::NG) * nc) : 0;
   auto publish = [&](int j) {
     if (k == j) {
 #pragma unroll
-      for (int t = 0; t < SK_OWN; ++t) sm.col[q + 4 * t] = c[t];
-      if (q == 0) sm.alpha = sm.R[j + j * (NC + 1)];
+      for (int t = 0; t < K::OWN; ++t) sg.col[q + K::LPC * t] = c[t];
+      if (q == 0) sg.alpha = sm.R[j + j * (NC + 1)];
     }
   };
+  auto group_sync = [&]() {
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(K::GROUP) : "memory");
+  };
+  // rows 0 .. j of R are the chunk's own from here on
+  auto follow = [&](int j) {
+    if (ahead && threadIdx.x % K::GROUP == 0) {
+      wait_group(ahead, ahead0 + min(j + 1, nc), &sm.late);
+      __threadfence_block();
+    }
+  };
+  follow(1);
+  group_sync();
   if (w >= 0) publish(0);
-  __syncthreads();
-  if (w < 0) make_reflector<NC>(sm, 0, w + 2, lane);
-  __syncthreads();
+  group_sync();
+  if (w < 0) make_reflector<NC>(sg, sm.R, 0, w + 2, lane);
+  group_sync();
   for (int j = 0; j < nc; ++j) {
     if (w < 0) {
       if (j + 1 < nc) {
-        asm volatile("bar.sync 1, 96;" ::: "memory");
-        make_reflector<NC>(sm, j + 1, w + 2, lane);
+        __syncwarp();
+        asm volatile("bar.sync %0, 96;" ::"r"(1 + K::NG + group) : "memory");
+        make_reflector<NC>(sg, sm.R, j + 1, w + 2, lane);
       }
-    } else if (8 * w + 7 > j && 8 * w < nc) {
-      if (sm.go[j & 1]) {
+      follow(j + 2);
+    } else if (K::CPW * (w + 1) - 1 > j && K::CPW * w < nc) {
+      if (sg.go[j & 1]) {
         const bool active = k > j && k < nc;
-        const double tau = sm.tau[j & 1];
+        const double tau = sg.tau[j & 1];
         double* r = sm.R + j + (active ? k : j) * (NC + 1);
-        const double rv = *r;               // before the shuffles: lane 0 of the four changes it after them
-        const double2* v2 = reinterpret_cast<const double2*>(sm.v[j & 1] + q * SK_OWN);
-        double v[SK_OWN], p[SK_OWN];
+        const double rv = *r;               // before the shuffles: the column's first lane changes it after them
+        const double2* v = reinterpret_cast<const double2*>(sg.v[j & 1] + q * K::OWN);
+        double p[K::OWN];
 #pragma unroll
-        for (int t = 0; t < SK_OWN / 2; ++t) {
-          const double2 x = v2[t];
-          v[2 * t] = x.x;
-          v[2 * t + 1] = x.y;
+        for (int t = 0; t < K::OWN / 2; ++t) {
+          const double2 x = v[t];
+          p[2 * t] = __dmul_rn(x.x, c[2 * t]);
+          p[2 * t + 1] = __dmul_rn(x.y, c[2 * t + 1]);
         }
 #pragma unroll
-        for (int t = 0; t < SK_OWN; ++t) p[t] = __dmul_rn(v[t], c[t]);
-        double s = __dadd_rn(__dadd_rn(__dadd_rn(p[0], p[4]), __dadd_rn(p[2], p[6])),
-                             __dadd_rn(__dadd_rn(p[1], p[5]), __dadd_rn(p[3], p[7])));
-        s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, 2));
-        s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, 1));
+        for (int h = K::OWN / 2; h > 0; h >>= 1)
+#pragma unroll
+          for (int t = 0; t < h; ++t) p[t] = __dadd_rn(p[t], p[t + h]);
+        double s = p[0];
+#pragma unroll
+        for (int o = K::LPC / 2; o > 0; o >>= 1) s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, o));
         if (active) {
           const double wk = __dmul_rn(tau, __dadd_rn(rv, s));
           if (q == 0) *r = __dsub_rn(rv, wk);
 #pragma unroll
-          for (int t = 0; t < SK_OWN; ++t) c[t] = __fma_rn(-wk, v[t], c[t]);
+          for (int t = 0; t < K::OWN / 2; ++t) {
+            const double2 x = v[t];
+            c[2 * t] = __fma_rn(-wk, x.x, c[2 * t]);
+            c[2 * t + 1] = __fma_rn(-wk, x.y, c[2 * t + 1]);
+          }
         }
       }
-      if (j + 1 < nc && (j + 1) >> 3 == w) {
+      if (j + 1 < nc && (j + 1) / K::CPW == w) {
         __syncwarp();
         publish(j + 1);
         __syncwarp();
-        asm volatile("bar.arrive 1, 96;" ::: "memory");
+        asm volatile("bar.arrive %0, 96;" ::"r"(1 + K::NG + group) : "memory");
       }
     }
-    __syncthreads();
+    group_sync();
+    if (threadIdx.x % K::GROUP == 0) {
+      __threadfence_block();
+      *(volatile int*)&sg.done = before + j + 1;
+    }
   }
 }
 
-// One CTA of 4 NC + 64 threads per cluster of the level.
+// One CTA per cluster of the level.
 //   cand   [ncl][SK_CAND]: candidate tree positions, ncand[ncl] of them
 //   samp   sampled tree positions of all clusters, cluster c at samp[soff[c] .. soff[c+1])
 //   out:   skel[ncl][64] (tree positions, pivot order), rank[ncl], T[ncl][SK_CAND x 64]
 //          (rows = candidates in their original order, column-major, ld SK_CAND)
 template <int NC>
-__global__ void __launch_bounds__(4 * NC + 64)
+__global__ void __launch_bounds__(Skel<NC>::THREADS)
     k_skeletonize(const int* __restrict__ cand, const int* __restrict__ ncand, const int* __restrict__ samp,
                   const int64_t* __restrict__ soff, const double* __restrict__ X, const double* __restrict__ sw,
                   int dim, KernelParams kp, double tol, int rank_max, int* __restrict__ skel,
-                  int* __restrict__ rank_out, double* __restrict__ Tout) {
+                  int* __restrict__ rank_out, double* __restrict__ Tout, int* __restrict__ late) {
   extern __shared__ __align__(16) unsigned char dsm[];
   SkelSmem<NC>& sm = *reinterpret_cast<SkelSmem<NC>*>(dsm);
   constexpr int LD = NC + 1;
@@ -198,38 +267,49 @@ __global__ void __launch_bounds__(4 * NC + 64)
   const int c = blockIdx.x;
   const int nc = ncand[c];
   const int* cd = cand + (int64_t)c * SK_CAND;
-  const int own = (int)threadIdx.x - 64;             // the first two warps own no column
-  const int k = own >= 0 ? own >> 2 : NC, q = own & 3;
+  using K = Skel<NC>;
+  const int group = threadIdx.x / K::GROUP;
+  const int own = (int)(threadIdx.x % K::GROUP) - 64;      // the group's first two warps own no column
+  const int k = own >= 0 ? own / K::LPC : NC, q = own & (K::LPC - 1);
   const int64_t s0 = soff[c], s1 = soff[c + 1];
   const int64_t m = s1 - s0;
   for (int i = threadIdx.x; i < nc; i += blockDim.x) piv[i] = i;
   for (int i = threadIdx.x; i < NC * LD; i += blockDim.x) R[i] = 0.0;
+  if (threadIdx.x < K::NG) sm.g[threadIdx.x].done = 0;
+  if (threadIdx.x == 0) sm.late = 0;
   __syncthreads();
   int r = 0;
   if (m > 0 && nc > 0) {
     // ---- 2. tall-skinny QR of the sampled rows
-    double cc[SK_OWN];
+    double cc[K::OWN];
     double x[3] = {0.0, 0.0, 0.0}, wk = 0.0;
     if (k < nc) {
       const int p = cd[k];
       for (int d = 0; d < dim; ++d) x[d] = X[(int64_t)p * dim + d];
       wk = sw[p];
     }
-    for (int64_t row0 = 0; row0 < m; row0 += SK_CHUNK) {
-#pragma unroll 1
-      for (int t = 0; t < SK_OWN; ++t) {
-        const int64_t row = row0 + q + 4 * t;
-        double v = 0.0;
-        if (k < nc && row < m) {
-          const int f = samp[s0 + row];
-          v = sw[f] * kernel_eval(kp, X + (int64_t)f * dim, x, dim) * wk;
-        }
-        if (own >= 0) sm.stage[t * 4 * NC + own] = v;      // read back by this thread alone
-      }
+    double* stage = sm.g[group].stage + max(own, 0);
+    for (int64_t ch = group; ch * SK_CHUNK < m; ch += K::NG) {
+      const int64_t row0 = ch * SK_CHUNK + q;
 #pragma unroll
-      for (int t = 0; t < SK_OWN; ++t) cc[t] = own >= 0 ? sm.stage[t * 4 * NC + own] : 0.0;
-      fold_chunk<NC>(sm, nc, k, q, cc);
+      for (int f0 = 0; f0 < K::OWN; f0 += K::FILL) {
+#pragma unroll 1
+        for (int t = 0; t < K::FILL; ++t) {
+          const int64_t row = row0 + K::LPC * (f0 + t);
+          double v = 0.0;
+          if (k < nc && row < m) {
+            const int f = samp[s0 + row];
+            v = sw[f] * kernel_eval(kp, X + (int64_t)f * dim, x, dim) * wk;
+          }
+          if (own >= 0) stage[t * NC * K::LPC] = v;        // read back by this thread alone
+        }
+#pragma unroll
+        for (int t = 0; t < K::FILL; ++t) cc[f0 + t] = own >= 0 ? stage[t * NC * K::LPC] : 0.0;
+      }
+      fold_chunk<NC>(sm, nc, ch, group, k, q, cc);
     }
+    __syncthreads();
+    if (sm.late && threadIdx.x == 0) atomicExch(late, 1);
     // ---- 3. greedy column-pivoted Householder QR of R0 (rows: min(m, nc))
     const int rows = (int)(m < nc ? m : nc);
     const int kmax = min(rank_max, min(rows, nc));
@@ -404,8 +484,8 @@ static void skeletonize_level(Matrix& M, int ncl, const int* cand, const int* nc
                               const int64_t* soff, int* skel, int* rank, double* T) {
   const int smem = (int)sizeof(SkelSmem<NC>);
   H2_CUDA(cudaFuncSetAttribute(k_skeletonize<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  { k_skeletonize<NC><<<ncl, 4 * NC + 64, smem, M.stream>>>(cand, ncand, samp, soff, M.d_X, M.d_sw, M.dim, M.kp,
-                                                            M.basis_tol, M.k, skel, rank, T);
+  { k_skeletonize<NC><<<ncl, Skel<NC>::THREADS, smem, M.stream>>>(cand, ncand, samp, soff, M.d_X, M.d_sw, M.dim, M.kp,
+                                                                  M.basis_tol, M.k, skel, rank, T, M.d_flag + 2);
     ::h2mg::count_launch(); }
   H2_LAUNCH_CHECK();
 }
@@ -425,7 +505,7 @@ void build_skeletons(Matrix& M) {
   std::vector<int> ncand_h;                      // of level ell
   int* d_cand = (int*)M.alloc(sizeof(int) * ((size_t)1 << L) * SK_CAND);
   int* d_ncand = (int*)M.alloc(sizeof(int) * ((size_t)1 << L));
-  std::vector<int> partners_own, partners_par;
+  H2_CUDA(cudaMemsetAsync(M.d_flag + 2, 0, sizeof(int), s));
   for (int ell = L; ell >= ts; --ell) {
     const int ncl = 1 << ell;
     if (ell == L) {
@@ -485,7 +565,10 @@ void build_skeletons(Matrix& M) {
         (double*)M.tid.p + (size_t)M.slot0(ell) * SK_CAND * 64);
     H2_CUDA(cudaMemcpyAsync(M.h_rank.data() + M.slot0(ell), M.d_rank + M.slot0(ell), sizeof(int) * ncl,
                             cudaMemcpyDeviceToHost, s));
+    int late = 0;
+    H2_CUDA(cudaMemcpyAsync(&late, M.d_flag + 2, sizeof(int), cudaMemcpyDeviceToHost, s));
     H2_CUDA(cudaStreamSynchronize(s));
+    H2_REQUIRE(late == 0, H2MG_ERR_CUDA, "a skeletonization timed out waiting for its warps");
     M.free_owned(d_samp);
     M.free_owned(d_soff);
     M.free_owned(d_seg);
