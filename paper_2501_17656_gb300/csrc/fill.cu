@@ -552,13 +552,6 @@ __device__ __forceinline__ void store_block64(void* pool, int fmt, int64_t blk, 
       store_elem(pool, fmt, blk * FXT * FXT + swz(fx_a() + r, fx_b() + 16 * q, FXT, V), v[r][q]);
 }
 
-__device__ __forceinline__ void fx_values(const FxPair& t, const FxAcc& c, double (&v)[4][4]) {
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) v[r][q] = fx_value(t, c, r, q);
-}
-
 // Encodes a stored block (transposed where its reference says so) as operand P (row, k),
 // with exponents that cover the block of `O` too and one bit of headroom. Threads read the
 // pool in storage order.

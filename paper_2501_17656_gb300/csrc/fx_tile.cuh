@@ -141,4 +141,12 @@ __device__ __forceinline__ double fx_value(const FxPair& t, const FxAcc& c, int 
          fx_row_scale(t.eq[fx_b() + 16 * q]);
 }
 
+// All elements of this thread.
+__device__ __forceinline__ void fx_values(const FxPair& t, const FxAcc& c, double (&v)[4][4]) {
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[r][q] = fx_value(t, c, r, q);
+}
+
 }  // namespace h2mg
