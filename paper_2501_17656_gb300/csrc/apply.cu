@@ -194,19 +194,12 @@ constexpr int bsgemv_min_ctas() {
   return FMT == FMT_F32 ? (NR >= 4 ? 2 : (NR == 2 ? 3 : 4)) : 2;
 }
 
-// Asks the memory system to bring `bytes` (a multiple of 16, 16-byte aligned) from
-// global memory into L2 without waiting: the next block a warp will read streams in
-// while it works on the current one.
-__device__ __forceinline__ void prefetch_l2_bulk(const void* p, unsigned bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
 template <int K, int FMT, int NR>
 __global__ void __launch_bounds__(256, bsgemv_min_ctas<FMT, NR>()) k_bsgemv(const int* __restrict__ rowptr,
                                                 const int* __restrict__ col,
                                                 const void* const* __restrict__ blk,
-                                                const typename Ar<FMT>::vec_t* __restrict__ x,
-                                                typename Ar<FMT>::yo_t* __restrict__ yrow, int split) {
+                                                const typename Ar<FMT>::vec_t* x,
+                                                typename Ar<FMT>::yo_t* yrow, int split, bool first) {
   using A = Ar<FMT>;
   using vec_t = typename A::vec_t;
   using mel_t = typename A::mel_t;
@@ -222,6 +215,11 @@ __global__ void __launch_bounds__(256, bsgemv_min_ctas<FMT, NR>()) k_bsgemv(cons
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int row = blockIdx.x / split, part = blockIdx.x % split;
   const int rb = 8 * (lane % LPC), cl = lane / LPC;
+  const int e0 = rowptr[row], e1 = rowptr[row + 1];
+  constexpr unsigned kBlockBytes = K * K / V * (unsigned)sizeof(ld_t);   // one stored block
+  // the warp's first block, while the kernel before this one runs
+  if (first && lane == 0 && e0 + part * 8 + w < e1) prefetch_l2_bulk(blk[e0 + part * 8 + w], kBlockBytes);
+  chain_wait();
   for (int i = threadIdx.x; i < K * NR; i += blockDim.x) {
     const int r = i / NR;
     sxt[(r + r / 8) * NR + i % NR] = x[(int64_t)row * K * NR + i];
@@ -233,8 +231,6 @@ __global__ void __launch_bounds__(256, bsgemv_min_ctas<FMT, NR>()) k_bsgemv(cons
   for (int r = 0; r < 8; ++r)
 #pragma unroll
     for (int j = 0; j < NR; ++j) ya[r][j] = A::zero();
-  const int e0 = rowptr[row], e1 = rowptr[row + 1];
-  constexpr unsigned kBlockBytes = K * K / V * (unsigned)sizeof(ld_t);   // one stored block
   for (int e = e0 + part * 8 + w; e < e1; e += 8 * split) {
     const int s = col[e];
     const ld_t* B = (const ld_t*)blk[e];
@@ -336,8 +332,8 @@ __global__ void __launch_bounds__(256, bsgemv_min_ctas<FMT, NR>()) k_bsgemv(cons
 template <int K, int FMT, int NR>
 __global__ void __launch_bounds__(256) k_bsgemv_small(const int* __restrict__ erow, const int* __restrict__ col,
                                                       const void* const* __restrict__ blk,
-                                                      const typename Ar<FMT>::vec_t* __restrict__ x,
-                                                      typename Ar<FMT>::yo_t* __restrict__ yrow, int nnz, int per) {
+                                                      const typename Ar<FMT>::vec_t* x,
+                                                      typename Ar<FMT>::yo_t* yrow, int nnz, int per) {
   using A = Ar<FMT>;
   using vec_t = typename A::vec_t;
   using mel_t = typename A::mel_t;
@@ -349,6 +345,8 @@ __global__ void __launch_bounds__(256) k_bsgemv_small(const int* __restrict__ er
   const int rb = 8 * (lane % LPC), cl = lane / LPC;
   const int64_t e0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * per;
   const int e1 = (int)min(e0 + per, (int64_t)nnz);
+  if (lane == 0 && e0 < e1) prefetch_l2_bulk(blk[e0], K * K / V * (unsigned)sizeof(ld_t));
+  chain_wait();
   acc_t ya[8][NR];
   vec_t xt[8][NR];
   int row = -1;
@@ -483,7 +481,7 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 template <int K, int NR>
 __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
     k_bsgemv_fx(const int* __restrict__ erow, const int* __restrict__ col, const void* const* __restrict__ blk,
-                const short* __restrict__ bexp, const double* __restrict__ x, double* __restrict__ yrow,
+                const short* __restrict__ bexp, const double* x, double* yrow,
                 int64_t units, int per) {
   constexpr int LPC = K / 8, CPP = 32 / LPC, T = K * K / 256, CH = T < LPC ? T : LPC, NCH = T / CH;
   constexpr int XL = K * NR / 32;                // elements of x_s per lane
@@ -533,6 +531,7 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
   static_assert(CH % FX_RING == 0, "a unit starts at slot 0");
 #pragma unroll
   for (int tt = 0; tt < FX_RING - 1; ++tt) issue(cur, tt);
+  chain_wait();                                  // the first blocks are under way before it
 
   // adds the row sums of the lanes that share rows (32 / LPC of them) and stores them
   auto flush = [&]() {
@@ -807,9 +806,10 @@ __device__ __forceinline__ void clear_regions(const VecIn& in) {
 
 // coefficient vectors (KC per cluster) -> interleaved, for operators without transfers
 template <int FMT, int NR>
-__global__ void __launch_bounds__(256) k_coef_in(VecIn in, int64_t n, typename Ar<FMT>::vec_t* __restrict__ xc) {
+__global__ void __launch_bounds__(256) k_coef_in(VecIn in, int64_t n, typename Ar<FMT>::vec_t* xc) {
   bool go[NR];
   double be[NR];
+  chain_wait();
   cg_beta<NR>(in, go, be);
   clear_regions(in);
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256)
@@ -860,14 +860,16 @@ constexpr int LEAF_CTAS = CG_PARTS;   // the leaf kernels' grids: one partial pe
 template <int FMT, class BT, int NR>
 __global__ void __launch_bounds__(256) k_leaf_in(VecIn in, const BT* __restrict__ UT, int KD, int KC, int nleaf,
                                                  const int* __restrict__ leafoff, const int* __restrict__ perm,
-                                                 typename Ar<FMT>::vec_t* __restrict__ xp,
-                                                 typename Ar<FMT>::vec_t* __restrict__ xc) {
+                                                 typename Ar<FMT>::vec_t* xp,
+                                                 typename Ar<FMT>::vec_t* xc) {
   using V = LeafVal<FMT>;
   using v_t = typename V::t;
   __shared__ v_t xs[64 * NR];
   __shared__ v_t red[256 * NR];
   bool go[NR];
   double be[NR];
+  if (UT && threadIdx.x == 0) prefetch_l2_bulk(UT + (int64_t)blockIdx.x * KD * KC, KD * KC * (unsigned)sizeof(BT));
+  chain_wait();
   cg_beta<NR>(in, go, be);
   clear_regions(in);
   const int b = threadIdx.x % KC, part = threadIdx.x / KC, parts = 256 / KC;
@@ -1068,8 +1070,8 @@ __device__ __forceinline__ void warp_transfer(const void* __restrict__ Bv, const
 // between launches: the second arrival resets its own.
 template <int K, int FMT, int NR>
 __global__ void __launch_bounds__(256) k_up_tree(const char* __restrict__ epool, VecIn in,
-                                                 typename Ar<FMT>::vec_t* __restrict__ xc, int lb, int lt, int ts,
-                                                 unsigned* __restrict__ ticket) {
+                                                 typename Ar<FMT>::vec_t* xc, int lb, int lt, int ts,
+                                                 unsigned* ticket) {
   using A = Ar<FMT>;
   using vec_t = typename A::vec_t;
   using acc_t = typename A::acc_t;
@@ -1080,6 +1082,12 @@ __global__ void __launch_bounds__(256) k_up_tree(const char* __restrict__ epool,
   const int w = threadIdx.x >> 5;
   auto slot0 = [&](int l) { return (int64_t)((1 << l) - (1 << ts)); };
   int idx = blockIdx.x;                       // parent at level l - 1
+  if (threadIdx.x == 0)
+    for (int l = lb, i = idx; l > lt; --l, i >>= 1) {
+      prefetch_l2_bulk(epool + (size_t)(slot0(l) + 2 * (int64_t)i) * kBlk, 2 * (unsigned)kBlk);
+      if (i & 1) break;
+    }
+  chain_wait();
   vec_t* xb = xc + (slot0(lb) + 2 * (int64_t)idx) * K * NR;
   if (in.x) {
     bool go[NR];
@@ -1153,11 +1161,11 @@ __device__ __forceinline__ void column_partials(double v, double* __restrict__ p
 // else to yc.
 template <int K, int FMT, int NR, int S>
 __global__ void __launch_bounds__(256) k_down_tree(const char* __restrict__ epool,
-                                                   const typename Ar<FMT>::yo_t* __restrict__ yrow,
-                                                   const typename Ar<FMT>::vec_t* __restrict__ ypar,
-                                                   typename Ar<FMT>::vec_t* __restrict__ yc, int lt, int lb, int ts,
-                                                   double* __restrict__ yout, int64_t ldo,
-                                                   const double* __restrict__ pdot, double* __restrict__ part) {
+                                                   const typename Ar<FMT>::yo_t* yrow,
+                                                   const typename Ar<FMT>::vec_t* ypar,
+                                                   typename Ar<FMT>::vec_t* yc, int lt, int lb, int ts,
+                                                   double* yout, int64_t ldo,
+                                                   const double* pdot, double* part) {
   using A = Ar<FMT>;
   using vec_t = typename A::vec_t;
   using acc_t = typename A::acc_t;
@@ -1169,6 +1177,12 @@ __global__ void __launch_bounds__(256) k_down_tree(const char* __restrict__ epoo
   auto slot0 = [&](int l) { return (int64_t)((1 << l) - (1 << ts)); };
   double dot = 0.0;
   const int nb = 1 << lb;
+  if (threadIdx.x == 0)
+    for (int l = lb, c = blockIdx.x * S, n = min(S, nb); l >= max(lt, ts + 1); --l, c >>= 1, n = max(1, n >> 1)) {
+      prefetch_l2_bulk(epool + (size_t)(slot0(l) + c) * kBlk, n * (unsigned)kBlk);
+      if (n == 1 && (c & 1)) break;
+    }
+  chain_wait();
   for (int c0 = blockIdx.x * S; c0 < nb; c0 += gridDim.x * S)
     for (int l = lt; l <= lb; ++l) {
       const int first = c0 >> (lb - l);                            // clusters first .. first + per - 1
@@ -1235,18 +1249,20 @@ __global__ void k_swizzle_blocks(const double* __restrict__ in, int K, void* __r
 // each sum.
 template <int FMT, class BT, int NR>
 __global__ void __launch_bounds__(256) k_leaf_final(int KD, int KC, int nleaf,
-                                                    const typename Ar<FMT>::yo_t* __restrict__ yrow,
+                                                    const typename Ar<FMT>::yo_t* yrow,
                                                     const BT* __restrict__ U,
-                                                    const typename Ar<FMT>::vec_t* __restrict__ yleaf,
+                                                    const typename Ar<FMT>::vec_t* yleaf,
                                                     const int* __restrict__ leafoff, const int* __restrict__ perm,
-                                                    double* __restrict__ y, int64_t ldy,
-                                                    const double* __restrict__ pdot, double* __restrict__ part) {
+                                                    double* y, int64_t ldy,
+                                                    const double* pdot, double* part) {
   using V = LeafVal<FMT>;
   using v_t = typename V::t;
   __shared__ v_t ps[64 * NR];
   __shared__ v_t red[256 * NR];
   const int i = threadIdx.x % KD, pt = threadIdx.x / KD, parts = 256 / KD;
   double dot = 0.0;
+  if (U && threadIdx.x == 0) prefetch_l2_bulk(U + (int64_t)blockIdx.x * KD * KC, KD * KC * (unsigned)sizeof(BT));
+  chain_wait();
   for (int l = blockIdx.x; l < nleaf; l += gridDim.x) {
     const int p0 = leafoff[l], nl = leafoff[l + 1] - p0;
     if (U) {
@@ -1505,11 +1521,12 @@ static void launch_bsgemv_fx(const SymOp& op, const double* x, double* yrow, int
   const int per = (int)((units + warps - 1) / warps);
   const int grid = (int)((units + 8 * (int64_t)per - 1) / (8 * (int64_t)per));
   if (op.K == 64) {
-    k_bsgemv_fx<64, NR><<<grid, 256, fx_smem<64, NR>(), s>>>(op.erow, op.col, op.blk, op.bexp, x, yrow, units, per);
+    launch_chain(k_bsgemv_fx<64, NR>, grid, 256, fx_smem<64, NR>(), s, op.erow, op.col, op.blk, op.bexp, x, yrow, units,
+                 per);
   } else {
-    k_bsgemv_fx<32, NR><<<grid, 256, fx_smem<32, NR>(), s>>>(op.erow, op.col, op.blk, op.bexp, x, yrow, units, per);
+    launch_chain(k_bsgemv_fx<32, NR>, grid, 256, fx_smem<32, NR>(), s, op.erow, op.col, op.blk, op.bexp, x, yrow, units,
+                 per);
   }
-  ::h2mg::count_launch();
 }
 
 // Once per matrix (setup_operators): the kernels' dynamic shared memory.
@@ -1558,19 +1575,23 @@ static void launch_bsgemv(Matrix& M, const SymOp& op, bool f32, const void* x, v
   if (op.bexp && FMT == FMT_F64) {
   } else if (op.K == 64) {
     if constexpr (FMT != FMT_F64) {
-      k_bsgemv<64, FMT, NR><<<grid, 256, 0, s>>>(op.rowptr, op.col, blk, (const vt*)x, (yt*)yrow, split);
-      ::h2mg::count_launch();
+      // The warps' first blocks are asked for ahead (about 80 MB over the first wave of CTAs). One
+      // column: only where the previous kernel runs beside it, and not for operators of several
+      // times the L2, whose other blocks then miss it (level 2 of 30011 points, 0.9 GB: 6.53 ->
+      // 6.69 ms for 40 steps; 16384 points of a dense cube, 0.25 GB: 9.50 -> 8.86 ms a cycle).
+      const double bytes = (double)op.nnz * 4096 * (FMT == FMT_F32 ? 4 : 8);
+      const bool first = NR >= 2 || (bytes <= 512e6 && chained(s));
+      launch_chain(k_bsgemv<64, FMT, NR>, grid, 256, 0, s, op.rowptr, op.col, blk, (const vt*)x, (yt*)yrow, split, first);
     }
   } else if (op.nnz > 0) {
     const int64_t warps = (int64_t)(waves > 0 ? waves : FX_WAVES) * FX_SMS * 8;
     const int per = (int)((op.nnz + warps - 1) / warps);
     const int g = ceil_div(op.nnz, 8 * (int64_t)per);
     if (op.K == 16) {
-      k_bsgemv_small<16, FMT, NR><<<g, 256, 0, s>>>(op.erow, op.col, blk, (const vt*)x, (yt*)yrow, op.nnz, per);
+      launch_chain(k_bsgemv_small<16, FMT, NR>, g, 256, 0, s, op.erow, op.col, blk, (const vt*)x, (yt*)yrow, op.nnz, per);
     } else if constexpr (FMT != FMT_F64) {
-      k_bsgemv_small<32, FMT, NR><<<g, 256, 0, s>>>(op.erow, op.col, blk, (const vt*)x, (yt*)yrow, op.nnz, per);
+      launch_chain(k_bsgemv_small<32, FMT, NR>, g, 256, 0, s, op.erow, op.col, blk, (const vt*)x, (yt*)yrow, op.nnz, per);
     }
-    ::h2mg::count_launch();
   }
   H2_LAUNCH_CHECK();
   if (rec && P.cap_ev) {
@@ -1595,16 +1616,16 @@ static void pass_up(const Matrix& M, const char* epool, void* xc, int lb, int ts
   if (lb == ts) {
     if (!in) return;
     const int64_t n = (int64_t)(1 << lb) * KC;
-    { k_coef_in<FMT, NR><<<std::min(ceil_div(n, 256), 1024), 256, 0, s>>>(*in, n, x); ::h2mg::count_launch(); }
+    launch_chain(k_coef_in<FMT, NR>, std::min(ceil_div(n, 256), 1024), 256, 0, s, *in, n, x);
     H2_LAUNCH_CHECK();
     return;
   }
   const VecIn vi = in ? *in : VecIn{};
   const int grid = 1 << (lb - 1);
   switch (KC) {
-    case 16: { k_up_tree<16, FMT, NR><<<grid, 256, 0, s>>>(epool, vi, x, lb, ts, ts, ticket); ::h2mg::count_launch(); } break;
-    case 32: { k_up_tree<32, FMT, NR><<<grid, 256, 0, s>>>(epool, vi, x, lb, ts, ts, ticket); ::h2mg::count_launch(); } break;
-    default: { k_up_tree<64, FMT, NR><<<grid, 256, 0, s>>>(epool, vi, x, lb, ts, ts, ticket); ::h2mg::count_launch(); } break;
+    case 16: launch_chain(k_up_tree<16, FMT, NR>, grid, 256, 0, s, epool, vi, x, lb, ts, ts, ticket); break;
+    case 32: launch_chain(k_up_tree<32, FMT, NR>, grid, 256, 0, s, epool, vi, x, lb, ts, ts, ticket); break;
+    default: launch_chain(k_up_tree<64, FMT, NR>, grid, 256, 0, s, epool, vi, x, lb, ts, ts, ticket); break;
   }
   H2_LAUNCH_CHECK();
 }
@@ -1630,8 +1651,7 @@ static int pass_down(const Matrix& M, const char* epool, const void* yrow, void*
     const int S = (1 << lb) >= 4 * 152 ? 4 : 2;
     grid = std::min(std::max(1, (1 << lb) / S), CG_PARTS);
     auto go = [&](auto kernel) {
-      kernel<<<grid, 256, 0, s>>>(epool, (const yt*)yrow, ypar, (vt*)yc, lt, lb, ts, yo, ldo, pd, part);
-      ::h2mg::count_launch();
+      launch_chain(kernel, grid, 256, 0, s, epool, (const yt*)yrow, ypar, (vt*)yc, lt, lb, ts, yo, ldo, pd, part);
     };
     switch (KC) {
       case 16: S == 4 ? go(k_down_tree<16, FMT, NR, 4>) : go(k_down_tree<16, FMT, NR, 2>); break;
@@ -1689,8 +1709,8 @@ static int apply_impl(Matrix& M, int i, const double* x, int64_t ldx, double* y,
     in.zero[2] = (uint4*)ticket;
     in.nzero[2] = ts >= 0 ? ((int64_t)M.nslots() * sizeof(unsigned) + 15) / 16 : 0;
     const int grid = std::min(1 << L, LEAF_CTAS);
-    { k_leaf_in<FMT, BT, NR><<<grid, 256, 0, s>>>(in, ts >= 0 ? UT : nullptr, KD, KC, 1 << L, M.d_leafoff, M.d_perm, xp,
-                                                  ts >= 0 ? xc + cslot(L) : nullptr); ::h2mg::count_launch(); }
+    launch_chain(k_leaf_in<FMT, BT, NR>, grid, 256, 0, s, in, ts >= 0 ? UT : nullptr, KD, KC, 1 << L, M.d_leafoff, M.d_perm, xp,
+                                                  ts >= 0 ? xc + cslot(L) : nullptr);
     H2_LAUNCH_CHECK();
     if (ts >= 0) pass_up<FMT, NR>(M, epool, xc, L, ts, ticket, s);
     launch_bsgemv<FMT, NR>(M, M.opD, f32, xp, yp, s);
@@ -1698,10 +1718,9 @@ static int apply_impl(Matrix& M, int i, const double* x, int64_t ldx, double* y,
       launch_bsgemv<FMT, NR>(M, M.opC[1], f32, xc, yr, s);
       pass_down<FMT, NR>(M, epool, yr, yc, ts, L, nullptr, 0, nullptr, nullptr, s);
     }
-    { k_leaf_final<FMT, BT, NR><<<grid, 256, 0, s>>>(KD, KC, 1 << L, yp, ts >= 0 ? U : nullptr,
+    launch_chain(k_leaf_final<FMT, BT, NR>, grid, 256, 0, s, KD, KC, 1 << L, yp, ts >= 0 ? U : nullptr,
                                                      ts >= 0 ? yc + cslot(L) : nullptr, M.d_leafoff, M.d_perm, y, ldy,
                                                      pdot, part);
-      ::h2mg::count_launch(); }
     H2_LAUNCH_CHECK();
     return grid;
   }

@@ -205,4 +205,20 @@ __device__ __forceinline__ void dd_atomic_add(double2* p, double2 v) {
   atomicAdd(&p->y, err + v.y);
 }
 
+// First statement of a kernel launched by launch_chain, before it reads or writes anything
+// that another kernel of the stream writes or reads: waits until the kernel before it has
+// ended (which had waited for the one before that), then lets the next one be placed. Vectors
+// that kernels of the chain write are not __restrict__: the compiler may move loads through
+// such pointers ahead of the wait, or make them loads of constant memory.
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Asks the memory system to bring `bytes` (a multiple of 16, 16-byte aligned) from
+// global memory into L2 without waiting.
+__device__ __forceinline__ void prefetch_l2_bulk(const void* p, unsigned bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
 }  // namespace h2mg

@@ -343,8 +343,9 @@ __global__ void __launch_bounds__(256, 2) k_chol_inverse(const double* __restric
 }
 
 // e[i] = sum_j Ainv[j, i] r[j]: one warp per output, reading column i (contiguous).
-__global__ void k_symv_cols(const double* __restrict__ Ainv, int64_t n, const double* __restrict__ r,
-                            double* __restrict__ e) {
+__global__ void k_symv_cols(const double* __restrict__ Ainv, int64_t n, const double* r,
+                            double* e) {
+  chain_wait();
   int64_t i = (int64_t)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
   int lane = threadIdx.x & 31;
   if (i >= n) return;
@@ -358,8 +359,9 @@ __global__ void k_symv_cols(const double* __restrict__ Ainv, int64_t n, const do
 // E[:, c] = A^{-1} R[:, c] for NR columns (leading dimension n): one warp per output
 // row reads that column of the symmetric inverse once for all NR right-hand sides.
 template <int NR>
-__global__ void k_symv_multi(const double* __restrict__ Ainv, int64_t n, const double* __restrict__ r,
-                             double* __restrict__ e) {
+__global__ void k_symv_multi(const double* __restrict__ Ainv, int64_t n, const double* r,
+                             double* e) {
+  chain_wait();
   int64_t i = (int64_t)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
   int lane = threadIdx.x & 31;
   if (i >= n) return;
@@ -544,7 +546,7 @@ void coarse_solve(Matrix& M, const double* r, double* e, cudaStream_t s) {
     H2_CUDA(cudaMemcpyAsync(w, r, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
     rin = w;
   }
-  { k_symv_cols<<<ceil_div(n, 8), 256, 0, s>>>(M.d_Ainv, n, rin, eout); ::h2mg::count_launch(); }
+  launch_chain(k_symv_cols, ceil_div(n, 8), 256, 0, s, M.d_Ainv, n, rin, eout);
   H2_LAUNCH_CHECK();
   if (M.lev == 1) {
     { k_from_slots<<<ceil_div(M.n, 256), 256, 0, s>>>(x, M.d_slot_of, M.n, e); ::h2mg::count_launch(); }
@@ -562,10 +564,10 @@ void coarse_solve_multi(Matrix& M, const double* r, double* e, int nr, cudaStrea
   }
   const int g = ceil_div(n, 8);
   switch (nr) {
-    case 1: { k_symv_multi<1><<<g, 256, 0, s>>>(M.d_Ainv, n, r, e); ::h2mg::count_launch(); } break;
-    case 2: { k_symv_multi<2><<<g, 256, 0, s>>>(M.d_Ainv, n, r, e); ::h2mg::count_launch(); } break;
-    case 3: { k_symv_multi<3><<<g, 256, 0, s>>>(M.d_Ainv, n, r, e); ::h2mg::count_launch(); } break;
-    case 4: { k_symv_multi<4><<<g, 256, 0, s>>>(M.d_Ainv, n, r, e); ::h2mg::count_launch(); } break;
+    case 1: launch_chain(k_symv_multi<1>, g, 256, 0, s, M.d_Ainv, n, r, e); break;
+    case 2: launch_chain(k_symv_multi<2>, g, 256, 0, s, M.d_Ainv, n, r, e); break;
+    case 3: launch_chain(k_symv_multi<3>, g, 256, 0, s, M.d_Ainv, n, r, e); break;
+    case 4: launch_chain(k_symv_multi<4>, g, 256, 0, s, M.d_Ainv, n, r, e); break;
     default: throw Error{H2MG_ERR_INVALID_ARG, "too many columns for one coarse solve"};
   }
   H2_LAUNCH_CHECK();

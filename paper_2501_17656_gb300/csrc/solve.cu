@@ -30,8 +30,8 @@ __device__ double block_reduce_sum(double v) {
 }
 
 // part[col * NPART + block] = partial of a_col^T b_col (column = blockIdx.y)
-__global__ void k_dot_part(const double* __restrict__ a, const double* __restrict__ b, int64_t n, int64_t ld,
-                           double* __restrict__ part) {
+__global__ void k_dot_part(const double* a, const double* b, int64_t n, int64_t ld, double* part) {
+  chain_wait();
   const double* ac = a + blockIdx.y * ld;
   const double* bc = b + blockIdx.y * ld;
   double s = 0.0;
@@ -44,7 +44,7 @@ __global__ void k_dot_part(const double* __restrict__ a, const double* __restric
 static int part_grid(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>(NPART, (n + 1023) / 1024)); }
 
 // Sum of np partials, by every CTA (blockDim 256).
-__device__ double cta_sum_parts(const double* __restrict__ part, int np) {
+__device__ double cta_sum_parts(const double* part, int np) {
   __shared__ double sh[8];
   double v = 0.0;
   for (int i = threadIdx.x; i < np; i += 256) v += part[i];
@@ -58,10 +58,9 @@ __device__ double cta_sum_parts(const double* __restrict__ part, int np) {
 }
 
 // Start of a CG: r = f - q (q null: r = f, and x = 0), p = r, partials of r^T r and f^T f.
-__global__ void __launch_bounds__(256) k_cg_start(const double* __restrict__ f, const double* __restrict__ q,
-                                                  int64_t n, double* __restrict__ x, double* __restrict__ r,
-                                                  double* __restrict__ p, double* __restrict__ prr,
-                                                  double* __restrict__ pff) {
+__global__ void __launch_bounds__(256) k_cg_start(const double* f, const double* q, int64_t n, double* x,
+                                                  double* r, double* p, double* prr, double* pff) {
+  chain_wait();
   const int64_t c = blockIdx.y * n;
   double rr = 0.0, ff = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
@@ -81,8 +80,9 @@ __global__ void __launch_bounds__(256) k_cg_start(const double* __restrict__ f, 
 }
 
 // per column (CTA c): rho = r.r, thresh = (1e-30 |f|)^2
-__global__ void __launch_bounds__(256) k_cg_init(const double* __restrict__ prr, const double* __restrict__ pff,
+__global__ void __launch_bounds__(256) k_cg_init(const double* prr, const double* pff,
                                                  int np, CGState* st) {
+  chain_wait();
   const int c = blockIdx.x;
   const double rr = cta_sum_parts(prr + c * CG_PARTS, np), ff = cta_sum_parts(pff + c * CG_PARTS, np);
   if (threadIdx.x == 0) {
@@ -97,10 +97,11 @@ __global__ void __launch_bounds__(256) k_cg_init(const double* __restrict__ prr,
 // r -= alpha q; partials of r^T r. Every CTA of a column (blockIdx.y) takes the same
 // decision from the same partials. The new direction p = r + (rho' / rho) p is formed by the
 // next step's product (VecIn in apply.cu).
-__global__ void __launch_bounds__(256) k_cg_update(double* __restrict__ x, double* __restrict__ r,
-                                                   const double* __restrict__ p, const double* __restrict__ q,
-                                                   int64_t n, CGState* st, const double* __restrict__ ppq, int np,
-                                                   int par, double* __restrict__ part) {
+__global__ void __launch_bounds__(256) k_cg_update(double* x, double* r,
+                                                   const double* p, const double* q,
+                                                   int64_t n, CGState* st, const double* ppq, int np,
+                                                   int par, double* part) {
+  chain_wait();
   const int c = blockIdx.y;
   x += c * n;
   r += c * n;
@@ -142,8 +143,9 @@ __global__ void __launch_bounds__(256) k_cg_update(double* __restrict__ x, doubl
 }
 
 // y_c += a[c] x_c for every column c = blockIdx.y (a in device memory)
-__global__ void k_axpy_cols(const double* __restrict__ a, const double* __restrict__ x, double* __restrict__ y,
+__global__ void k_axpy_cols(const double* a, const double* x, double* y,
                             int64_t n, int64_t ld) {
+  chain_wait();
   const int c = blockIdx.y;
   const double al = a[c];
   x += c * ld;
@@ -152,8 +154,9 @@ __global__ void k_axpy_cols(const double* __restrict__ a, const double* __restri
     y[i] = fma(al, x[i], y[i]);
 }
 // y_c = x_c + b[c] y_c for every column c = blockIdx.y (b in device memory)
-__global__ void k_xpby_cols(const double* __restrict__ b, const double* __restrict__ x, double* __restrict__ y,
+__global__ void k_xpby_cols(const double* b, const double* x, double* y,
                             int64_t n, int64_t ld) {
+  chain_wait();
   const int c = blockIdx.y;
   const double be = b[c];
   x += c * ld;
@@ -162,12 +165,14 @@ __global__ void k_xpby_cols(const double* __restrict__ b, const double* __restri
     y[i] = fma(be, y[i], x[i]);
 }
 // z = x - y
-__global__ void k_sub(const double* __restrict__ x, const double* __restrict__ y, double* __restrict__ z, int64_t n) {
+__global__ void k_sub(const double* x, const double* y, double* z, int64_t n) {
+  chain_wait();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     z[i] = x[i] - y[i];
 }
 // z = x + y
-__global__ void k_add(const double* __restrict__ x, const double* __restrict__ y, double* __restrict__ z, int64_t n) {
+__global__ void k_add(const double* x, const double* y, double* z, int64_t n) {
+  chain_wait();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     z[i] = x[i] + y[i];
 }
@@ -177,9 +182,10 @@ static int vec_grid(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64
 // ----------------------------------------------------------------------------- transfers
 // Column blockIdx.y of each: input leading dimension ldv / lde, output ldo / ldv.
 // out[j*KC + b] = sum_i U_j[i, b] v[perm[leafoff[j] + i]]
-__global__ void k_restrict_leaf(const double* __restrict__ UT, int KD, int KC, const double* __restrict__ v,
+__global__ void k_restrict_leaf(const double* __restrict__ UT, int KD, int KC, const double* v,
                                 int64_t ldv, const int* __restrict__ leafoff, const int* __restrict__ perm,
-                                double* __restrict__ out, int64_t ldo) {
+                                double* out, int64_t ldo) {
+  chain_wait();
   __shared__ double xs[64];
   v += blockIdx.y * ldv;
   out += blockIdx.y * ldo;
@@ -195,9 +201,10 @@ __global__ void k_restrict_leaf(const double* __restrict__ UT, int KD, int KC, c
   }
 }
 // v[perm[...]] += sum_b U_j[i, b] e[j*KC + b]
-__global__ void k_prolong_leaf(const double* __restrict__ U, int KD, int KC, const double* __restrict__ e,
+__global__ void k_prolong_leaf(const double* __restrict__ U, int KD, int KC, const double* e,
                                int64_t lde, const int* __restrict__ leafoff, const int* __restrict__ perm,
-                               double* __restrict__ v, int64_t ldv) {
+                               double* v, int64_t ldv) {
+  chain_wait();
   __shared__ double es[64];
   e += blockIdx.y * lde;
   v += blockIdx.y * ldv;
@@ -213,8 +220,9 @@ __global__ void k_prolong_leaf(const double* __restrict__ U, int KD, int KC, con
   }
 }
 // out[p*KC + b] = sum_{c in children(p)} sum_a E'_c[a, b] v[c*KC + a]
-__global__ void k_restrict(const double* __restrict__ ET, int KC, const double* __restrict__ v, int64_t ldv,
-                           double* __restrict__ out, int64_t ldo) {
+__global__ void k_restrict(const double* __restrict__ ET, int KC, const double* v, int64_t ldv,
+                           double* out, int64_t ldo) {
+  chain_wait();
   __shared__ double xs[128];
   v += blockIdx.y * ldv;
   out += blockIdx.y * ldo;
@@ -231,8 +239,9 @@ __global__ void k_restrict(const double* __restrict__ ET, int KC, const double* 
   }
 }
 // v[c*KC + a] += sum_b E'_c[a, b] e[parent*KC + b]
-__global__ void k_prolong(const double* __restrict__ E, int KC, const double* __restrict__ e, int64_t lde,
-                          double* __restrict__ v, int64_t ldv) {
+__global__ void k_prolong(const double* __restrict__ E, int KC, const double* e, int64_t lde,
+                          double* v, int64_t ldv) {
+  chain_wait();
   __shared__ double es[64];
   e += blockIdx.y * lde;
   v += blockIdx.y * ldv;
@@ -301,7 +310,7 @@ void alloc_solve_workspace(Matrix& M) { work(M); }
 
 static void dot_part(const double* a, const double* b, int64_t n, int64_t ld, int nr, double* part,
                      cudaStream_t s) {
-  { k_dot_part<<<dim3(part_grid(n), nr), 256, 0, s>>>(a, b, n, ld, part); ::h2mg::count_launch(); }
+  launch_chain(k_dot_part, dim3(part_grid(n), nr), 256, 0, s, a, b, n, ld, part);
   H2_LAUNCH_CHECK();
 }
 
@@ -309,7 +318,8 @@ static void dot_part(const double* a, const double* b, int64_t n, int64_t ld, in
 // the product's first kernel forms the direction and its last one the partials of p^T q.
 // Nine or ten launches, with vectors converted, cleared and reduced in kernels of their own,
 // took 196 us per step on level 2 of 30011 points in the cube (FP32; the blocks alone 128)
-// and 87 us on the 1024 unknowns of level 2 of 4096 points (F64); now 165 and 29.
+// and 87 us on the 1024 unknowns of level 2 of 4096 points (F64); now 163 and 29, and less
+// where the launches overlap (launch_chain: a V-cycle of the 4096 points 979 -> 779 us).
 //
 // n CG iterations on A_i X = F from X0 (nullptr: zero) for nr columns of length N_i.
 // X receives the iterates; R (if not null) the recurrence residuals. Hestenes-Stiefel
@@ -332,16 +342,16 @@ void smooth_multi(Matrix& M, int i, bool f32, const double* f, const double* x0,
   }
   // one element per thread where the vector is short: the steps are latency, not bandwidth
   const int g = (int)std::max<int64_t>(1, std::min<int64_t>(2 * 152, (N + 255) / 256));
-  { k_cg_start<<<dim3(g, nr), 256, 0, s>>>(f, q0, N, x, rr, W.cp, W.pb, W.pa); ::h2mg::count_launch(); }
+  launch_chain(k_cg_start, dim3(g, nr), 256, 0, s, f, q0, N, x, rr, W.cp, W.pb, W.pa);
   H2_LAUNCH_CHECK();
   if (n == 0) return;
-  { k_cg_init<<<nr, 256, 0, s>>>(W.pb, W.pa, g, W.st); ::h2mg::count_launch(); }
+  launch_chain(k_cg_init, nr, 256, 0, s, W.pb, W.pa, g, W.st);
   H2_LAUNCH_CHECK();
   for (int it = 0; it < n; ++it) {
     // the direction of step `it` comes from step it - 1's residual: rho' and rho there
     const CgStep cg{it > 0 ? rr : nullptr, W.pb, g, (it - 1) & 1, W.st, W.pa};
     const int np = apply_cg_step(M, i, f32, W.cp, W.cq, N, nr, cg, s);
-    { k_cg_update<<<dim3(g, nr), 256, 0, s>>>(x, rr, W.cp, W.cq, N, W.st, W.pa, np, it & 1, W.pb); ::h2mg::count_launch(); }
+    launch_chain(k_cg_update, dim3(g, nr), 256, 0, s, x, rr, W.cp, W.cq, N, W.st, W.pa, np, it & 1, W.pb);
     H2_LAUNCH_CHECK();
   }
 }
@@ -355,12 +365,10 @@ static void restrict_multi(Matrix& M, int i, const double* v, double* out, int n
   const int KC = M.KC, KD = M.KD, L = M.L;
   const int64_t nf = level_size(M, i), nc = level_size(M, i + 1);
   if (i == 1) {
-    { k_restrict_leaf<<<dim3(1 << L, nr), std::max(KC, 32), 0, s>>>(M.d_UT, KD, KC, v, nf, M.d_leafoff, M.d_perm,
-                                                                    out, nc); ::h2mg::count_launch(); }
+    launch_chain(k_restrict_leaf, dim3(1 << L, nr), std::max(KC, 32), 0, s, M.d_UT, KD, KC, v, nf, M.d_leafoff, M.d_perm, out, nc);
   } else {
     int m = L - i + 2;
-    { k_restrict<<<dim3(1 << (m - 1), nr), std::max(KC, 32), 0, s>>>(M.d_ET + (size_t)M.slot0(m) * KC * KC, KC, v,
-                                                                     nf, out, nc); ::h2mg::count_launch(); }
+    launch_chain(k_restrict, dim3(1 << (m - 1), nr), std::max(KC, 32), 0, s, M.d_ET + (size_t)M.slot0(m) * KC * KC, KC, v, nf, out, nc);
   }
   H2_LAUNCH_CHECK();
 }
@@ -369,12 +377,10 @@ static void prolong_add_multi(Matrix& M, int i, const double* e, double* out, in
   const int KC = M.KC, KD = M.KD, L = M.L;
   const int64_t nf = level_size(M, i), nc = level_size(M, i + 1);
   if (i == 1) {
-    { k_prolong_leaf<<<dim3(1 << L, nr), std::max(KD, 32), 0, s>>>(M.d_U, KD, KC, e, nc, M.d_leafoff, M.d_perm,
-                                                                   out, nf); ::h2mg::count_launch(); }
+    launch_chain(k_prolong_leaf, dim3(1 << L, nr), std::max(KD, 32), 0, s, M.d_U, KD, KC, e, nc, M.d_leafoff, M.d_perm, out, nf);
   } else {
     int m = L - i + 2;
-    { k_prolong<<<dim3(1 << m, nr), std::max(KC, 32), 0, s>>>(M.d_E + (size_t)M.slot0(m) * KC * KC, KC, e, nc,
-                                                              out, nf); ::h2mg::count_launch(); }
+    launch_chain(k_prolong, dim3(1 << m, nr), std::max(KC, 32), 0, s, M.d_E + (size_t)M.slot0(m) * KC * KC, KC, e, nc, out, nf);
   }
   H2_LAUNCH_CHECK();
 }
@@ -428,7 +434,7 @@ static void cycle_visit(Matrix& M, const h2mg_solve_opts& o, int i, const double
   smooth_multi(M, i, f32, f, from_zero ? nullptr : W.et[i], ni, W.et[i], W.cr, nr, s);   // e~_i = Iter(A_i, r_i, .)
   if (o.explicit_restrict_residual) {                                // r_i - A_i e~_i, explicitly
     apply_level_multi(M, i, f32, W.et[i], N, W.cq, N, nr, s);
-    { k_sub<<<vec_grid(N * nr), 256, 0, s>>>(f, W.cq, W.cr, N * nr); ::h2mg::count_launch(); }
+    launch_chain(k_sub, vec_grid(N * nr), 256, 0, s, f, W.cq, W.cr, N * nr);
     H2_LAUNCH_CHECK();
   }
   restrict_multi(M, i, W.cr, W.r[i + 1], nr, s);                     // r_{i+1} = U_i^T (r_i - A_i e~_i)
@@ -454,7 +460,7 @@ void vcycle_multi(Matrix& M, const h2mg_solve_opts& o, const double* x0, const d
   Work W = work(M);
   vcycle_core(M, o, r1, nr, s);
   const int64_t n1 = M.n;
-  { k_add<<<vec_grid(n1 * nr), 256, 0, s>>>(x0, W.et[1], xout, n1 * nr); ::h2mg::count_launch(); }   // x* = x0 + e_1
+  launch_chain(k_add, vec_grid(n1 * nr), 256, 0, s, x0, W.et[1], xout, n1 * nr);   // x* = x0 + e_1
   H2_LAUNCH_CHECK();
 }
 
@@ -608,8 +614,9 @@ static void vcycle_solve_step(Matrix& M, const h2mg_solve_opts& o, int nr, cudaS
 }
 
 // out[c] = sum of the np partials of column c (blockIdx.x), in a fixed order.
-__global__ void __launch_bounds__(256) k_sum_parts(const double* __restrict__ part, int np,
-                                                   double* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_sum_parts(const double* part, int np,
+                                                   double* out) {
+  chain_wait();
   const double t = cta_sum_parts(part + blockIdx.x * NPART, np);
   if (threadIdx.x == 0) out[blockIdx.x] = t;
 }
@@ -630,7 +637,7 @@ double device_dot(const double* a, const double* b, int64_t n, cudaStream_t s) {
   if (!g_dot_ws[dev]) H2_CUDA(cudaMalloc(&g_dot_ws[dev], sizeof(double) * (NPART + 32)));
   double* part = g_dot_ws[dev];
   dot_part(a, b, n, n, 1, part, s);
-  { k_sum_parts<<<1, 256, 0, s>>>(part, part_grid(n), part + NPART); ::h2mg::count_launch(); }
+  launch_chain(k_sum_parts, 1, 256, 0, s, part, part_grid(n), part + NPART);
   H2_LAUNCH_CHECK();
   double t = 0.0;
   H2_CUDA(cudaMemcpyAsync(&t, part + NPART, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -643,7 +650,7 @@ double device_dot(const double* a, const double* b, int64_t n, cudaStream_t s) {
 static void dots_host(Matrix& M, const double* a, const double* b, int64_t n, int nr, double* out, cudaStream_t s) {
   Work W = work(M);
   dot_part(a, b, n, n, nr, W.pa, s);
-  { k_sum_parts<<<nr, 256, 0, s>>>(W.pa, part_grid(n), W.scal + 4 * NRMAX); ::h2mg::count_launch(); }
+  launch_chain(k_sum_parts, nr, 256, 0, s, W.pa, part_grid(n), W.scal + 4 * NRMAX);
   H2_LAUNCH_CHECK();
   H2_CUDA(cudaMemcpyAsync(out, W.scal + 4 * NRMAX, sizeof(double) * nr, cudaMemcpyDeviceToHost, s));
   H2_CUDA(cudaStreamSynchronize(s));
@@ -659,7 +666,7 @@ static void axpy_cols(Matrix& M, const double* alpha, const double* x, double* y
                       cudaStream_t s) {
   Work W = work(M);
   H2_CUDA(cudaMemcpyAsync(W.scal, alpha, sizeof(double) * nr, cudaMemcpyHostToDevice, s));
-  { k_axpy_cols<<<dim3(vec_grid(n), nr), 256, 0, s>>>(W.scal, x, y, n, n); ::h2mg::count_launch(); }
+  launch_chain(k_axpy_cols, dim3(vec_grid(n), nr), 256, 0, s, W.scal, x, y, n, n);
   H2_LAUNCH_CHECK();
 }
 
@@ -680,7 +687,7 @@ static void outer_residual(Matrix& M, const h2mg_solve_opts& o, const double* b,
     for (int c = 0; c < nr; ++c)
       if (M.fmt == FMT_F64 && (o.residual_dd == 1 || (o.residual_dd == 2 && dd && dd[c])))
         apply_level1_dd(M, x + c * n, tmp + c * n, s);
-  { k_sub<<<vec_grid(n * nr), 256, 0, s>>>(b, tmp, r, n * nr); ::h2mg::count_launch(); }
+  launch_chain(k_sub, vec_grid(n * nr), 256, 0, s, b, tmp, r, n * nr);
   H2_LAUNCH_CHECK();
 }
 
@@ -688,7 +695,7 @@ static void outer_residual(Matrix& M, const h2mg_solve_opts& o, const double* b,
 static void xpby_cols(Matrix& M, const double* beta, const double* x, double* y, int64_t n, int nr, cudaStream_t s) {
   Work W = work(M);
   H2_CUDA(cudaMemcpyAsync(W.scal + NRMAX, beta, sizeof(double) * nr, cudaMemcpyHostToDevice, s));
-  { k_xpby_cols<<<dim3(vec_grid(n), nr), 256, 0, s>>>(W.scal + NRMAX, x, y, n, n); ::h2mg::count_launch(); }
+  launch_chain(k_xpby_cols, dim3(vec_grid(n), nr), 256, 0, s, W.scal + NRMAX, x, y, n, n);
   H2_LAUNCH_CHECK();
 }
 
@@ -716,7 +723,7 @@ static h2mg_status solve_cg_multi(Matrix& M, const double* b, double* x, int nr,
     info[c] = h2mg_solve_info{};
   }
   apply_level_multi(M, 1, false, x, n, W.t2, n, nr, s);
-  { k_sub<<<vec_grid(n * nr), 256, 0, s>>>(b, W.t2, r, n * nr); ::h2mg::count_launch(); }
+  launch_chain(k_sub, vec_grid(n * nr), 256, 0, s, b, W.t2, r, n * nr);
   H2_LAUNCH_CHECK();
   H2_CUDA(cudaMemcpyAsync(p, r, sizeof(double) * n * nr, cudaMemcpyDeviceToDevice, s));
   dots_host(M, r, r, n, nr, rho, s);
@@ -926,7 +933,7 @@ static void dots_many(const std::vector<Matrix*>& Ms, const std::vector<const do
     if (!want[p]) continue;
     Work W = work(*Ms[p]);
     dot_part(a[p], b[p], Ms[p]->n, Ms[p]->n, 1, W.pa, s);
-    { k_sum_parts<<<1, 256, 0, s>>>(W.pa, part_grid(Ms[p]->n), W.scal + 4 * NRMAX); ::h2mg::count_launch(); }
+    launch_chain(k_sum_parts, 1, 256, 0, s, W.pa, part_grid(Ms[p]->n), W.scal + 4 * NRMAX);
     H2_LAUNCH_CHECK();
     H2_CUDA(cudaMemcpyAsync(hp.h + p, W.scal + 4 * NRMAX, sizeof(double), cudaMemcpyDeviceToHost, s));
   }
