@@ -11,7 +11,8 @@
 // K x K blocks (swizzled so that every warp load is one contiguous 512 B segment),
 // and each block is used twice -- y_t += B x_s for its row and, for s != t, the
 // transposed product B^T x_t for its column, both added atomically into a zeroed row
-// buffer. The upward pass (k_leaf_in, k_up_tree) forms the cluster coefficients of
+// buffer. Float64 blocks of 32 and 64 go through k_bsgemv_fx (fixed point on the integer
+// pipe), smaller blocks through k_bsgemv_small; these deal entries to warps. The upward pass (k_leaf_in, k_up_tree) forms the cluster coefficients of
 // every level; the downward pass (k_down_tree) adds the transfer from the parent to
 // each level's row results and writes the finest level out (k_leaf_final at i = 1).
 //
