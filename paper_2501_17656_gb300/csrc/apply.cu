@@ -12,11 +12,12 @@
 // and each block is used twice -- y_t += B x_s for its row and, for s != t, the
 // transposed product B^T x_t for its column, both added atomically into a zeroed row
 // buffer. Float64 blocks of 32 and 64 go through k_bsgemv_fx (fixed point on the integer
-// pipe), smaller blocks through k_bsgemv_small; these deal entries to warps. The upward pass (k_leaf_in, k_up_tree) forms the cluster coefficients of
-// every level; the downward pass (k_down_tree) adds the transfer from the parent to
-// each level's row results and writes the finest level out (k_leaf_final at i = 1).
+// pipe), smaller blocks through k_bsgemv_small; these deal entries to warps. The upward pass
+// (k_leaf_in, k_up_tree) forms the cluster coefficients of every level; the downward pass
+// (k_down_tree) adds the transfer from the parent to each level's row results and writes the
+// finest level out (k_leaf_final at i = 1).
 //
-// Arithmetic per block format: F64 (DFMA), DF (double-float on the FP32 pipes: the
+// Arithmetic per block format: F64 (fixed point, DFMA where it does not serve), DF (double-float on the FP32 pipes: the
 // error-free products/sums of Dekker and Knuth), F32 (FP32 FMA). Vectors inside the
 // product are in the same format; the multigrid vectors outside are float64.
 #include <algorithm>
