@@ -139,8 +139,8 @@ struct Matrix {
 
   // ---- dense coarsest operator and Cholesky factor
   int nl = 0;                   // size of A_l
-  double* d_Al = nullptr;       // [nl * nl] column-major: A_l until it is factored
-  double* d_Ainv = nullptr;     // [nl * nl] A_l^{-1} formed from the factor (A_l's memory)
+  double* d_Al = nullptr;       // [nl * nl] A_l, column-major
+  double* d_Ainv = nullptr;     // [nl * nl] A_l^{-1} formed from the factor
   bool coarse_ok = false;
 
   // ---- workspaces
@@ -149,7 +149,7 @@ struct Matrix {
   DevBuf wstage;                // host staging
   DevBuf wvec;                  // multigrid vectors (float64)
   DevBuf wred;                  // reduction partials + scalars
-  DevBuf wcoarse;               // three vectors of the coarse size (triangular solves)
+  DevBuf wcoarse;               // 2 + NRMAX vectors of the coarse size
   DevBuf wfcg;                  // five point vectors of the flexible-CG outer loop
   int* d_flag = nullptr;        // device error flags
   unsigned* d_ticket = nullptr; // upward pass: arrivals per pair of clusters (slots), zero between launches
