@@ -1550,7 +1550,9 @@ static void launch_bsgemv(Matrix& M, const SymOp& op, bool f32, const void* x, v
   if (op.nrows == 0) return;
   // CTAs per block row: the autotuner's choice, else enough CTAs to fill the GPU when
   // the operator has few block rows
-  const int tuned = op.split[FMT == FMT_DD ? FMT_F64 : FMT][nr_index(NR)];
+  // the double-double product has no tuned value: the float64 one counts CTAs per SM
+  int tuned = 0;
+  if constexpr (FMT != FMT_DD) tuned = op.split[FMT][nr_index(NR)];
   const int waves = force_split > 0 ? force_split : tuned;   // CTAs per SM of the kernels that take warps by entry
   const int split = waves > 0 ? waves : split_heuristic(op.nrows);
   const int grid = op.nrows * split;
