@@ -549,6 +549,24 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
       }
   };
 
+  // z[.][j]: this lane's part of the CH column sums of chunk ch, block column s. Sums them over
+  // the LPC lanes that share a column; lane keeps column lane % CH
+  auto add_column = [&](auto& z, int j, int ch, int s, double scale) {
+#pragma unroll
+    for (int h = CH / 2; h >= 1; h >>= 1) {
+      const bool up = (lane & h) != 0;
+#pragma unroll
+      for (int q = 0; q < h; ++q) {
+        const auto send = up ? z[q][j] : z[q + h][j], keep = up ? z[q + h][j] : z[q][j];
+        z[q][j] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+      }
+    }
+#pragma unroll
+    for (int h = CH; h < LPC; h <<= 1) z[0][j] += __shfl_xor_sync(0xffffffffu, z[0][j], h);
+    if ((lane % LPC) < CH)
+      atomicAdd(yrow + ((int64_t)s * K + cl + CPP * (ch * CH + (lane & (CH - 1)))) * NR + j, (double)z[0][j] * scale);
+  };
+
   for (int64_t u = u0; u < u1;) {
     const int e = (int)(u / NCH);
     const int c0 = (int)(u % NCH), c1 = (int)min((int64_t)NCH, c0 + (u1 - u));
@@ -663,26 +681,9 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
 #pragma unroll
           for (int j = 0; j < NR; ++j) z[tt][j] = fx_join(zh[j], zm[j]);
         }
-        if (off) {
-          // sum over the LPC lanes that share a column; lane keeps column lane % CH
+        if (off)
 #pragma unroll
-          for (int j = 0; j < NR; ++j) {
-#pragma unroll
-            for (int h = CH / 2; h >= 1; h >>= 1) {
-              const bool up = (lane & h) != 0;
-#pragma unroll
-              for (int q = 0; q < h; ++q) {
-                const int64_t send = up ? z[q][j] : z[q + h][j], keep = up ? z[q + h][j] : z[q][j];
-                z[q][j] = keep + __shfl_xor_sync(0xffffffffu, send, h);
-              }
-            }
-#pragma unroll
-            for (int h = CH; h < LPC; h <<= 1) z[0][j] += __shfl_xor_sync(0xffffffffu, z[0][j], h);
-            if ((lane % LPC) < CH)
-              atomicAdd(yrow + ((int64_t)s * K + cl + CPP * (ch * CH + (lane & (CH - 1)))) * NR + j,
-                        (double)z[0][j] * sc[j]);
-          }
-        }
+          for (int j = 0; j < NR; ++j) add_column(z, j, ch, s, sc[j]);
         next_unit(uc++);
       }
 #pragma unroll
@@ -693,34 +694,47 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
           y = fma((double)fx_join(yh[r][j], ym[r][j]), sr[j], y);
         }
     } else {
-      // float64 arithmetic: blocks or vectors outside the range of fixed point
+      // Float64 arithmetic: blocks or vectors outside the range of fixed point. Bound by the
+      // float64 pipe like k_bsgemv, with sums in registers and column sums exchanged as above:
+      // all blocks of 65536 Gaussian points that way 1.90 ms (one column) and 3.80 ms (two),
+      // k_bsgemv 1.92 and 3.73; with row sums in shared memory and a sum over the lanes per
+      // column it was 2.12 and 4.21.
+      double y[8][NR], xr[8][NR];
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int j = 0; j < NR; ++j) {
+          y[r][j] = 0.0;
+          xr[r][j] = xrow[(rb + r) * NR + j];
+        }
 #pragma unroll 1
       for (int ch = c0; ch < c1; ++ch) {
+        double z[CH][NR];
 #pragma unroll
         for (int tt = 0; tt < CH; ++tt) {
-          const int p = ch * CH + tt;
           double2 d[4];
           take(tt, d);
           const double m[8] = {d[0].x, d[0].y, d[1].x, d[1].y, d[2].x, d[2].y, d[3].x, d[3].y};
 #pragma unroll
           for (int j = 0; j < NR; ++j) {
-            const double xv = xcol[(cl + CPP * p) * NR + j];
-            double z = 0.0;
+            const double xv = xcol[(cl + CPP * (ch * CH + tt)) * NR + j];
+            z[tt][j] = 0.0;
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
-              double& y = yad[r * NR + j][lane];
-              y = fma(m[r], xv, y);
-              z = fma(m[r], xrow[(rb + r) * NR + j], z);
-            }
-            if (off) {
-#pragma unroll
-              for (int h = 1; h < LPC; h <<= 1) z += __shfl_xor_sync(0xffffffffu, z, h);
-              if ((lane % LPC) == 0) atomicAdd(yrow + ((int64_t)s * K + cl + CPP * p) * NR + j, z);
+              y[r][j] = fma(m[r], xv, y[r][j]);
+              z[tt][j] = fma(m[r], xr[r][j], z[tt][j]);
             }
           }
         }
+        if (off)
+#pragma unroll
+          for (int j = 0; j < NR; ++j) add_column(z, j, ch, s, 1.0);
         next_unit(uc++);
       }
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int j = 0; j < NR; ++j) yad[r * NR + j][lane] += y[r][j];
     }
   }
   flush();
