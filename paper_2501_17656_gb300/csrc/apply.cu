@@ -442,22 +442,25 @@ __global__ void k_block_exponents(const void* const* __restrict__ blk, const int
   }
 }
 
-// Leaves whose diagonal entries |A_ii| differ by more than 2^12: their rows have natural
-// scales sqrt(A_ii) of their own (widely varying weights), which one exponent per block
-// would not carry, so their close blocks stay with the float64 path.
-__global__ void k_leaf_spread(const int* __restrict__ leafoff, const double* __restrict__ dg, int nleaf,
-                              unsigned char* __restrict__ skip) {
+// Smallest and largest exponents of the diagonal entries |A_ii| and of sqrt(w_i) of every leaf:
+// (dg, dg, sw, sw).
+__global__ void k_leaf_spread(const int* __restrict__ leafoff, const double* __restrict__ dg,
+                              const double* __restrict__ sw, int nleaf, short4* __restrict__ out) {
   const int l = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (l >= nleaf) return;
-  int lo = 4095, hi = 0;
+  int lo = 4095, hi = 0, slo = 4095, shi = 0;
   for (int p = leafoff[l] + lane; p < leafoff[l + 1]; p += 32) {
-    const int x = fx_exponent(dg[p]);
+    const int x = fx_exponent(dg[p]), s = fx_exponent(sw[p]);
     lo = min(lo, x);
     hi = max(hi, x);
+    slo = min(slo, s);
+    shi = max(shi, s);
   }
   lo = __reduce_min_sync(0xffffffffu, lo);
   hi = __reduce_max_sync(0xffffffffu, hi);
-  if (lane == 0) skip[l] = hi - lo > 12;
+  slo = __reduce_min_sync(0xffffffffu, slo);
+  shi = __reduce_max_sync(0xffffffffu, shi);
+  if (lane == 0) out[l] = make_short4((short)lo, (short)hi, (short)slo, (short)shi);
 }
 
 // The product of k_bsgemv for float64 blocks in fixed point (fixed.cuh). Every warp owns
@@ -1359,7 +1362,7 @@ static std::vector<int64_t> ubase(const HostCSR& C, int nrows, bool strict) {
 static bool fx_product(int fmt, int K) { return fmt == FMT_F64 && K >= 32; }
 
 static SymOp upload_op(Matrix& M, const OpHost& H, int K, const void* pool0, const void* pool1,
-                       const void* pool0_32, const void* pool1_32, const unsigned char* skip = nullptr) {
+                       const void* pool0_32, const void* pool1_32, const std::vector<unsigned char>& skip) {
   SymOp op;
   op.K = K;
   op.nrows = (int)H.rowptr.size() - 1;
@@ -1392,9 +1395,12 @@ static SymOp upload_op(Matrix& M, const OpHost& H, int K, const void* pool0, con
   op.erow = (int*)up(rowof.data(), sizeof(int) * rowof.size());
   if (fx_product(M.fmt, K) && op.nnz > 0) {
     op.bexp = (short*)M.alloc(sizeof(short) * op.nnz);
-    { k_block_exponents<<<ceil_div(op.nnz, 8), 256, 0, s>>>(op.blk, op.erow, op.col, skip, op.nnz, K * K, op.bexp);
+    unsigned char* d_skip = nullptr;
+    if (std::find(skip.begin(), skip.end(), 1) != skip.end()) d_skip = (unsigned char*)up(skip.data(), skip.size());
+    { k_block_exponents<<<ceil_div(op.nnz, 8), 256, 0, s>>>(op.blk, op.erow, op.col, d_skip, op.nnz, K * K, op.bexp);
       ::h2mg::count_launch(); }
     H2_LAUNCH_CHECK();
+    M.free_owned(d_skip);
   }
   H2_CUDA(cudaStreamSynchronize(s));   // the host lists go out of scope
   return op;
@@ -1431,6 +1437,47 @@ static OpHost coupling_rows(const Matrix& M, int top, int i) {
   return H;
 }
 
+// Rows have natural scales: sqrt(w_i) off the diagonal, sqrt(A_ii) on it. Where they differ by
+// more than 2^6 inside a cluster, one exponent per block or tile row would not carry the
+// digits of the small ones, so everything that touches the cluster stays in float64: the
+// close blocks of a leaf (either scale), and for the clusters of all levels (weights) the
+// couplings, the coarse near fields and the dense expansion, whose orthonormal bases are
+// then graded. Without the guard above the leaves, the middle row of a product with 3000
+// points, a far field and weights over 24 decades was off by 1.6e-12 of itself (float64:
+// 5.4e-16). The skeletons and bases themselves are made in float64. A sibling on its base's
+// bases (Chebyshev) takes over the base's marks.
+void mark_spread(Matrix& M, const Matrix* base) {
+  const int L = M.L, nleaf = 1 << L;
+  short4* d = (short4*)M.alloc(sizeof(short4) * nleaf);
+  { k_leaf_spread<<<ceil_div(nleaf, 8), 256, 0, M.stream>>>(M.d_leafoff, M.d_dg, M.d_sw, nleaf, d); ::h2mg::count_launch(); }
+  H2_LAUNCH_CHECK();
+  std::vector<short4> h(nleaf);
+  H2_CUDA(cudaMemcpyAsync(h.data(), d, sizeof(short4) * nleaf, cudaMemcpyDeviceToHost, M.stream));
+  H2_CUDA(cudaStreamSynchronize(M.stream));
+  M.free_owned(d);
+  constexpr int BITS = 6;
+  M.spread_leaf.assign(nleaf, 0);
+  for (int j = 0; j < nleaf; ++j) M.spread_leaf[j] = h[j].y - h[j].x > 2 * BITS || h[j].w - h[j].z > BITS;
+  if (base) {
+    M.spread_slot = base->spread_slot;
+    return;
+  }
+  M.spread_slot.assign(std::max(M.nslots(), 0), 0);
+  if (M.tstar < 0) return;
+  for (int ell = L; ell >= M.tstar; --ell) {
+    for (int j = 0; j < (1 << ell); ++j) M.spread_slot[M.slot0(ell) + j] = h[j].w - h[j].z > BITS;
+    for (int j = 0; j < (1 << ell) / 2; ++j) {
+      h[j].z = std::min(h[2 * j].z, h[2 * j + 1].z);
+      h[j].w = std::max(h[2 * j].w, h[2 * j + 1].w);
+    }
+  }
+}
+
+bool level_spread(const Matrix& M, int ell) {
+  const auto b = M.spread_slot.begin() + M.slot0(ell);
+  return std::find(b, b + (1 << ell), 1) != b + (1 << ell);
+}
+
 static void allow_fx_smem();
 
 void setup_operators(Matrix& M) {
@@ -1452,14 +1499,7 @@ void setup_operators(Matrix& M) {
         }
       H.rowptr.push_back((int)H.col.size());
     }
-    unsigned char* skip = nullptr;
-    if (fx_product(M.fmt, M.KD)) {
-      skip = (unsigned char*)M.alloc(1 << L);
-      { k_leaf_spread<<<ceil_div(1 << L, 8), 256, 0, s>>>(M.d_leafoff, M.d_dg, 1 << L, skip); ::h2mg::count_launch(); }
-      H2_LAUNCH_CHECK();
-    }
-    M.opD = upload_op(M, H, M.KD, M.poolD.p, nullptr, M.poolD32.p, nullptr, skip);
-    M.free_owned(skip);
+    M.opD = upload_op(M, H, M.KD, M.poolD.p, nullptr, M.poolD32.p, nullptr, M.spread_leaf);
   }
   M.opC.assign(M.lev + 1, SymOp{});
   if (M.tstar >= 0) {
@@ -1469,7 +1509,8 @@ void setup_operators(Matrix& M) {
       OpHost H = coupling_rows(M, top, i);
       const void* pP = (i >= 2) ? M.poolP[i].p : nullptr;
       const void* pP32 = (i >= 2 && M.with_f32) ? M.poolP32[i].p : nullptr;
-      M.opC[i] = upload_op(M, H, M.KC, M.poolS.p, pP, M.with_f32 ? M.poolS32.p : nullptr, pP32);
+      M.opC[i] = upload_op(M, H, M.KC, M.poolS.p, pP, M.with_f32 ? M.poolS32.p : nullptr, pP32,
+                            M.spread_slot);
     }
     // transposed copies of the transfers and leaf bases (coalesced upward pass) and the
     // swizzled transfer pools; a sibling matrix already has its base's

@@ -185,6 +185,7 @@ static void build_all(Matrix& M, const double* points, const h2mg_kernel* k, con
   H2_REQUIRE(M.lev >= 1 && M.lev <= M.lev_nat, H2MG_ERR_INVALID_ARG,
              "coarse_level must be -1 or in [1, " + std::to_string(M.lev_nat) + "]");
   if (M.apply_only) M.lev = std::min(M.lev, 1);
+  mark_spread(M, nullptr);
   build_bases(M);
   build_blocks(M, nullptr);
   if (!M.apply_only) build_coarse_near(M);
@@ -225,6 +226,7 @@ static void build_sibling(Matrix& B, const Matrix& A, const h2mg_kernel* k) {
   { k_point_weights<<<ceil_div(B.n, 256), 256, 0, s>>>(B.d_perm, B.n, B.dim, B.d_X, nullptr, nullptr, B.kp,
                                                        B.d_sw, B.d_dg); ::h2mg::count_launch(); }
   H2_LAUNCH_CHECK();
+  mark_spread(B, own_bases ? nullptr : &A);
   if (own_bases) build_bases(B);
   build_blocks(B, &A);
   setup_operators(B);

@@ -460,10 +460,11 @@ static void scatter_level(Matrix& M, const HostCSR& C, int ncl, bool strict, con
   H2_LAUNCH_CHECK();
 }
 
-// One step of the chain: every block of `out` from its block of G.
-static void expand(const double* G, int64_t ng, const double* B, int Ra, int C, int ncl, int shift, double* out,
-                   int64_t no, cudaStream_t s) {
-  if (Ra == FXT && C == FXT) {
+// One step of the chain: every block of `out` from its block of G. `spread`: clusters whose
+// rows have widely different scales are among them (mark_spread).
+static void expand(const double* G, int64_t ng, const double* B, int Ra, int C, int ncl, int shift, bool spread,
+                   double* out, int64_t no, cudaStream_t s) {
+  if (Ra == FXT && C == FXT && !spread) {
     H2_CUDA(cudaFuncSetAttribute(k_expand64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DENSE_SMEM));
     { k_expand64<<<ncl * (ncl + 1) / 2, 256, DENSE_SMEM, s>>>(G, ng, B, shift, out, no); ::h2mg::count_launch(); }
   } else {
@@ -490,7 +491,8 @@ void build_dense_coarse(Matrix& M) {
       int64_t nn = (int64_t)(1 << (ell + 1)) * KC;
       double* G2 = (double*)M.alloc(sizeof(double) * nn * nn);
       int ncl = 1 << (ell + 1);
-      expand(G, ng, M.d_E + (size_t)M.slot0(ell + 1) * KC * KC, KC, KC, ncl, 1, G2, nn, s);
+      expand(G, ng, M.d_E + (size_t)M.slot0(ell + 1) * KC * KC, KC, KC, ncl, 1,
+             level_spread(M, ell) || level_spread(M, ell + 1), G2, nn, s);
       scatter_level(M, M.far[ell + 1], ncl, true, M.poolS.p, M.s_level_base[ell + 1], KC, G2, nn);
       H2_CUDA(cudaStreamSynchronize(s));
       cudaFree(G);   // intermediate levels are released right away
@@ -517,7 +519,7 @@ void build_dense_coarse(Matrix& M) {
     double* A1 = (double*)M.alloc(sizeof(double) * np * np);
     if (M.tstar >= 0) {
       int ncl = 1 << L;
-      expand(G, ng, M.d_U, KD, KC, ncl, 0, A1, np, s);
+      expand(G, ng, M.d_U, KD, KC, ncl, 0, level_spread(M, L), A1, np, s);
     }
     M.nl = (int)np;
     valid.assign(np, 0);

@@ -826,8 +826,9 @@ void build_coarse_near(Matrix& M) {
     M.poolP[i].bytes = pool_bytes(M.nP[i], KC, M.fmt);
     M.poolP[i].p = M.alloc(M.poolP[i].bytes);
     const double* Ef = M.d_E + (size_t)M.slot0(mf) * KC * KC;
+    const bool fx = KC == FXT && !level_spread(M, mc) && !level_spread(M, mf);
     chunked(M.nP[i], [&](int64_t b0, int nb) {
-      if (KC == FXT) {
+      if (fx) {
         k_fill_Pi64<<<nb, 256, FILL64_SMEM, s>>>(d_t + b0, d_s + b0, d_ref + b0 * 4, M.poolP[i - 1].p, M.poolS.p,
                                                  M.fmt, Ef, (char*)M.poolP[i].p + pool_bytes(b0, KC, M.fmt));
         ::h2mg::count_launch();

@@ -99,6 +99,8 @@ struct Matrix {
   double* d_X = nullptr;       // [n * dim] points in compact tree order
   double* d_sw = nullptr;      // [n] sqrt(w) in compact tree order
   double* d_dg = nullptr;      // [n] diagonal entries A_ii in compact tree order
+  std::vector<unsigned char> spread_leaf;   // leaves (and clusters, by slot) whose rows have
+  std::vector<unsigned char> spread_slot;   // widely different scales (mark_spread)
   std::vector<double*> d_box;  // per level, [2^ell * 2 * dim] (lo, hi)
   double* d_nodes = nullptr;   // coupling points of clusters at levels tstar..L (heap slots):
                                // Chebyshev nodes (k per slot) or skeleton points (KC per slot)
@@ -171,6 +173,8 @@ void build_partition(Matrix& M);
 void build_skeletons(Matrix& M);
 // ---- fill.cu
 void build_bases(Matrix& M);
+void mark_spread(Matrix& M, const Matrix* base);
+bool level_spread(const Matrix& M, int ell);   // any marked cluster on tree level ell
 void build_blocks(Matrix& M, const Matrix* base);
 void build_coarse_near(Matrix& M);
 void build_f32_copies(Matrix& M);
