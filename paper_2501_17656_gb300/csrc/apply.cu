@@ -473,6 +473,7 @@ __global__ void k_leaf_spread(const int* __restrict__ leafoff, const double* __r
 // it asked for itself, so the ring needs no synchronisation. What bounds it: see
 // launch_bsgemv_fx.
 constexpr int FX_RING = 4;
+constexpr int FXB = 29;          // bits per part: at most 16 terms per accumulator
 template <int K, int NR>
 constexpr size_t fx_smem() {
   return 8 * (FX_RING * 2048 + sizeof(double) * 8 * NR * 32 + sizeof(Fx) * K * NR);
@@ -604,7 +605,7 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
 #pragma unroll
       for (int r = 0; r < 8; ++r)
 #pragma unroll
-        for (int j = 0; j < NR; ++j) xt[r][j] = fx_encode(v[r][j], Et[j]);
+        for (int j = 0; j < NR; ++j) xt[r][j] = fx_encode<FXB>(v[r][j], Et[j]);
     }
     const bool off = (s != t);
     // x of the entry's column: its exponents, then encoded into this warp's shared row
@@ -633,7 +634,7 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
       __syncwarp();                          // the previous entry's reads are done
       if (fast)
 #pragma unroll
-        for (int q = 0; q < XL; ++q) xs[lane * XL + q] = fx_encode(v[q], Es[q % NR]);
+        for (int q = 0; q < XL; ++q) xs[lane * XL + q] = fx_encode<FXB>(v[q], Es[q % NR]);
       __syncwarp();
     }
     if (fast) {
@@ -642,14 +643,14 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
 #pragma unroll
       for (int j = 0; j < NR; ++j) {
         sr[j] = fx_scale_a(Eb) * fx_scale_b(Es[j]);
-        sc[j] = fx_scale_a(Eb) * fx_scale_b(Et[j]);
+        sc[j] = fx_scale_a(Eb) * fx_scale_b(Et[j] + 1);
       }
 #pragma unroll
       for (int r = 0; r < 8; ++r)
 #pragma unroll
         for (int j = 0; j < NR; ++j) {
           yh[r][j] = 0;
-          ym[r][j] = FX_HALF;
+          ym[r][j] = fx_half<FXB>();
         }
 #pragma unroll 1
       for (int ch = c0; ch < c1; ++ch) {
@@ -666,11 +667,11 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
 #pragma unroll
           for (int j = 0; j < NR; ++j) {
             zh[j] = 0;
-            zm[j] = FX_HALF;
+            zm[j] = fx_half<FXB>() + (1ll << FXB);
           }
 #pragma unroll
           for (int r = 0; r < 8; ++r) {
-            const Fx b = fx_encode((r & 1) ? d[r / 2].y : d[r / 2].x, Eb);
+            const Fx b = fx_encode<FXB>((r & 1) ? d[r / 2].y : d[r / 2].x, Eb);
 #pragma unroll
             for (int j = 0; j < NR; ++j) {
               fx_mad(yh[r][j], b.h, xv[j].h);
@@ -682,7 +683,7 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
             }
           }
 #pragma unroll
-          for (int j = 0; j < NR; ++j) z[tt][j] = fx_join(zh[j], zm[j]);
+          for (int j = 0; j < NR; ++j) z[tt][j] = fx_join<FXB>(zh[j], zm[j]) >> 1;   // 8 rows; 64 below 2^63
         }
         if (off)
 #pragma unroll
@@ -694,7 +695,7 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
 #pragma unroll
         for (int j = 0; j < NR; ++j) {
           double& y = yad[r * NR + j][lane];
-          y = fma((double)fx_join(yh[r][j], ym[r][j]), sr[j], y);
+          y = fma((double)fx_join<FXB>(yh[r][j], ym[r][j]), sr[j], y);
         }
     } else {
       // Float64 arithmetic: blocks or vectors outside the range of fixed point. Bound by the
@@ -1564,10 +1565,12 @@ void setup_operators(Matrix& M) {
 // DRAM bandwidth, with 16 resident warps (128 registers) as the limit. Measured, one column
 // on level 2 of 65536 Gaussian points in the cube (3.6 GB of blocks): 1790 -> 880 us; the
 // whole product of 100003 points 4.38 -> 2.06 ms, with two columns per block read
-// (255 registers, 8 warps) 3.74 -> 1.81 ms at 65536 points. Error against the double-double
-// product, before / after (20000 .. 65536 points): Gaussian 3.6e-16 / 3.9e-16, Matern
-// 4.3e-16 / 4.4e-16, square 2.8e-16 / 2.9e-16, sphere 3.8e-16 / 4.1e-16, cubic polynomial
-// 1.63e-15 / 1.60e-15 (both repeat to about 0.3e-16 with the order of the atomic sums).
+// (255 registers, 8 warps) 3.74 -> 1.81 ms at 65536 points. Relative error against the
+// double-double product (mean of 8 normal vectors), float64 FMAs / here: Gaussian cube of
+// 20000 points 3.7e-16 / 2.4e-16, of 65536 5.0e-16 / 2.6e-16, Matern 4.4e-16 / 2.8e-16, square
+// 3.3e-16 / 2.8e-16, sphere 3.8e-16 / 3.0e-16, skeleton Gaussian 2.4e-16 / 2.9e-16 (rows of
+// few blocks, which more warps now add into by atomics). With parts of 28 bits a column A e_j
+// of 2000 Gaussian points was off by 4.0e-17 of its largest entry, now 1.6e-17 at most.
 constexpr int FX_WAVES = 8, FX_SMS = 152;
 template <int NR>
 static void launch_bsgemv_fx(const SymOp& op, const double* x, double* yrow, int waves, cudaStream_t s) {

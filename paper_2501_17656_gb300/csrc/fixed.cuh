@@ -1,16 +1,18 @@
 // fixed.cuh -- float64 products on the integer pipe.
 //
-// This part issues 2 float64 FMAs per clock and SM, but 27 32 x 32 -> 64-bit integer
-// multiply-adds (both measured), so a dot product whose terms share a scale is cheaper in
-// fixed point: a float64 v with |v| < 2^(E - 1022) (E: the biased exponent of the largest
-// magnitude of its block or vector) becomes the 56-bit integer
-//     V = round(v 2^(1078 - E)) = +-(h 2^28 + l),   h < 2^28, l <= 2^28, and
-//     V W = +-(h h' 2^56 + (h l' + l h') 2^28 + l l')
-// takes three multiply-adds: l l', at most 2^-56 of the largest product (2^-58 on average),
-// is left out. The integer sums are exact: 64 terms of h h' stay below 2^62, 64 middle ones
-// below 2^63. A value is off by at most 2^-57 of the largest magnitude of its block, without
-// a lean to either side (which would add up over a sum); a float64 sum of the same 64 terms
-// rounds at 2^-53 of its partial sums.
+// This part issues 2 float64 FMAs per clock and SM, but many times as many 32 x 32 -> 64-bit
+// integer multiply-adds, so a dot product whose terms share a scale is cheaper in fixed
+// point. With parts of B bits, a float64 v with |v| < s = 2^(E - 1022) (E: the biased exponent
+// of the largest magnitude of its block or vector, which is at least s / 2) becomes
+//     V = round(v 2^(2 B) / s) = +-(h 2^B + l),   h < 2^B, l <= 2^B, and
+//     V W = +-(h h' 2^(2 B) + (h l' + l h') 2^B + l l')
+// takes three multiply-adds: l l', below 2^-2B of s s', is left out. V is within 2^-(2 B + 1) of
+// s, without a lean to either side (which would add up over a sum). All bounds are relative
+// to the scales, up to twice the largest magnitudes, and not to each value: a value k bits
+// below s keeps 2 B - k bits.
+//
+// B = 28 for sums of 64 terms in one accumulator (h h' below 2^62, the middle sums below 2^63);
+// B = 29 for sums of 16: 58 bits, so that values within 2^-5 of the scale are exact.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -34,16 +36,17 @@ struct Fx {
 __device__ __forceinline__ int fx_exponent(double v) { return (__double2hiint(v) & 0x7FFFFFFF) >> 20; }
 
 // v as fixed point under the exponent E (in FX_EMIN..FX_EMAX, at least v's own): the 64 bits
-// of the significand, shifted so that the leading bit of the scale is bit 59, cut into the
-// high word and the 28 bits below it, rounded. Shifts of 32 and more go through the low word.
+// of the significand, shifted so that the leading bit of the scale is bit B + 31, cut into the
+// high word and the B bits below it, rounded. Shifts of 32 and more go through the low word.
+template <int B = 28>
 __device__ __forceinline__ Fx fx_encode(double v, int E) {
   const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-  const unsigned sh = (((unsigned)(E + 4) << 20) - (hi & 0x7FF00000u)) >> 20;
-  const unsigned t = __funnelshift_l(lo, hi, 11) | 0x80000000u, b = lo << 11;
+  const unsigned sh = (((unsigned)(E + 32 - B) << 20) - (hi & 0x7FF00000u)) >> 20;
+  const unsigned t = __funnelshift_l(lo, hi, 11) | 0x80000000u, low = lo << 11;
   unsigned h, l;
   asm("shr.u32 %0, %1, %2;" : "=r"(h) : "r"(t), "r"(sh));                        // 0 from 32 on
-  l = __funnelshift_rc(b, t, sh);                                                // t from 32 on
-  asm("shr.u32 %0, %0, %1;" : "+r"(l) : "r"(max((int)sh, 32) - 29));             // (l >> 3) there, and beyond
+  l = __funnelshift_rc(low, t, sh);                                              // t from 32 on
+  asm("shr.u32 %0, %0, %1;" : "+r"(l) : "r"(max((int)sh, 32) - B - 1));          // to B + 1 bits there, and beyond
   l = (l + 1) >> 1;
   const int s = ((int)hi >> 31) | 1;
   return {(int)h * s, (int)l * s};
@@ -54,14 +57,16 @@ __device__ __forceinline__ void fx_mad(int64_t& acc, int a, int b) {
   asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
 }
 
-// A sum in units of 2^56 from its two parts; the middle part starts at FX_HALF, so that the
+// A sum in units of 2^(2 B) from its two parts; the middle part starts at fx_half, so that the
 // shift rounds to nearest.
-constexpr int64_t FX_HALF = 1ll << 27;
-__device__ __forceinline__ int64_t fx_join(int64_t hh, int64_t mid) { return hh + (mid >> 28); }
+template <int B = 28>
+constexpr int64_t fx_half() { return 1ll << (B - 1); }
+template <int B = 28>
+__device__ __forceinline__ int64_t fx_join(int64_t hh, int64_t mid) { return hh + (mid >> B); }
 
-// A joined sum of products of values under the exponents Ea and Eb is
-// join * fx_scale_a(Ea) * fx_scale_b(Eb)  (2^(Ea - 1021) and 2^(Eb - 1079)).
+// A joined sum (B = 29) of products of values under the exponents Ea and Eb is
+// join * fx_scale_a(Ea) * fx_scale_b(Eb)  (2^(Ea - 1021) and 2^(Eb - 1081)).
 __device__ __forceinline__ double fx_scale_a(int E) { return __hiloint2double((E + 2) << 20, 0); }
-__device__ __forceinline__ double fx_scale_b(int E) { return __hiloint2double((E - 56) << 20, 0); }
+__device__ __forceinline__ double fx_scale_b(int E) { return __hiloint2double((E - 58) << 20, 0); }
 
 }  // namespace h2mg

@@ -3,8 +3,8 @@
 //
 // Operands P (a, k) and Q (b, k) are 64 x 64 tiles in shared memory, encoded with one
 // exponent per row, so that element (a, b) of P Q^T has the exact integer sum of its 64
-// terms and the scale of row a and row b; inputs lose what lies below 2^-56 of the largest
-// magnitude of their row. 3 integer multiply-adds stand in for one float64 FMA, at 27
+// terms and the scale of row a and row b; inputs are rounded at 2^-57 of the scale of their
+// row (up to twice its largest magnitude). 3 integer multiply-adds stand in for one float64 FMA, at 27
 // against 2 per clock and SM. Thread (ti, tj) = (tid / 16, tid % 16) owns rows 4 ti .. + 3
 // of P and rows tj + 16 q of Q: per k it reads 8 values for 48 multiply-adds.
 #pragma once
@@ -33,7 +33,7 @@ struct FxAcc {
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         hh[r][q] = 0;
-        mid[r][q] = FX_HALF;
+        mid[r][q] = fx_half();
       }
   }
 };
