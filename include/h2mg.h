@@ -75,9 +75,18 @@ typedef struct {
 } h2mg_kernel;
 
 /* Block storage format of the primary copy of D, the couplings S and the coarse
- * near fields P_i. F64 = IEEE double, products on the FP64 pipe. DF64 = each
- * entry stored as a pair of floats (hi, lo), hi + lo = the double to ~2^-48
- * relative, products in double-float arithmetic on the FP32 pipes (same bytes). */
+ * near fields P_i. DF64 = each entry stored as a pair of floats (hi, lo), hi + lo = the
+ * double to ~2^-48 relative, products in double-float arithmetic on the FP32 pipes (same
+ * bytes). F64 = IEEE double. Its products with blocks of 16 x 16 are float64 sums; those
+ * with blocks of 32 and 64 run in 58-bit fixed point on the integer pipe, one exponent per
+ * block and per cluster's piece of x, float64 between blocks. Each term is then off by at
+ * most 2^-55 of max|B| max|x| of its block B and piece of x: accurate in norm, like a
+ * float64 sum of terms of one size, but not entry by entry. An entry of y that is much
+ * smaller than its block's products (a column A e_j of a kernel that decays fast inside a
+ * leaf) has that absolute accuracy. Float64 sums take over, for the blocks concerned, where
+ * sqrt(w) spans more than 2^6 inside a cluster (or the diagonal 2^12 inside a leaf), where x
+ * spans more than 2^20 inside a leaf, and for magnitudes outside 2^-895..2^477, products of
+ * scales below 2^-1022, Inf and NaN. */
 typedef enum { H2MG_STORE_F64 = 0, H2MG_STORE_DF64 = 1 } h2mg_storage;
 
 /* How the nested cluster bases are made before their QR orthonormalisation (Sec. 3.3).

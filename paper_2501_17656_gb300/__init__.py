@@ -338,7 +338,7 @@ class H2Matrix:
     # ----------------------------------------------------------------- products
     def apply(self, x, y=None, precision: str | None = None):
         """y = A x for a vector or an (n, nrhs) block of columns. Default: the primary
-        storage, the columns through the products in groups of four. ``precision``
+        storage (accurate in norm, not entry by entry: h2mg_storage), the columns through the products in groups of four. ``precision``
         "f64", "mixed_f32" (the FP32 copy on the CUDA cores) or "tf32x3" (the FP32 copy
         on the tensor cores, 128 columns per block read; see h2mg_apply_ex)."""
         _expect(x, self.n, "x", cols=True, dev=self.device)

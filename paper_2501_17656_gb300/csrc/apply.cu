@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(256) k_bsgemv_small(const int* __restrict__ er
 
 // ----------------------------------------------------------------------------- float64 block GEMV
 // Exponent of every stored float64 block (one warp per block): the biased exponent of its
-// largest magnitude, FX_EMIN for an all-zero block, FX_NONE where fixed point does not
+// largest magnitude, FX_EZERO for an all-zero block, FX_NONE where fixed point does not
 // serve: exponents outside FX_EMIN..FX_VMAX (Inf and NaN among them), or, with `skip`
 // given, a row or column cluster it marks.
 __global__ void k_block_exponents(const void* const* __restrict__ blk, const int* __restrict__ row,
@@ -436,7 +436,7 @@ __global__ void k_block_exponents(const void* const* __restrict__ blk, const int
   m = __reduce_max_sync(0xffffffffu, m);
   any = __any_sync(0xffffffffu, any);
   if (lane == 0) {
-    int E = any ? ((m < FX_EMIN || m > FX_VMAX) ? FX_NONE : m) : FX_EMIN;
+    int E = any ? ((m < FX_EMIN || m > FX_VMAX) ? FX_NONE : m) : FX_EZERO;
     if (skip && (skip[row[e]] || skip[col[e]])) E = FX_NONE;
     bexp[e] = (short)E;
   }
@@ -474,6 +474,12 @@ __global__ void k_leaf_spread(const int* __restrict__ leafoff, const double* __r
 // launch_bsgemv_fx.
 constexpr int FX_RING = 4;
 constexpr int FXB = 29;          // bits per part: at most 16 terms per accumulator
+// Point values that span more than 2^20 inside a leaf go through float64 with the leaf's
+// blocks: below that the smallest keep 38 bits. Normally distributed values exceed it in one
+// leaf of 10000. (At 2^16, one of 700, the few warps that meet such leaves end last: two
+// columns of 65536 points took 1.85 ms instead of 1.76.) Coefficients, of orthonormal bases,
+// have no such limit: what counts there is their norm, and smooth vectors span many decades.
+constexpr int FX_SPREAD = 20;
 template <int K, int NR>
 constexpr size_t fx_smem() {
   return 8 * (FX_RING * 2048 + sizeof(double) * 8 * NR * 32 + sizeof(Fx) * K * NR);
@@ -488,7 +494,7 @@ template <int K, int NR>
 __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
     k_bsgemv_fx(const int* __restrict__ erow, const int* __restrict__ col, const void* const* __restrict__ blk,
                 const short* __restrict__ bexp, const double* x, double* yrow,
-                int64_t units, int per) {
+                int64_t units, int per, int spread) {
   constexpr int LPC = K / 8, CPP = 32 / LPC, T = K * K / 256, CH = T < LPC ? T : LPC, NCH = T / CH;
   constexpr int XL = K * NR / 32;                // elements of x_s per lane
   extern __shared__ __align__(16) unsigned char dsm[];
@@ -571,6 +577,25 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
       atomicAdd(yrow + ((int64_t)s * K + cl + CPP * (ch * CH + (lane & (CH - 1)))) * NR + j, (double)z[0][j] * scale);
   };
 
+  // largest exponent, and smallest of a value that is not zero (a subnormal one: 0)
+  auto widest = [](double v, int& hi, int& lo) {
+    const int x = fx_exponent(v);
+    hi = max(hi, x);
+    lo = min(lo, fx_is_zero(v) ? 4095 : x);
+  };
+  // exponents of a piece of the vector, from all lanes' hi and lo; false: float64
+  auto vector_exponents = [&](int (&hi)[NR], const int (&lo)[NR]) {
+    bool out = false;
+#pragma unroll
+    for (int j = 0; j < NR; ++j) hi[j] = __reduce_max_sync(0xffffffffu, hi[j]);
+#pragma unroll
+    for (int j = 0; j < NR; ++j) {
+      out = out || lo[j] < hi[j] - spread || (hi[j] < FX_EMIN && lo[j] < 4095) || hi[j] > FX_VMAX;
+      hi[j] = hi[j] == 0 ? FX_EZERO : hi[j];
+    }
+    return !__any_sync(0xffffffffu, out);
+  };
+
   for (int64_t u = u0; u < u1;) {
     const int e = (int)(u / NCH);
     const int c0 = (int)(u % NCH), c1 = (int)min((int64_t)NCH, c0 + (u1 - u));
@@ -582,26 +607,19 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
       row = t;
       xrow = x + (int64_t)t * K * NR;
       double v[8][NR];
-      tfast = true;
+      int lo[NR];
 #pragma unroll
       for (int j = 0; j < NR; ++j) {
-        int m = 0;
+        Et[j] = 0;
+        lo[j] = 4095;
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
           v[r][j] = xrow[(rb + r) * NR + j];
-          m = max(m, fx_exponent(v[r][j]));
+          widest(v[r][j], Et[j], lo[j]);
           yad[r * NR + j][lane] = 0.0;
         }
-        m = __reduce_max_sync(0xffffffffu, m);
-        Et[j] = m == 0 ? FX_EMIN : m;   // a zero column (subnormals count as zero only if all are 0, below)
-        tfast = tfast && Et[j] >= FX_EMIN && Et[j] <= FX_VMAX;
-        if (m == 0) {
-          bool nz = false;
-#pragma unroll
-          for (int r = 0; r < 8; ++r) nz = nz || v[r][j] != 0.0;
-          tfast = tfast && !__any_sync(0xffffffffu, nz);
-        }
       }
+      tfast = vector_exponents(Et, lo);
 #pragma unroll
       for (int r = 0; r < 8; ++r)
 #pragma unroll
@@ -614,23 +632,20 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
     bool fast = tfast && Eb != FX_NONE;
     {
       double v[XL];
-      int m[NR];
-      bool nz = false;
+      int lo[NR];
 #pragma unroll
-      for (int j = 0; j < NR; ++j) m[j] = 0;
+      for (int j = 0; j < NR; ++j) {
+        Es[j] = 0;
+        lo[j] = 4095;
+      }
 #pragma unroll
       for (int q = 0; q < XL; ++q) {
         v[q] = xcol[lane * XL + q];          // XL is a multiple of NR: element q is column q % NR
-        m[q % NR] = max(m[q % NR], fx_exponent(v[q]));
-        nz = nz || (fx_exponent(v[q]) == 0 && v[q] != 0.0);
+        widest(v[q], Es[q % NR], lo[q % NR]);
       }
-      nz = __any_sync(0xffffffffu, nz);
+      fast = vector_exponents(Es, lo) && fast;
 #pragma unroll
-      for (int j = 0; j < NR; ++j) {
-        m[j] = __reduce_max_sync(0xffffffffu, m[j]);
-        Es[j] = m[j] == 0 ? FX_EMIN : m[j];
-        fast = fast && Es[j] >= FX_EMIN && Es[j] <= FX_VMAX && !(m[j] == 0 && nz);
-      }
+      for (int j = 0; j < NR; ++j) fast = fast && Eb + min(Es[j], Et[j]) >= FX_VSUM;
       __syncwarp();                          // the previous entry's reads are done
       if (fast)
 #pragma unroll
@@ -1501,6 +1516,7 @@ void setup_operators(Matrix& M) {
       H.rowptr.push_back((int)H.col.size());
     }
     M.opD = upload_op(M, H, M.KD, M.poolD.p, nullptr, M.poolD32.p, nullptr, M.spread_leaf);
+    M.opD.spread = FX_SPREAD;
   }
   M.opC.assign(M.lev + 1, SymOp{});
   if (M.tstar >= 0) {
@@ -1582,10 +1598,10 @@ static void launch_bsgemv_fx(const SymOp& op, const double* x, double* yrow, int
   const int grid = (int)((units + 8 * (int64_t)per - 1) / (8 * (int64_t)per));
   if (op.K == 64) {
     launch_chain(k_bsgemv_fx<64, NR>, grid, 256, fx_smem<64, NR>(), s, op.erow, op.col, op.blk, op.bexp, x, yrow, units,
-                 per);
+                 per, op.spread);
   } else {
     launch_chain(k_bsgemv_fx<32, NR>, grid, 256, fx_smem<32, NR>(), s, op.erow, op.col, op.blk, op.bexp, x, yrow, units,
-                 per);
+                 per, op.spread);
   }
 }
 

@@ -23,8 +23,9 @@ namespace h2mg {
 // Biased exponents for which values go through fixed point: Inf, NaN and subnormal
 // magnitudes stay outside, and no scale factor below overflows or loses bits.
 constexpr int FX_EMIN = 128, FX_EMAX = 2000;
-// The same for blocks and vectors whose two scales are multiplied with each other first.
-constexpr int FX_VMAX = 1500;
+// The same for blocks and vectors whose two scales are multiplied with each other first, and
+// the least sum of the two: the product stays a normal number.
+constexpr int FX_VMAX = 1500, FX_VSUM = 1080;
 // Marks a block that the float64 path multiplies (see k_block_exponents).
 constexpr int FX_NONE = -1;
 
@@ -32,8 +33,16 @@ struct Fx {
   int h, l;
 };
 
+// The exponent of a block or vector of zeros, which any would fit.
+constexpr int FX_EZERO = 1023;
+
 // Biased exponent field of |v| (2047: Inf or NaN).
 __device__ __forceinline__ int fx_exponent(double v) { return (__double2hiint(v) & 0x7FFFFFFF) >> 20; }
+
+// On the integer pipe: a float64 comparison issues like a float64 FMA.
+__device__ __forceinline__ bool fx_is_zero(double v) {
+  return ((__double2hiint(v) & 0x7FFFFFFF) | __double2loint(v)) == 0;
+}
 
 // v as fixed point under the exponent E (in FX_EMIN..FX_EMAX, at least v's own): the 64 bits
 // of the significand, shifted so that the leading bit of the scale is bit B + 31, cut into the

@@ -30,6 +30,7 @@ struct SymOp {
   const void** blk32 = nullptr;    // [nnz] block pointers into the FP32 pool (or null)
   int* erow = nullptr;    // [nnz] row of each entry
   short* bexp = nullptr;  // [nnz] exponent of each block (fixed.cuh): float64 blocks of 32 and 64 only
+  int spread = 2047;      // fixed point: exponents that a cluster's piece of the vector may span
   int64_t noff = 0;       // off-diagonal entries (each adds K transposed partials)
   // CTAs per block row (per SM, for the kernels that deal warps by entry) chosen by the autotuner, per element format
   // (F64, DF, F32) and column group size (NR = 1, 2, 4); 0 = the fixed heuristic
