@@ -853,7 +853,8 @@ __global__ void __launch_bounds__(256) k_coef_in(VecIn in, int64_t n, typename A
 }
 
 // Float -> double by moving the bits: the conversion instruction runs at the float64 rate (2
-// per clock and SM), as many as the products it feeds. Subnormals become zero.
+// per clock and SM), as many as the products it feeds. For finite values; subnormals become
+// zero, which the bases do not hold: QR leaves roundings of 1e-17 in the rows of least weight.
 __device__ __forceinline__ double widen(float f) {
   const unsigned u = __float_as_uint(f), m = u & 0x7FFFFFFFu;
   return m < 0x00800000u ? 0.0 : __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
