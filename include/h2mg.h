@@ -374,14 +374,16 @@ int64_t h2mg_launch_count(void);
 h2mg_status h2mg_profile(h2mg_matrix A, int enable, int64_t* launches, double* ms, double* bytes);
 
 /* Autotuner of the block-sparse product (the kernel that streams D, S and P_i). The
- * library launches it with a number of CTAs per block row; by default a fixed rule
- * (enough CTAs to fill the GPU when an operator has few block rows). This call times
- * trial launches of every operator of the hierarchy (index 0: the close part of level
- * 1; index i >= 1: the coupling operator of level i), for the primary format with 1
- * and 2 columns and the FP32 copy with 1, 2 and 4 columns, over the splits 1..64, and
- * keeps the fastest in the handle; later products, smoothers and solves use it (a
- * CUDA graph captured before the call keeps the old choice). report (optional, cap
- * entries of 4 doubles) receives (operator index, columns, ms with the fixed rule, ms
+ * library launches it with a number of CTAs per block row (64 x 64 blocks in FP32 and
+ * double-float) or per SM (float64 blocks of 32 and 64, and blocks of 16 and 32, whose
+ * entries are dealt to warps); by default a fixed rule (enough CTAs to fill the GPU when
+ * an operator has few block rows; 8 per SM). This call times trial launches of every
+ * operator of the hierarchy (index 0: the close part of level 1; index i >= 1: the
+ * coupling operator of level i), for the primary format with 1 and 2 columns and the FP32
+ * copy with 1, 2 and 4 columns, over the numbers 1..64, and keeps the fastest in the
+ * handle; later products, smoothers and solves use it (a CUDA graph captured before the
+ * call keeps the old choice; the double-double product is not tuned). report (optional,
+ * cap entries of 4 doubles) receives (operator index, columns, ms with the fixed rule, ms
  * tuned) per combination; *count (optional) = the number of combinations. Runs on
  * `stream` and synchronises it; h2mg_profile must be off. No counterpart in the paper
  * (a launch-configuration choice of this implementation). */

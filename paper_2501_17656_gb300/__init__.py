@@ -315,7 +315,7 @@ class H2Matrix:
         return int(n.value), float(ms.value), float(by.value)
 
     def autotune(self):
-        """Tune the block product's CTAs per block row on trial launches (h2mg_autotune).
+        """Tune the block product's CTAs per block row or per SM on trial launches (h2mg_autotune).
         Returns a list of (operator, columns, fixed-rule ms, tuned ms)."""
         cap = 256
         buf = (ctypes.c_double * (4 * cap))()

@@ -1887,14 +1887,16 @@ void apply_level1_ws_sizes(const Matrix& M, size_t* coef, size_t* pts) {
 }
 
 // ----------------------------------------------------------------------------- autotuner
-// Times `reps` launches of one block product with row split `split` on the handle's
-// workspaces (contents irrelevant: only the launch time is wanted).
+// Times `reps` launches of one block product with launch shape `split` on the handle's
+// workspaces. The vector is cleared: the float64 product takes its arithmetic from the data,
+// and zeros take the usual one (earlier contents can be NaN or the halves of other formats).
 template <int FMT, int NR>
 static float time_product(Matrix& M, SymOp& op, bool pts, int split, int reps, cudaStream_t s, cudaEvent_t e0,
                           cudaEvent_t e1) {
   const bool f32 = FMT == FMT_F32;
   void* x = pts ? M.wxp.p : M.wx.p;
   void* y = pts ? M.wyp.p : M.wyrow.p;
+  H2_CUDA(cudaMemsetAsync(x, 0, sizeof(typename Ar<FMT>::vec_t) * (size_t)op.nrows * op.K * NR, s));
   H2_CUDA(cudaMemsetAsync(y, 0, sizeof(typename Ar<FMT>::yo_t) * (size_t)op.nrows * op.K * NR, s));
   launch_bsgemv<FMT, NR>(M, op, f32, x, y, s, split);   // warm-up
   H2_CUDA(cudaEventRecord(e0, s));
