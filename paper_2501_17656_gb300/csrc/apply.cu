@@ -1461,7 +1461,8 @@ static OpHost coupling_rows(const Matrix& M, int top, int i) {
 // couplings, the coarse near fields and the dense expansion, whose orthonormal bases are
 // then graded. Without the guard above the leaves, the middle row of a product with 3000
 // points, a far field and weights over 24 decades was off by 1.6e-12 of itself (float64:
-// 5.4e-16). The skeletons and bases themselves are made in float64. A sibling on its base's
+// 5.4e-16). So do clusters whose entries are all far too large or too small for the exponents
+// of fixed point. The skeletons and bases themselves are made in float64. A sibling on its base's
 // bases (Chebyshev) takes over the base's marks.
 void mark_spread(Matrix& M, const Matrix* base) {
   const int L = M.L, nleaf = 1 << L;
@@ -1473,8 +1474,15 @@ void mark_spread(Matrix& M, const Matrix* base) {
   H2_CUDA(cudaStreamSynchronize(M.stream));
   M.free_owned(d);
   constexpr int BITS = 6;
+  // scales of the entries that the tiles' exponents (FX_EMIN..FX_EMAX) carry with room to spare
+  constexpr int LEAST = 400, MOST = 1700;
+  std::vector<unsigned char> out(nleaf);                    // clusters with a leaf outside
   M.spread_leaf.assign(nleaf, 0);
-  for (int j = 0; j < nleaf; ++j) M.spread_leaf[j] = h[j].y - h[j].x > 2 * BITS || h[j].w - h[j].z > BITS;
+  for (int j = 0; j < nleaf; ++j) {
+    const int m = std::max<int>(h[j].y, 2 * h[j].w - 1023);
+    out[j] = m < LEAST || m > MOST;
+    M.spread_leaf[j] = out[j] || h[j].y - h[j].x > 2 * BITS || h[j].w - h[j].z > BITS;
+  }
   if (base) {
     M.spread_slot = base->spread_slot;
     return;
@@ -1482,10 +1490,11 @@ void mark_spread(Matrix& M, const Matrix* base) {
   M.spread_slot.assign(std::max(M.nslots(), 0), 0);
   if (M.tstar < 0) return;
   for (int ell = L; ell >= M.tstar; --ell) {
-    for (int j = 0; j < (1 << ell); ++j) M.spread_slot[M.slot0(ell) + j] = h[j].w - h[j].z > BITS;
+    for (int j = 0; j < (1 << ell); ++j) M.spread_slot[M.slot0(ell) + j] = out[j] || h[j].w - h[j].z > BITS;
     for (int j = 0; j < (1 << ell) / 2; ++j) {
       h[j].z = std::min(h[2 * j].z, h[2 * j + 1].z);
       h[j].w = std::max(h[2 * j].w, h[2 * j + 1].w);
+      out[j] = out[2 * j] || out[2 * j + 1];
     }
   }
 }
