@@ -693,7 +693,7 @@ void apply_panel(Matrix& M, const double* x, int64_t ldx, double* y, int64_t ldy
   int h = 0;
   H2_CUDA(cudaMemcpyAsync(&h, M.d_flag + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
   H2_CUDA(cudaStreamSynchronize(s));
-  H2_REQUIRE(h == 0, H2MG_ERR_CUDA, "a tensor-core product timed out waiting for its MMAs");
+  H2_REQUIRE(h == 0, H2MG_ERR_TIMEOUT, "a tensor-core product timed out waiting for its MMAs");
 }
 
 }  // namespace h2mg

@@ -568,7 +568,7 @@ void build_skeletons(Matrix& M) {
     int late = 0;
     H2_CUDA(cudaMemcpyAsync(&late, M.d_flag + 2, sizeof(int), cudaMemcpyDeviceToHost, s));
     H2_CUDA(cudaStreamSynchronize(s));
-    H2_REQUIRE(late == 0, H2MG_ERR_CUDA, "a skeletonization timed out waiting for its warps");
+    H2_REQUIRE(late == 0, H2MG_ERR_TIMEOUT, "a skeletonization timed out waiting for its warps");
     M.free_owned(d_samp);
     M.free_owned(d_soff);
     M.free_owned(d_seg);
