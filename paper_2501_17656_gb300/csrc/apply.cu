@@ -1597,13 +1597,13 @@ void setup_operators(Matrix& M) {
 // 3.3e-16 / 2.8e-16, sphere 3.8e-16 / 3.0e-16, skeleton Gaussian 2.4e-16 / 2.9e-16 (rows of
 // few blocks, which more warps now add into by atomics). With parts of 28 bits a column A e_j
 // of 2000 Gaussian points was off by 4.0e-17 of its largest entry, now 1.6e-17 at most.
-constexpr int FX_WAVES = 8, FX_SMS = 152;
+constexpr int FX_WAVES = 8;
 template <int NR>
 static void launch_bsgemv_fx(const SymOp& op, const double* x, double* yrow, int waves, cudaStream_t s) {
   const int nch = op.K == 64 ? 2 : 1;
   const int64_t units = (int64_t)op.nnz * nch;
   if (units == 0) return;
-  const int64_t warps = (int64_t)(waves > 0 ? waves : FX_WAVES) * FX_SMS * 8;
+  const int64_t warps = (int64_t)(waves > 0 ? waves : FX_WAVES) * SMS * 8;
   const int per = (int)((units + warps - 1) / warps);
   const int grid = (int)((units + 8 * (int64_t)per - 1) / (8 * (int64_t)per));
   if (op.K == 64) {
@@ -1672,7 +1672,7 @@ static void launch_bsgemv(Matrix& M, const SymOp& op, bool f32, const void* x, v
       launch_chain(k_bsgemv<64, FMT, NR>, grid, 256, 0, s, op.rowptr, op.col, blk, (const vt*)x, (yt*)yrow, split, first);
     }
   } else if (op.nnz > 0) {
-    const int64_t warps = (int64_t)(waves > 0 ? waves : FX_WAVES) * FX_SMS * 8;
+    const int64_t warps = (int64_t)(waves > 0 ? waves : FX_WAVES) * SMS * 8;
     const int per = (int)((op.nnz + warps - 1) / warps);
     const int g = ceil_div(op.nnz, 8 * (int64_t)per);
     if (op.K == 16) {
@@ -1736,7 +1736,7 @@ static int pass_down(const Matrix& M, const char* epool, const void* yrow, void*
     const bool last = lb == lbot;
     double* yo = last ? yout : nullptr;
     const double* pd = last ? pdot : nullptr;
-    const int S = (1 << lb) >= 4 * 152 ? 4 : 2;
+    const int S = (1 << lb) >= 4 * SMS ? 4 : 2;
     grid = std::min(std::max(1, (1 << lb) / S), CG_PARTS);
     auto go = [&](auto kernel) {
       launch_chain(kernel, grid, 256, 0, s, epool, (const yt*)yrow, ypar, (vt*)yc, lt, lb, ts, yo, ldo, pd, part);

@@ -40,6 +40,7 @@ struct SymOp {
   }
 };
 inline int nr_index(int nr) { return nr >= 4 ? 2 : nr - 1; }
+constexpr int SMS = 152;   // of a GB300
 // Fixed heuristic of the block product: enough CTAs to fill the GPU when the operator
 // has few block rows (at most 16 CTAs per row).
 inline int split_heuristic(int nrows) {

@@ -341,7 +341,7 @@ void smooth_multi(Matrix& M, int i, bool f32, const double* f, const double* x0,
     q0 = W.cq;
   }
   // one element per thread where the vector is short: the steps are latency, not bandwidth
-  const int g = (int)std::max<int64_t>(1, std::min<int64_t>(2 * 152, (N + 255) / 256));
+  const int g = (int)std::max<int64_t>(1, std::min<int64_t>(2 * SMS, (N + 255) / 256));
   launch_chain(k_cg_start, dim3(g, nr), 256, 0, s, f, q0, N, x, rr, W.cp, W.pb, W.pa);
   H2_LAUNCH_CHECK();
   if (n == 0) return;
