@@ -1665,8 +1665,11 @@ static void launch_bsgemv(Matrix& M, const SymOp& op, bool f32, const void* x, v
     if constexpr (FMT != FMT_F64) {
       // The warps' first blocks are asked for ahead (about 80 MB over the first wave of CTAs). One
       // column: only where the previous kernel runs beside it, and not for operators of several
-      // times the L2, whose other blocks then miss it (level 2 of 30011 points, 0.9 GB: 6.53 ->
-      // 6.69 ms for 40 steps; 16384 points of a dense cube, 0.25 GB: 9.50 -> 8.86 ms a cycle).
+      // times the L2, whose other blocks then miss it. Per FP32 CG step, without / with: level 2
+      // of 8000 points (0.10 GB) 39.5 / 35.1 us, of 16384 (0.31 GB) 76.2 / 73.3, of 20000 (0.85
+      // GB) 162.7 / 166.7, of 40000 (1.8 GB) 313.7 / 320.3; level 1, two operators in turn, of
+      // 8000 (36 MB) 58.4 / 52.5, of 16384 (0.13 and 0.18 GB) 96.1 / 99.6, of 20000 (0.54 GB) 195 /
+      // 203. The line lies between the level-2 operators of 0.31 and 0.85 GB.
       const double bytes = (double)op.nnz * 4096 * (FMT == FMT_F32 ? 4 : 8);
       const bool first = NR >= 2 || (bytes <= 512e6 && chained(s));
       launch_chain(k_bsgemv<64, FMT, NR>, grid, 256, 0, s, op.rowptr, op.col, blk, (const vt*)x, (yt*)yrow, split, first);
@@ -1721,7 +1724,8 @@ static void pass_up(const Matrix& M, const char* epool, void* xc, int lb, int ts
 // Downward pass from the coupling top level ts to level `lbot`, up to 5 levels per
 // launch (the first launch takes the odd ones); the last level goes to yout (when given)
 // instead of the coefficient buffer, with partials of pdot^T yout. Returns the last launch's
-// CTAs. Two clusters per CTA where four would leave SMs without one.
+// CTAs. Two clusters per CTA where four would leave SMs without one: per FP32 CG step on level
+// 2, S = 2 / 4: 256 clusters 72.9 / 73.7 us, 512 162.8 / 161.3, 1024 316.9 / 313.4.
 constexpr int DOWN_LEVELS = 5;
 template <int FMT, int NR>
 static int pass_down(const Matrix& M, const char* epool, const void* yrow, void* yc, int ts, int lbot, double* yout,
