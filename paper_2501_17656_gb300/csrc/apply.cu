@@ -17,9 +17,10 @@
 // (k_down_tree) adds the transfer from the parent to each level's row results and writes the
 // finest level out (k_leaf_final at i = 1).
 //
-// Arithmetic per block format: F64 (fixed point, DFMA where it does not serve), DF (double-float on the FP32 pipes: the
-// error-free products/sums of Dekker and Knuth), F32 (FP32 FMA). Vectors inside the
-// product are in the same format; the multigrid vectors outside are float64.
+// Arithmetic per block format: F64 (fixed point, DFMA where it does not serve), DF
+// (double-float on the FP32 pipes: the error-free products/sums of Dekker and Knuth), F32
+// (FP32 FMA). Vectors inside the product are in the same format; the multigrid vectors
+// outside are float64.
 #include <algorithm>
 
 #include "fixed.cuh"
@@ -1587,16 +1588,19 @@ void setup_operators(Matrix& M) {
 // `waves` CTAs per SM in all (0: the default), fewer when there is less than one unit per
 // warp. Float64 FMAs (k_bsgemv) take 2 x 4096 / 2 clocks of an SM per 64 x 64 block, where
 // its 32 KB take 1500 at the copy bandwidth; in fixed point the encoding (22 operations a
-// value) and the multiply-adds (6) keep the integer pipes at 60% and the stream at 64% of the
-// DRAM bandwidth, with 16 resident warps (128 registers) as the limit. Measured, one column
-// on level 2 of 65536 Gaussian points in the cube (3.6 GB of blocks): 1790 -> 880 us; the
-// whole product of 100003 points 4.38 -> 2.06 ms, with two columns per block read
-// (255 registers, 8 warps) 3.74 -> 1.81 ms at 65536 points. Relative error against the
-// double-double product (mean of 8 normal vectors), float64 FMAs / here: Gaussian cube of
-// 20000 points 3.7e-16 / 2.4e-16, of 65536 5.0e-16 / 2.6e-16, Matern 4.4e-16 / 2.8e-16, square
-// 3.3e-16 / 2.8e-16, sphere 3.8e-16 / 3.0e-16, skeleton Gaussian 2.4e-16 / 2.9e-16 (rows of
-// few blocks, which more warps now add into by atomics). With parts of 28 bits a column A e_j
-// of 2000 Gaussian points was off by 4.0e-17 of its largest entry, now 1.6e-17 at most.
+// value) and the multiply-adds (6) keep the ALU pipe at 60% and the DRAM at 57% of its peak
+// (30011 points, one column: 4.6 TB/s), with 16 resident warps (128 registers) as the limit;
+// two columns (252 registers, 8 warps) 43% and 30%. Whole products of 65536 Gaussian points in
+// the cube: one column 1.92 -> 0.91 ms, two 3.73 -> 1.75 ms; of 100003 points, one column,
+// 4.38 -> 2.06 ms. CTAs per SM 4 / 8 / 16, one column: 16384 points 215 / 204 / 216 us, 30011
+// 493 / 495 / 499, 65536 on the square 182 / 194 / 193.
+//
+// Relative error against the double-double product (mean of 8 normal vectors), float64 FMAs
+// / here: Gaussian cube of 20000 points 3.7e-16 / 2.4e-16, of 65536 5.0e-16 / 2.6e-16, Matern
+// 4.4e-16 / 2.8e-16, square 3.3e-16 / 2.8e-16, sphere 3.8e-16 / 3.0e-16, skeleton Gaussian
+// 2.4e-16 / 2.9e-16 (rows of few blocks, which more warps now add into by atomics). With parts
+// of 28 bits a column A e_j of 2000 Gaussian points was off by 4.0e-17 of its largest entry;
+// now it is within 2^-55.7.
 constexpr int FX_WAVES = 8;
 template <int NR>
 static void launch_bsgemv_fx(const SymOp& op, const double* x, double* yrow, int waves, cudaStream_t s) {

@@ -86,9 +86,8 @@ __global__ void k_expand(const double* __restrict__ G, int64_t nc, const double*
 
 // k_expand for 64 x 64 blocks, tile (a, ap <= a) per CTA: the other half of the symmetric
 // result is its mirror image. Two products of 64 x 64 matrices per tile on the integer pipe
-// (fx_tile.cuh), 29 k clocks of an SM each; on the float64 pipe, and for both halves, it was
-// bound by 131 k clocks each: order 4096 took 3.62 ms,
-// now 0.48 ms.
+// (fx_tile.cuh), 35 k clocks of an SM each with loads and encoding; on the float64 pipe, and
+// for both halves, it was bound by 131 k clocks each: order 4096 took 3.62 ms, now 0.48 ms.
 __global__ void __launch_bounds__(256, 2) k_expand64(const double* __restrict__ G, int64_t nc,
                                                      const double* __restrict__ B, int shift,
                                                      double* __restrict__ out, int64_t no) {
@@ -171,10 +170,12 @@ __global__ void k_scale_sym(const double* __restrict__ A, int64_t n, const doubl
 // inverted in float64 by the CTA that updates it first, beside the rest of its step.
 // X and B are stored transposed, so that every tile is read along consecutive addresses.
 //
-// Bound by the integer multiply-adds: n^3 / 2 FMAs at 3 each, 12 ms for n = 4096 at 27 per
-// clock and SM (the float64 pipe, 2 FMAs per clock and SM, would need 55 ms). Measured for
-// n = 4096: 21.7 ms (updates 14.7, inverse 5.3, panels 1.5), before 180 ms (32-column panels
-// with unblocked substitution, and an inverse from two dense triangular solves).
+// n^3 / 2 FMAs are 5 ms of integer multiply-adds for n = 4096 at the instruction's own 63 per
+// clock and SM, and 55 ms on the float64 pipe. Measured for n = 4096: 21.7 ms (updates 14.7,
+// inverse 5.3, panels 1.5), before 180 ms (32-column panels with unblocked substitution, and
+// an inverse from two dense triangular solves). A tile takes 40 k clocks of an SM, 12 k of
+// them multiply-adds at that rate: issue slots and the ALU pipe are 45 % busy, the FMA pipe
+// 21 %, with 16 warps that wait for one another's operands (dispatch and fixed latencies).
 constexpr int DB = FXT;                                     // block edge
 constexpr size_t DENSE_SMEM = FX_PAIR_BYTES;
 

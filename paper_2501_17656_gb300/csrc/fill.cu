@@ -533,7 +533,7 @@ __global__ void k_fill_Pi(const int* __restrict__ pt, const int* __restrict__ ps
 // ----------------------------------------------------------------------------- 64 x 64 blocks
 // P_i (i >= 3) of 64 x 64 blocks takes six products of 64 x 64 matrices per block (eight in
 // k_fill_Pi): on the float64 pipe 131 k clocks of an SM each, which bounded it; here they run
-// on the integer pipe (fx_tile.cuh), 29 k clocks each. One CTA per block, two CTAs per SM so
+// on the integer pipe (fx_tile.cuh), 43 k clocks each with loads and encoding. One CTA per block, two CTAs per SM so
 // that one's loads and encodings run beside the other's products. Measured on 20000 Gaussian
 // points in the cube (Chebyshev, P_3 .. P_5): 77.8 -> 12.5 ms. The couplings S = R_t k R_s^T
 // (k_fill_S) and P_2 = U^T D U (k_fill_P2) stay in float64: the factors R are graded, and one

@@ -1,9 +1,10 @@
 // fixed.cuh -- float64 products on the integer pipe.
 //
-// This part issues 2 float64 FMAs per clock and SM, but many times as many 32 x 32 -> 64-bit
-// integer multiply-adds, so a dot product whose terms share a scale is cheaper in fixed
-// point. With parts of B bits, a float64 v with |v| < s = 2^(E - 1022) (E: the biased exponent
-// of the largest magnitude of its block or vector, which is at least s / 2) becomes
+// This part issues 2 float64 FMAs per clock and SM, but 63 32 x 32 -> 64-bit integer
+// multiply-adds (both measured, from registers), so a dot product whose terms share a scale
+// is cheaper in fixed point. With parts of B bits, a float64 v with |v| < s = 2^(E - 1022) (E:
+// the biased exponent of the largest magnitude of its block or vector, which is at least
+// s / 2) becomes
 //     V = round(v 2^(2 B) / s) = +-(h 2^B + l),   h < 2^B, l <= 2^B, and
 //     V W = +-(h h' 2^(2 B) + (h l' + l h') 2^B + l l')
 // takes three multiply-adds: l l', below 2^-2B of s s', is left out. V is within 2^-(2 B + 1) of

@@ -4,9 +4,11 @@
 // Operands P (a, k) and Q (b, k) are 64 x 64 tiles in shared memory, encoded with one
 // exponent per row, so that element (a, b) of P Q^T has the exact integer sum of its 64
 // terms and the scale of row a and row b; inputs are rounded at 2^-57 of the scale of their
-// row (up to twice its largest magnitude). 3 integer multiply-adds stand in for one float64 FMA, at 27
-// against 2 per clock and SM. Thread (ti, tj) = (tid / 16, tid % 16) owns rows 4 ti .. + 3
-// of P and rows tj + 16 q of Q: per k it reads 8 values for 48 multiply-adds.
+// row (up to twice its largest magnitude). 3 integer multiply-adds stand in for one float64
+// FMA, at up to 57 against 2 per clock and SM (this pattern from registers, 8 warps; with the
+// reads and the encoding a product takes 35 to 43 k clocks of an SM, 131 k on the float64
+// pipe). Thread (ti, tj) = (tid / 16, tid % 16) owns rows 4 ti .. + 3 of P and rows tj + 16 q
+// of Q: per k it reads 8 values for 48 multiply-adds.
 #pragma once
 
 #include "fixed.cuh"
