@@ -624,7 +624,7 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
 #pragma unroll
       for (int r = 0; r < 8; ++r)
 #pragma unroll
-        for (int j = 0; j < NR; ++j) xt[r][j] = fx_encode<FXB>(v[r][j], Et[j]);
+        for (int j = 0; j < NR; ++j) xt[r][j] = fx_encode<FXB>(v[r][j], Et[j] + 1);   // a bit less: 64 terms below 2^63
     }
     const bool off = (s != t);
     // x of the entry's column: its exponents, then encoded into this warp's shared row
@@ -653,7 +653,7 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
         for (int q = 0; q < XL; ++q) xs[lane * XL + q] = fx_encode<FXB>(v[q], Es[q % NR]);
       __syncwarp();
     }
-    if (fast) {
+    if (__builtin_expect(fast, 1)) {
       int64_t yh[8][NR], ym[8][NR];
       double sr[NR], sc[NR];
 #pragma unroll
@@ -683,7 +683,7 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
 #pragma unroll
           for (int j = 0; j < NR; ++j) {
             zh[j] = 0;
-            zm[j] = fx_half<FXB>() + (1ll << FXB);
+            zm[j] = fx_half<FXB>();
           }
 #pragma unroll
           for (int r = 0; r < 8; ++r) {
@@ -699,7 +699,7 @@ __global__ void __launch_bounds__(256, NR == 1 ? 2 : 1)
             }
           }
 #pragma unroll
-          for (int j = 0; j < NR; ++j) z[tt][j] = fx_join<FXB>(zh[j], zm[j]) >> 1;   // 8 rows; 64 below 2^63
+          for (int j = 0; j < NR; ++j) z[tt][j] = fx_join<FXB>(zh[j], zm[j]);
         }
         if (off)
 #pragma unroll
@@ -1591,14 +1591,14 @@ void setup_operators(Matrix& M) {
 // value) and the multiply-adds (6) keep the ALU pipe at 60% and the DRAM at 57% of its peak
 // (30011 points, one column: 4.6 TB/s), with 16 resident warps (128 registers) as the limit;
 // two columns (252 registers, 8 warps) 43% and 30%. Whole products of 65536 Gaussian points in
-// the cube: one column 1.92 -> 0.91 ms, two 3.73 -> 1.75 ms; of 100003 points, one column,
-// 4.38 -> 2.06 ms. CTAs per SM 4 / 8 / 16, one column: 16384 points 215 / 204 / 216 us, 30011
+// the cube: one column 1.92 -> 0.91 ms, two 3.73 -> 1.73 ms; of 100003 points, one column,
+// 4.38 -> 2.05 ms. CTAs per SM 4 / 8 / 16, one column: 16384 points 215 / 204 / 216 us, 30011
 // 493 / 495 / 499, 65536 on the square 182 / 194 / 193.
 //
 // Relative error against the double-double product (mean of 8 normal vectors), float64 FMAs
-// / here: Gaussian cube of 20000 points 3.7e-16 / 2.4e-16, of 65536 5.0e-16 / 2.6e-16, Matern
-// 4.4e-16 / 2.8e-16, square 3.3e-16 / 2.8e-16, sphere 3.8e-16 / 3.0e-16, skeleton Gaussian
-// 2.4e-16 / 2.9e-16 (rows of few blocks, which more warps now add into by atomics). With parts
+// / here: Gaussian cube of 20000 points 3.7e-16 / 2.3e-16, of 65536 5.0e-16 / 2.3e-16, Matern
+// 4.4e-16 / 2.6e-16, square 3.3e-16 / 2.8e-16, sphere 3.8e-16 / 2.7e-16, skeleton Gaussian
+// 2.4e-16 / 2.8e-16 (rows of few blocks, which more warps now add into by atomics). With parts
 // of 28 bits a column A e_j of 2000 Gaussian points was off by 4.0e-17 of its largest entry;
 // now it is within 2^-55.7.
 constexpr int FX_WAVES = 8;

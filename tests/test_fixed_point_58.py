@@ -49,8 +49,9 @@ def test_sums_of_the_largest_values_fit():
     h, l = 2 ** B - 1, 2 ** B
     hh, mid = 16 * h * h, 16 * 2 * h * l + 2 ** (B - 1)                 # a row: 16 passes
     assert hh + (mid >> B) < 2 ** 63 and mid < 2 ** 63
-    hh, mid = 8 * h * h, 8 * 2 * h * l + 2 ** (B - 1) + 2 ** B          # a column: 8 rows, halved,
-    assert mid < 2 ** 63 and 8 * ((hh + (mid >> B)) >> 1) < 2 ** 63     # then 8 lanes
+    g, m = 2 ** (B - 1) - 1, 2 ** B                                     # the row's x: an exponent more
+    hh, mid = 8 * h * g, 8 * (h * m + l * g) + 2 ** (B - 1)             # a column: 8 rows,
+    assert mid < 2 ** 63 and 8 * (hh + (mid >> B)) < 2 ** 63            # then 8 lanes
 
 
 @pytest.mark.parametrize("spread", [0, 5, 60])
@@ -59,18 +60,18 @@ def test_column_of_64_terms(spread):
     for _ in range(50):
         a = [rng.gauss(0, 1) * 2.0 ** -rng.randint(0, spread) for _ in range(64)]
         b = [rng.gauss(0, 1) * 2.0 ** -rng.randint(0, spread) for _ in range(64)]
-        Ea, Eb = max(map(exponent, a)), max(map(exponent, b))
+        Ea, Eb = max(map(exponent, a)), max(map(exponent, b)) + 1
         total = 0
         for lane in range(8):
-            hh, mid = 0, 2 ** (B - 1) + 2 ** B
+            hh, mid = 0, 2 ** (B - 1)
             for x, y in zip(a[8 * lane:8 * lane + 8], b[8 * lane:8 * lane + 8]):
                 (h, l), (g, m) = encode(x, Ea), encode(y, Eb)
                 hh += h * g
                 mid += h * m + l * g
-            total += (hh + (mid >> B)) >> 1
-        got = Fraction(total) * Fraction(2) ** (Ea + Eb - 2101)
+            total += hh + (mid >> B)
+        got = Fraction(total) * Fraction(2) ** (Ea + Eb - 2102)
         exact = sum(Fraction(x) * Fraction(y) for x, y in zip(a, b))
         scale = Fraction(2) ** (Ea + Eb - 2044)
-        # per term: two encodings at 2^-59 and the part left out at 2^-58; per lane: one rounding
-        # to a unit of 2^-57
-        assert abs(got - exact) <= scale * (64 * Fraction(2, 2 ** 58) + 8 * Fraction(1, 2 ** 57))
+        # relative to the scales, b's doubled by its exponent: per term two encodings at 2^-59 and the
+        # part left out at 2^-58; per lane half a unit of 2^-58
+        assert abs(got - exact) <= scale * (64 * Fraction(2, 2 ** 58) + 8 * Fraction(1, 2 ** 59))
