@@ -581,7 +581,7 @@ __device__ void fx_tile_load_block(Fx* T, int* ex, const ChildRef& R, const Chil
       i = j;
       j = x;
     }
-    T[j * FXLD + i] = fx_encode(v[q], ex[i]);
+    T[j * FXLD + i] = fx_encode_even(v[q], ex[i]);
   }
 }
 

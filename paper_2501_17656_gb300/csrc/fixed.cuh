@@ -62,6 +62,17 @@ __device__ __forceinline__ Fx fx_encode(double v, int E) {
   return {(int)h * s, (int)l * s};
 }
 
+// The same value as h 2^B + l with |l| <= 2^(B - 1) (and |h| <= 2^B): the part l l' that a product
+// leaves out is then a quarter of that and has no lean either. With l of v's own sign it always
+// pulls sums of equal signs towards zero, by 2^-(2 B + 2) of the scales per term, which in the
+// update of a factor adds up over all of it.
+template <int B = 28>
+__device__ __forceinline__ Fx fx_encode_even(double v, int E) {
+  Fx f = fx_encode<B>(v, E);
+  const int c = (f.l + (1 << (B - 1))) >> B;     // -1, 0 or 1
+  return {f.h + c, f.l - (c << B)};
+}
+
 // acc += a * b (32 x 32 -> 64 bits)
 __device__ __forceinline__ void fx_mad(int64_t& acc, int a, int b) {
   asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));

@@ -62,7 +62,7 @@ __device__ __forceinline__ void fx_tile_load(Fx* T, int* ex, F load) {
   __syncthreads();
   const int E = ex[r];
 #pragma unroll
-  for (int q = 0; q < 16; ++q) T[(k0 + 4 * q) * FXLD + r] = fx_encode(v[q], E);
+  for (int q = 0; q < 16; ++q) T[(k0 + 4 * q) * FXLD + r] = fx_encode_even(v[q], E);
 }
 
 // The same with k along consecutive threads: thread t asks for k = t % 64 and rows t / 64 +
@@ -85,7 +85,7 @@ __device__ __forceinline__ void fx_tile_load_k(Fx* T, int* ex, F load, int margi
   }
   __syncthreads();
 #pragma unroll
-  for (int q = 0; q < 16; ++q) T[k * FXLD + r0 + 4 * q] = fx_encode(v[q], ex[r0 + 4 * q]);
+  for (int q = 0; q < 16; ++q) T[k * FXLD + r0 + 4 * q] = fx_encode_even(v[q], ex[r0 + 4 * q]);
 }
 
 // c += P Q^T.
@@ -133,7 +133,7 @@ __device__ __forceinline__ void fx_tile_store_q(Fx* T, int* ex, const double (&v
   for (int q = 0; q < 4; ++q) {
     const int b = fx_b() + 16 * q, E = ex[b];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) T[(fx_a() + r) * FXLD + b] = fx_encode(v[r][q], E);
+    for (int r = 0; r < 4; ++r) T[(fx_a() + r) * FXLD + b] = fx_encode_even(v[r][q], E);
   }
 }
 
