@@ -826,6 +826,7 @@ void build_coarse_near(Matrix& M) {
     M.poolP[i].bytes = pool_bytes(M.nP[i], KC, M.fmt);
     M.poolP[i].p = M.alloc(M.poolP[i].bytes);
     const double* Ef = M.d_E + (size_t)M.slot0(mf) * KC * KC;
+    // levels with clusters of widely different row scales stay in float64 (mark_spread)
     const bool fx = KC == FXT && !level_spread(M, mc) && !level_spread(M, mf);
     chunked(M.nP[i], [&](int64_t b0, int nb) {
       if (fx) {
