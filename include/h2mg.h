@@ -338,7 +338,8 @@ h2mg_status h2mg_apply_level(h2mg_matrix A, int level, int precision, const doub
                              double* y, void* stream);
 
 /* e = dir_sol(A_l, r) through A_l^{-1}, formed at build from the Cholesky factor of
- * the coarsest operator (Sec. 3.3, the dir_sol step of Algorithm 1). Vectors as for h2mg_apply_level at i = l. */
+ * the coarsest operator, and one step of refinement with A_l (Sec. 3.3, the dir_sol step of
+ * Algorithm 1). Vectors as for h2mg_apply_level at i = l. */
 h2mg_status h2mg_coarse_solve(h2mg_matrix A, const double* r, double* e, void* stream);
 
 /* One call of the smoother Iter(A_i, f, x0) = n iterations of CG (Sec. 3.3) on

@@ -152,10 +152,10 @@ __device__ __forceinline__ void wait_group(const int* done, int want, int* late)
 //
 // A step is the columns' work, 98 float64 operations per column of 32 rows (3700 clocks on
 // average for 128 columns on a pipe of 2 per clock and SM), and the next reflector's chain: a
-// sum, a square root and a division. Together they keep the float64 pipe 72 to 83% busy. A warp per column spent 8 operations for
-// every 2 of the columns' own, mostly on warp-wide sums and on the reflector in every warp:
-// 8192 points in 296 ms. One group of four lanes per column 171 ms; with the groups, one's
-// chain runs beside another's columns: 138 ms.
+// sum, a square root and a division. Together they keep the float64 pipe 72 to 83% busy. A
+// warp per column spent 8 operations for every 2 of the columns' own, mostly on warp-wide sums
+// and on the reflector in every warp: 8192 points in 296 ms. One group of four lanes per
+// column 171 ms; with the groups, one's chain runs beside another's columns: 138 ms.
 template <int NC>
 __device__ __forceinline__ void fold_chunk(SkelSmem<NC>& sm, int nc, int64_t ch, int group, int k, int q,
                                            double (&c)[Skel<NC>::OWN]) {
